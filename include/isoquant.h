@@ -22,9 +22,9 @@
  *     before anything is launched; on an error nothing has been enqueued.
  *   - Device-side conditions that cannot be known on the host are reported through an optional
  *     `status_dev` array of 4 uint32 (zeroed by the caller): [0] bit mask of IQ_STATUS_* flags,
- *     [1] rows whose codes were re-decided in fp64 (see iq_quantize_append), [2] rows skipped because
- *     they fell outside the cache, [3] reserved. Nothing on the device traps or spins without a bound: the
- *     decode kernel's waits on its asynchronous copies and tensor-core results give up after 65536 polls of at most
+ *     [1] rows with codes re-decided in fp64 (see iq_quantize_append; a row may count once per 32 coordinates), [2] rows skipped because
+ *     they fell outside the cache, [3] reserved. Nothing on the device traps or spins without a bound: the waits of the
+ *     decode and bulk append kernels on asynchronous copies and tensor-core results give up after 65536 polls of at most
  *     20 us each (about a second at worst; a wait that works lasts microseconds), flag IQ_STATUS_WAIT_TIMEOUT and
  *     the kernel returns with invalid results.
  *
@@ -93,7 +93,7 @@ enum {
 
 enum {
   IQ_STATUS_ROW_OUT_OF_RANGE = 1u, /* quantize-append: append_pos + i >= t_cap, row skipped */
-  IQ_STATUS_WAIT_TIMEOUT = 2u,     /* decode: a bounded wait on an asynchronous copy ran out; results invalid */
+  IQ_STATUS_WAIT_TIMEOUT = 2u,     /* decode, bulk append: a bounded wait on an asynchronous copy or tensor-core result ran out; results invalid */
   IQ_STATUS_SCALE_OVERFLOW = 8u,   /* binary16 scales: a row norm above 65504 was stored as 65504 */
   IQ_STATUS_BAD_PAGE = 4u          /* paged cache: a block-table entry outside [0, num_pages) was met: read as page 0 by
                                       decode / reconstruct, the rows skipped (and counted in [2]) by quantize-append */
@@ -195,7 +195,8 @@ int iq_make_rotation(int32_t head_dim, int32_t n_kv_heads, uint64_t seed, const 
  *                  sequence-length array: the caller advances its lengths. Calls that append to the same
  *                  (sequence, KV head) must be ordered on one stream.
  *   status_dev     optional (see top). Rows with append_pos + i outside [0, t_cap) are skipped and flagged.
- * Arithmetic: fp32 butterfly WHT and 4x4 block products; any row with a coordinate closer than 2^-15 to a
+ * Arithmetic: fp32 sums (calls of up to 4 rows per sequence: butterfly WHT and 4x4 block products; larger ones: one
+ * tensor-core contraction with the rotation as two binary16 terms); a coordinate closer than 2^-15 (2^-16) to a
  * decision threshold is re-decided in fp64 inside the kernel, so the codes equal those of an fp64
  * evaluation except for ties at the fp64 rounding level. The stored scale is sqrt(sum x^2) accumulated
  * in fp64 and rounded to fp32. A zero row stores scale 0 and the code of u = 0 everywhere.

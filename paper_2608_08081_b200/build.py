@@ -8,7 +8,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libisoquant.so")
-SOURCES = ["iq_api.cu", "iq_quantize.cu", "iq_decode.cu", "iq_decode_b2.cu", "iq_decode_b3.cu", "iq_decode_b4.cu", "iq_combine.cu",
+SOURCES = ["iq_api.cu", "iq_quantize.cu", "iq_append_bulk.cu", "iq_decode.cu", "iq_decode_b2.cu", "iq_decode_b3.cu", "iq_decode_b4.cu", "iq_combine.cu",
            "iq_static.cu", "iq_reconstruct.cu"]
 HEADERS = ["iq_common.cuh", "iq_decode_common.cuh", "iq_decode_kernel.cuh", "iq_quantize_common.cuh", "iq_append_row.cuh", "iq_format.cuh",
            "iq_kernels.h", os.path.join("..", "..", "include", "isoquant.h")]

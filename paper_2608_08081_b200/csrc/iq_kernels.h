@@ -16,7 +16,6 @@ struct PageMap {
 // ---- quantize-append
 constexpr int QA_WARPS = 4;
 constexpr int QA_FEW_ROWS = 4;        // calls with at most this many new rows per sequence take the one-warp-per-row latency path
-constexpr int QA_ROWS_PER_WARP = 16;  // K rows per warp and launch (a warp holds 4 rows at a time at head_dim 128)
 
 struct QuantizeParams {
   const __half* k_new;
@@ -39,6 +38,8 @@ struct QuantizeParams {
   int scale_f16;
 };
 cudaError_t launch_quantize_append(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream);
+bool append_bulk_takes(const QuantizeParams& p, int head_dim);
+cudaError_t launch_append_bulk(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream);
 
 // ---- calibration: histogram of the rotated, normalised coordinates of a set of rows
 constexpr int HIST_MAX_BINS = 4096;

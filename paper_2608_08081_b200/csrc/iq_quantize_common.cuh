@@ -25,17 +25,4 @@ __device__ __forceinline__ int decide_code(T u, const float (&th)[7], bool& near
   return (b2 ? 4 : 0) + (b1 ? 2 : 0) + (b0 ? 1 : 0);
 }
 
-// The same decision for a codebook that is symmetric about zero (t_3 = 0, t_{6-k} = -t_k; the Lloyd-Max codebooks of a
-// symmetric density are): two compares on |u| and the sign. Exact ties fall inside the guard band and are re-decided.
-// dmin carries the smallest distance to a threshold seen so far, so that one test serves all coordinates of a lane.
-__device__ __forceinline__ int decide_code_sym(float u, float a1, float a2, float a3, float& dmin) {
-  const float a = fabsf(u);
-  const bool b1 = a > a2;
-  const float p0 = b1 ? a3 : a1;
-  const bool b0 = a > p0;
-  dmin = fminf(fminf(dmin, a), fminf(fabsf(a - a2), fabsf(a - p0)));
-  const int mag = (b1 ? 2 : 0) + (b0 ? 1 : 0);
-  return u > 0.f ? 4 + mag : 3 - mag;
-}
-
 }  // namespace iq

@@ -1,0 +1,104 @@
+"""The bulk append kernel (Algorithm 1 on the tensor cores) against the warp-per-row kernel that calls of up to four rows
+take, byte for byte, and against the oracle: tile edges (first and last rows inside 128-row blocks), every bit width, both
+forms of the decision (thresholds symmetric about zero or not), two codebooks, strided inputs, paged caches, binary16
+scales, rows whose coordinates all sit on a threshold, zero rows, rows that end a sequence outside the cache."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from helpers import cache_to_numpy
+from test_gpu_bits import compare_codes, iq, torch, two_codebooks  # noqa: F401 (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+def _append(iq, torch, shape, rot, cb, k, v, first, lens, rows, page_rows, scales):
+    """The rows of k, v appended `rows` at a time into a cache whose bytes are not zero to begin with."""
+    B, T = k.shape[:2]
+    if page_rows:
+        n = B * (shape.t_cap // page_rows)
+        table = torch.arange(n - 1, -1, -1, dtype=torch.int32, device="cuda").reshape(B, -1).contiguous()
+        cache = iq.new_paged_cache(shape, n, page_rows, table, scales_dtype=scales)
+    else:
+        cache = iq.new_cache(shape, scales_dtype=scales)
+    for a in (cache.k_codes, cache.v_codes):
+        a.fill_(0x5A)
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    for i in range(0, T, rows):
+        n = [int(min(max(x - i, 0), rows)) for x in lens]
+        iq.iq_quantize_append(shape, rot, cb, k[:, i:i + rows], v[:, i:i + rows], torch.tensor([f + i for f in first], dtype=torch.int32, device="cuda"),
+                              torch.tensor(n, dtype=torch.int32, device="cuda"), min(rows, T - i), cache, status)
+    torch.cuda.synchronize()
+    return cache, status.cpu().numpy()
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("variant", ["symmetric", "shifted", "two codebooks, paged, binary16 scales"])
+def test_bulk_append_equals_the_row_kernel(iq, torch, bits, d, variant):  # noqa: F811
+    B, H, T, t_cap = 5, 3, 300, 512
+    first, lens = [0, 3, 127, 128, 400], [300, 125, 129, 5, 200]   # sequence 4 runs past t_cap
+    lv, th, lvv, thv = two_codebooks(d, bits, "int8", variant.startswith("two"))
+    if variant == "shifted":
+        th = (th.astype(np.float64) + 0.01 * ((np.arange(len(th)) * 7) % 5 - 2)).astype(np.float32)
+        thv = th
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)), tuple(map(float, lvv)), tuple(map(float, thv)))
+    shape = iq.Shape(B, H, H, d, t_cap, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 11 + bits, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits)
+    kv = torch.randn((B, T, H, 2 * d), generator=gen, device="cuda").half()
+    kv[..., ::37] *= 20
+    kv[:, 2::11] = 0                    # zero rows
+    kv[:, 5::13] = 1                    # all but four coordinates exactly on a threshold at zero: more than a warp's list takes
+    kv[:, 7::17, :, 1:] = 0             # one element
+    kv[:, 9::19] *= 1e-4                # subnormal elements
+    k, v = kv[..., :d], kv[..., d:]     # strided
+    page_rows, scales = (128, torch.float16) if variant.startswith("two") else (0, torch.float32)
+    bulk, st = _append(iq, torch, shape, rot, cb, k, v, first, lens, T, page_rows, scales)
+    rows, st_rows = _append(iq, torch, shape, rot, cb, k, v, first, lens, 4, page_rows, scales)
+    for name in ("k_codes", "v_codes", "k_scales", "v_scales"):
+        a, b = getattr(bulk, name), getattr(rows, name)
+        assert torch.equal(a, b), f"{name}: {int((a != b).sum())} of {a.numel()} differ"
+    assert st[0] == st_rows[0] == 1 and st[2] == st_rows[2] == 88 * H * 2
+
+
+@pytest.mark.parametrize("n", [5, 64, 127, 128, 129, 257])
+@pytest.mark.parametrize("d,bits", [(128, 3), (256, 4)])
+def test_bulk_append_codes_match_the_oracle(iq, torch, d, bits, n):  # noqa: F811
+    w = workloads.tiny(840 + n, 1, 2, 2, d, n, lens=[n])
+    lv, th, _, _ = two_codebooks(d, bits, "int8", False)
+    shape = iq.Shape(1, 2, 2, d, w.t_cap, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, 2), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, 2, 0, np.ascontiguousarray(w.quats), rot)
+    cache, status = iq.new_cache(shape), torch.zeros(4, dtype=torch.int32, device="cuda")
+    iq.iq_quantize_append(shape, rot, iq.Codebook(tuple(map(float, lv)), tuple(map(float, th))), torch.from_numpy(w.k).cuda(),
+                          torch.from_numpy(w.v).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda"), None, n, cache, status)
+    torch.cuda.synchronize()
+    ref = oracle.new_cache(1, 2, d, w.t_cap, bits)
+    oracle.quantize_append(w.quats, th, w.k, w.v, np.zeros(1, np.int32), np.array([n], np.int32), ref, thresholds_v=th)
+    assert status[0] == 0 and status[2] == 0
+    compare_codes(w, bits, th, th, cache_to_numpy(cache), ref, [n])
+
+
+def test_codebook_with_close_thresholds_keeps_its_path(iq, torch):  # noqa: F811
+    """Thresholds 1e-5 apart cannot be told apart by the bulk kernel's decision: such a call takes the row kernel whatever
+    its size and gives what calls of four rows give."""
+    d, T = 128, 200
+    lv, th, _, _ = two_codebooks(d, 3, "int8", False)
+    th = th.copy()
+    th[4] = th[3] + np.float32(1e-5)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)))
+    shape = iq.Shape(1, 1, 1, d, 256)
+    rot = torch.empty(iq.iq_rotation_floats(d, 1), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, 1, 1, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    k, v = (torch.randn((1, T, 1, d), generator=gen, device="cuda").half() for _ in range(2))
+    a, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], T, 0, torch.float32)
+    b, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], 4, 0, torch.float32)
+    assert torch.equal(a.k_codes, b.k_codes) and torch.equal(a.v_codes, b.v_codes)
