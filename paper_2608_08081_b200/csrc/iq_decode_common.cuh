@@ -76,9 +76,11 @@ __device__ __forceinline__ uint64_t smem_desc_mn(uint32_t addr, uint32_t lbo, ui
 }
 // Instruction descriptor: D = f32, A = B = f16, A K-major (TMEM), B MN-major, N = 16, M = 128.
 constexpr uint32_t DEC_IDESC = (1u << 4) | (1u << 16) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
-// Integer path: D = s32, A = s8 (K-major, TMEM), B MN-major, N = 32, M = 128; B = s8 (query digits) or u8 (probability digits).
-constexpr uint32_t DEC_IDESC_I8_SS = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t DEC_IDESC_I8_SU = (2u << 4) | (1u << 7) | (0u << 10) | (1u << 16) | ((32u >> 3) << 17) | ((128u >> 4) << 24);
+// Integer path: D = s32, A = s8 (K-major, TMEM), B MN-major, N = 16 or 32, M = 128; B = s8 (query digits) or u8 (probability digits).
+template <int N>
+constexpr uint32_t DEC_IDESC_I8_SS = (2u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (((uint32_t)N >> 3) << 17) | ((128u >> 4) << 24);
+template <int N>
+constexpr uint32_t DEC_IDESC_I8_SU = (2u << 4) | (1u << 7) | (0u << 10) | (1u << 16) | (((uint32_t)N >> 3) << 17) | ((128u >> 4) << 24);
 
 // ---------------------------------------------------------------------------------------------- dequantisation
 // x >> s for a compile-time s, computed as the high word of x * 2^(32-s): the multiply issues on the integer

@@ -30,7 +30,8 @@
 //
 // Template parameters of the kernel: head_dim D; ARGMAX (exact slot maxima and their rows); I8 (levels on an 8-bit grid:
 // int8 operands, int32 accumulation; otherwise fp16 operands); APPEND (the launch also appends the step's new rows: a few
-// CTAs at the start of the grid do only that, see dec_aux_work); BITS (2, 3 or 4 bits per code: tile sizes and lookups).
+// CTAs at the start of the grid do only that, see dec_aux_work); BITS (2, 3 or 4 bits per code: tile sizes and lookups); HN
+// (query heads of an item that the columns are computed for: 4 when no item has more, otherwise 8).
 #pragma once
 #include <climits>
 
@@ -361,6 +362,15 @@ static __device__ __noinline__ void dec_aux_work(const DecodeParams& p, int lane
   }
 }
 
+// HN values per lane as the 8 that the warp reductions take.
+template <typename T, int HN>
+__device__ __forceinline__ void pad8(const T (&v)[HN], T fill, T (&out)[8]) {
+#pragma unroll
+  for (int h = 0; h < 8; h++) out[h] = h < HN ? v[h < HN ? h : 0] : fill;
+}
+__device__ __forceinline__ float max_of(const float (&v)[8]) { return max3f(max3f(v[0], v[1], v[2]), max3f(v[3], v[4], v[5]), fmaxf(v[6], v[7])); }
+__device__ __forceinline__ float max_of(const float (&v)[4]) { return fmaxf(max3f(v[0], v[1], v[2]), v[3]); }
+
 // Where the CTA's range starts (thread 0, set-up).
 struct DecStart {
   int b, y, len, piece;  // sequence, item within it, rows of the sequence, which piece of the item the range starts in
@@ -369,8 +379,9 @@ struct DecStart {
   int count, pad;       // blocks of the range
 };
 
-template <int D, bool ARGMAX, bool I8, bool APPEND, int BITS>
+template <int D, bool ARGMAX, bool I8, bool APPEND, int BITS, int HN>
 __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(const __grid_constant__ DecodeParams p) {
+  static_assert(HN == 4 || HN == DEC_HEADS, "heads per item");
   static_assert(!APPEND || BITS == 3, "the append inside the decode launch is built for the 3-bit layout");
   using L = DecLayout<D, BITS>;
   constexpr int DJ = L::DJ;
@@ -685,7 +696,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if constexpr (I8) {
 #pragma unroll
           for (int kk = 0; kk < D / 32; kk++)
-            tc_mma_i8(tmem_g + L::I8_S_COL, tmem_g + L::I8_K_COL + 8 * kk, bq_desc0 + 32 * kk, DEC_IDESC_I8_SS, kk > 0);
+            tc_mma_i8(tmem_g + L::I8_S_COL, tmem_g + L::I8_K_COL + 8 * kk, bq_desc0 + 32 * kk, DEC_IDESC_I8_SS<4 * HN>, kk > 0);
         } else {
 #pragma unroll
           for (int kk = 0; kk < D / 16; kk++)
@@ -706,7 +717,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           for (int j = 0; j < DJ; j++)
 #pragma unroll
             for (int kk = 0; kk < TB / 32; kk++)  // the values stay in TMEM (int32) over the blocks until the compute threads read them
-              tc_mma_i8(tmem_g + L::I8_O_COL + 32 * j, tmem_g + L::I8_V_COL + 32 * j + 8 * kk, bp_desc0 + 32 * kk, DEC_IDESC_I8_SU,
+              tc_mma_i8(tmem_g + L::I8_O_COL + 32 * j, tmem_g + L::I8_V_COL + 32 * j + 8 * kk, bp_desc0 + 32 * kk, DEC_IDESC_I8_SU<4 * HN>,
                         (kk > 0) || keep_values);
         } else {
 #pragma unroll
@@ -735,9 +746,9 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     const float inv_root_d = rsqrtf((float)D);
     const float kfac = p.sm_scale * LOG2E * inv_root_d;  // scores in log2 units: z2 = S_raw * scale_K * kfac
     const float vfac = inv_root_d;
-    float acc[DJ][8];  // thread c: coordinates c (+128), 8 heads
-    float m_run[8], l_run[8], best_v[8];
-    int best_i[8];
+    float acc[DJ][HN];  // thread c: coordinates c (+128), HN heads
+    float m_run[HN], l_run[HN], best_v[HN];
+    int best_i[HN];
     float sfac = 0.f;  // integer path: score digits -> log2-domain score per unit K scale (set when a segment is opened)
     int it = 0;        // staged slots of this group consumed so far (tile pipeline phases), the end marker included
     int nbk = 0;       // blocks this group has processed (phases of k_ready, s_bar, p_ready, o_bar)
@@ -768,11 +779,11 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     {
       const int n_pre = *n_pre_s;
       if (n_pre > 0) {
-        constexpr int NCW = NG * 4, JOBS = (8 * DEC_NPRE + NCW - 1) / NCW;
+        constexpr int NCW = NG * 4, JOBS = (HN * DEC_NPRE + NCW - 1) / NCW;
         float v[JOBS][E];
 #pragma unroll
         for (int t = 0; t < JOBS; t++) {
-          const int job = warp + t * NCW, sg = job >> 3, hh = job & 7;
+          const int job = warp + t * NCW, sg = job / HN, hh = job % HN;
           int kvh = 0, h0 = 0, nh = 0, b = 0;
           if (sg < n_pre) { b = pre_tab[sg].x; item_heads(pre_tab[sg].y, kvh, h0, nh); }
           rotate_head(b, kvh, h0 + hh, sg < n_pre && hh < nh, v[t]);
@@ -784,12 +795,12 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if (I8) cta_bar_sync_n(DEC_PRE_BAR, L::COMPUTE_THREADS);
 #pragma unroll
         for (int t = 0; t < JOBS; t++) {
-          const int job = warp + t * NCW, sg = job >> 3, hh = job & 7;
+          const int job = warp + t * NCW, sg = job / HN, hh = job % HN;
           if (sg < n_pre) {
             float qmax = 0.f;
             if (I8) {
 #pragma unroll
-              for (int h2 = 0; h2 < 8; h2++) qmax = fmaxf(qmax, pre_hmax[sg * 8 + h2]);
+              for (int h2 = 0; h2 < HN; h2++) qmax = fmaxf(qmax, pre_hmax[sg * 8 + h2]);
               if (hh == 0 && lane == 0) pre_sfac[sg] = score_factor(qmax);
             }
             write_operand(bq_pre + sg * L::BQ_BYTES, hh, v[t], qmax);
@@ -810,9 +821,9 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
       for (int j = 0; j < DJ; j++)
 #pragma unroll
-        for (int h = 0; h < 8; h++) acc[j][h] = 0.f;
+        for (int h = 0; h < HN; h++) acc[j][h] = 0.f;
 #pragma unroll
-      for (int h = 0; h < 8; h++) { m_run[h] = -INFINITY; l_run[h] = 0.f; best_v[h] = -INFINITY; best_i[h] = -1; }
+      for (int h = 0; h < HN; h++) { m_run[h] = -INFINITY; l_run[h] = 0.f; best_v[h] = -INFINITY; best_i[h] = -1; }
       if (bqbuf >= 0) {
         if (I8) sfac = pre_sfac[bqbuf];
         return;
@@ -820,19 +831,20 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       int kvh, h0, nh;
       item_heads(seg_y, kvh, h0, nh);
       const int wq = warp & 3;
-      float v[2][E];
+      constexpr int NT = HN / 4;  // heads per warp
+      float v[NT][E];
 #pragma unroll
-      for (int t = 0; t < 2; t++) rotate_head(seg_b, kvh, h0 + wq + 4 * t, wq + 4 * t < nh, v[t]);
+      for (int t = 0; t < NT; t++) rotate_head(seg_b, kvh, h0 + wq + 4 * t, wq + 4 * t < nh, v[t]);
       float qmax = 0.f;
       if constexpr (I8) {
-        qmax = fmaxf(abs_max(v[0]), abs_max(v[1]));
+        qmax = fmaxf(abs_max(v[0]), abs_max(v[NT - 1]));
         if (lane == 0) qtmp[wq] = qmax;
         group_bar_sync(bar_id);
         qmax = fmaxf(fmaxf(qtmp[0], qtmp[1]), fmaxf(qtmp[2], qtmp[3]));
         sfac = score_factor(qmax);
       }
 #pragma unroll
-      for (int t = 0; t < 2; t++) write_operand(bq, wq + 4 * t, v[t], qmax);
+      for (int t = 0; t < NT; t++) write_operand(bq, wq + 4 * t, v[t], qmax);
       fence_proxy_async();  // B_Q is written through the generic proxy and read by the tensor core through the async proxy
     };
 
@@ -848,16 +860,18 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         float* dst = p.part_acc + (((size_t)seg_b * p.n_q_heads + h0) * S + seg_slot) * D + gt;
         const size_t hstride = (size_t)S * D;
 #pragma unroll
-        for (int h = 0; h < 8; h++)
+        for (int h = 0; h < HN; h++)
           if (h < nh) {
 #pragma unroll
             for (int j = 0; j < DJ; j++) dst[h * hstride + 128 * j] = acc[j][h];
           }
         const int hr = warp_reduce8_head(lane);  // the head whose sum this lane ends up with
-        const float lsum = warp_reduce8(l_run, lane, [](float x, float y) { return x + y; });
+        float l8[8];
+        pad8(l_run, 0.f, l8);
+        const float lsum = warp_reduce8(l8, lane, [](float x, float y) { return x + y; });
         float msel = m_run[0];  // m_run[hr] (every thread of the group holds the same references)
 #pragma unroll
-        for (int h = 1; h < 8; h++) msel = (hr == h) ? m_run[h] : msel;
+        for (int h = 1; h < HN; h++) msel = (hr == h) ? m_run[h] : msel;
         if ((lane & 3) == 0) {
           red[(warp & 3) * 8 + hr] = lsum;
           if ((warp & 3) == 0) red2[hr] = msel;
@@ -872,19 +886,25 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       }
       {
         const int hr = warp_reduce8_head(lane);  // the head whose sums this lane ends up with
-        const float lsum = warp_reduce8(l_run, lane, [](float x, float y) { return x + y; });
+        float l8[8];
+        pad8(l_run, 0.f, l8);
+        const float lsum = warp_reduce8(l8, lane, [](float x, float y) { return x + y; });
         if ((lane & 3) == 0) red[(warp & 3) * 8 + hr] = lsum;
         if (ARGMAX) {
           float bv;
           int bi;
-          warp_argmax8(best_v, best_i, lane, bv, bi);
+          float v8[8];
+          int i8[8];
+          pad8(best_v, -INFINITY, v8);
+          pad8(best_i, -1, i8);
+          warp_argmax8(v8, i8, lane, bv, bi);
           if ((lane & 3) == 0) { red2[(warp & 3) * 8 + hr] = bv; redi[(warp & 3) * 8 + hr] = bi; }
         }
       }
       group_bar_sync(bar_id);
       float scale[8];  // the partial is reported relative to the exact maximum where that is tracked
 #pragma unroll
-      for (int h = 0; h < 8; h++) {
+      for (int h = 0; h < HN; h++) {
         float mt = m_run[h];  // every thread of the group holds the same reference
         int bi = -1;
         if (ARGMAX) {
@@ -903,7 +923,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
       }
 #pragma unroll
-      for (int h = 0; h < 8; h++)
+      for (int h = 0; h < HN; h++)
         if (h < nh) {
 #pragma unroll
           for (int j = 0; j < DJ; j++)
@@ -947,7 +967,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
         for (int j = 0; j < DJ; j++)
 #pragma unroll
-          for (int half = 0; half < 2; half++) {
+          for (int half = 0; half < HN / 4; half++) {
             uint32_t o_u[16];
             tc_ld16_issue(tmem_g + lane_sel + L::I8_O_COL + 32 * j + 16 * half, o_u);
             tc_wait_ld();
@@ -1023,7 +1043,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if (!failed) failed = !mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
         if (failed) break;
         tc_fence_after();
-        float s[8];
+        float s[HN];
         {
           auto digits_to_scores = [&](const uint32_t (&raw_u)[16], int half) {
 #pragma unroll
@@ -1032,39 +1052,46 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
               s[4 * half + hq] = fmaf(fmaf(__int2float_rn((int)raw_u[4 * hq + 2]), 16384.f, lo), kfs, mask);
             }
           };
-          uint32_t raw0[16], raw1[16];
+          uint32_t raw0[16];
           tc_ld16_issue(tmem_g + lane_sel + L::I8_S_COL, raw0);
           tc_wait_ld();
-          tc_ld16_issue(tmem_g + lane_sel + L::I8_S_COL + 16, raw1);  // heads 4..7 in flight while heads 0..3 are converted
-          digits_to_scores(raw0, 0);
-          tc_wait_ld();
-          digits_to_scores(raw1, 1);
+          if constexpr (HN == 8) {
+            uint32_t raw1[16];
+            tc_ld16_issue(tmem_g + lane_sel + L::I8_S_COL + 16, raw1);  // heads 4..7 in flight while heads 0..3 are converted
+            digits_to_scores(raw0, 0);
+            tc_wait_ld();
+            digits_to_scores(raw1, 1);
+          } else {
+            digits_to_scores(raw0, 0);
+          }
         }
         if (ARGMAX) {  // exact maximum seen by this thread and its row (a group sees the blocks of a segment in ascending order)
 #pragma unroll
-          for (int h = 0; h < 8; h++)
+          for (int h = 0; h < HN; h++)
             if (s[h] > best_v[h]) { best_v[h] = s[h]; best_i[h] = r0 + gt; }
         }
         // The running reference m_run is raised when a score exceeds it by more than DEC_MAX_SLACK_I8 log2 units, the
         // V-scale bound vref when a row exceeds it: both are rare after the first blocks (one barrier with an OR reduction
         // otherwise).
-        float over[8];
+        float over[HN];
 #pragma unroll
-        for (int h = 0; h < 8; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
-        const bool exceed = max3f(max3f(over[0], over[1], over[2]), max3f(over[3], over[4], over[5]), fmaxf(over[6], over[7])) > DEC_MAX_SLACK_I8 ||
+        for (int h = 0; h < HN; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
+        const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 ||
                             vf > vref || nacc >= 384;
         
         if (group_bar_or(bar_id, exceed)) {
           if (nacc > 0) flush();  // what TMEM holds is relative to the old references (the previous value MMAs have completed)
           {
-            const float wm = warp_reduce8(s, lane, [](float x, float y) { return fmaxf(x, y); });
+            float s8[8];
+            pad8(s, -INFINITY, s8);
+            const float wm = warp_reduce8(s8, lane, [](float x, float y) { return fmaxf(x, y); });
             if ((lane & 3) == 0) red[(warp & 3) * 8 + warp_reduce8_head(lane)] = wm;
           }
           const float wv_max = warp_max(vf);
           if (lane == 0) red2[warp & 3] = wv_max;
           group_bar_sync(bar_id);
 #pragma unroll
-          for (int h = 0; h < 8; h++) {
+          for (int h = 0; h < HN; h++) {
             const float bm = fmaxf(fmaxf(red[h], red[8 + h]), fmaxf(red[16 + h], red[24 + h]));
             const float mn = fmaxf(m_run[h], bm + DEC_RAISE_MARGIN);  // every head goes above its block maximum whichever head asked: fewer raises later
             const float alpha = ex2f(m_run[h] - mn);  // the accumulator holds the blocks before this one: rescale it now
@@ -1081,17 +1108,17 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         {
           // probabilities (times scale_V / sqrt(d)) as 30-bit fixed point: the bytes of round(p * vscale * pscale) are its four
           // base-256 digits. B_P[n][row], n = 4 head + digit.
-          uint32_t pb[8];
+          uint32_t pb[HN];
           const float vfp = vf * pscale;
 #pragma unroll
-          for (int h = 0; h < 8; h++) {
+          for (int h = 0; h < HN; h++) {
             const float pr = ex2f(over[h]);
             l_run[h] += pr;
             pb[h] = __float2uint_rn(pr * vfp);
           }
           const int off = (gt & 7) * 16 + (gt >> 3) * 128;
           *reinterpret_cast<uint4*>(bp + off) = make_uint4(pb[0], pb[1], pb[2], pb[3]);
-          *reinterpret_cast<uint4*>(bp + (TB / 8) * 128 + off) = make_uint4(pb[4], pb[5], pb[6], pb[7]);
+          if constexpr (HN == 8) *reinterpret_cast<uint4*>(bp + (TB / 8) * 128 + off) = make_uint4(pb[4], pb[5], pb[6], pb[7]);
           fence_proxy_async();
         }
         if (gt == 0) *accf = nacc;     // 0: this block's value product starts a new accumulation
@@ -1193,34 +1220,36 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 
         // ---- online softmax (log2 units); thread gt owns row r0 + gt, all 8 heads
         tc_wait_ld();
-        float s[8];
+        float s[HN];
         {
           const bool valid = gt < n;  // rows >= n of the last block hold stale bytes
           const float kf = valid ? ksc * kfac : 0.f;
           const float mask = valid ? 0.f : -INFINITY;  // stale rows: 0 * finite - inf = -inf
 #pragma unroll
-          for (int h = 0; h < 8; h++) s[h] = fmaf(__uint_as_float(raw_u[h]) + __uint_as_float(raw_u[8 + h]), kf, mask);
+          for (int h = 0; h < HN; h++) s[h] = fmaf(__uint_as_float(raw_u[h]) + __uint_as_float(raw_u[8 + h]), kf, mask);
         }
         if (ARGMAX) {  // exact maximum seen by this thread and its row (a group sees the blocks of a segment in ascending order)
 #pragma unroll
-          for (int h = 0; h < 8; h++)
+          for (int h = 0; h < HN; h++)
             if (s[h] > best_v[h]) { best_v[h] = s[h]; best_i[h] = r0 + gt; }
         }
         // The running reference m_run is raised only when some score of the block exceeds it by more than
         // DEC_MAX_SLACK (log2 units): exp2(s - m_run) then stays below 2^DEC_MAX_SLACK and nothing has to be
         // exchanged between the warps in the common case (one barrier with an OR reduction).
-        float over[8];
+        float over[HN];
 #pragma unroll
-        for (int h = 0; h < 8; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
-        const bool exceed = max3f(max3f(over[0], over[1], over[2]), max3f(over[3], over[4], over[5]), fmaxf(over[6], over[7])) > DEC_MAX_SLACK;
+        for (int h = 0; h < HN; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
+        const bool exceed = max_of(over) > DEC_MAX_SLACK;
         if (group_bar_or(bar_id, exceed)) {
           {
-            const float wm = warp_reduce8(s, lane, [](float x, float y) { return fmaxf(x, y); });
+            float s8[8];
+            pad8(s, -INFINITY, s8);
+            const float wm = warp_reduce8(s8, lane, [](float x, float y) { return fmaxf(x, y); });
             if ((lane & 3) == 0) red[(warp & 3) * 8 + warp_reduce8_head(lane)] = wm;
           }
           group_bar_sync(bar_id);
 #pragma unroll
-          for (int h = 0; h < 8; h++) {
+          for (int h = 0; h < HN; h++) {
             const float bm = fmaxf(fmaxf(red[h], red[8 + h]), fmaxf(red[16 + h], red[24 + h]));
             const float mn = fmaxf(m_run[h], bm + DEC_RAISE_MARGIN);  // every head goes above its block maximum whichever head asked: fewer raises later
             const float alpha = ex2f(m_run[h] - mn);  // the accumulator holds the blocks before this one: rescale it now
@@ -1235,17 +1264,17 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         for (int j = 0; j < DJ; j++) v_unit(j, 3);  // the last V unit, next to the exponentials
         {
           const float vf = (gt < n) ? vsc * vfac : 0.f;
-          float wv[8];
+          float wv[HN];
 #pragma unroll
-          for (int h = 0; h < 8; h++) {
+          for (int h = 0; h < HN; h++) {
             const float pr = ex2f(over[h]);
             l_run[h] += pr;
             wv[h] = pr * vf;
           }
           // probabilities (times scale_V / sqrt(d)) as fp16 hi + lo: B_P[n][row], n = head (hi) or 8 + head (lo)
-          uint32_t hp[4], lp[4];
+          uint32_t hp[4] = {0u, 0u, 0u, 0u}, lp[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-          for (int h2 = 0; h2 < 4; h2++) {
+          for (int h2 = 0; h2 < HN / 2; h2++) {
             const uint32_t hpk = pack_half2(wv[2 * h2], wv[2 * h2 + 1]);
             const float2 back = __half22float2(*reinterpret_cast<const __half2*>(&hpk));
             hp[h2] = hpk;
@@ -1282,7 +1311,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           float o[16];
           tc_ld16(tmem_g + lane_sel + L::O_COL + 16 * j, o);
 #pragma unroll
-          for (int h = 0; h < 8; h++) acc[j][h] += o[h] + o[8 + h];
+          for (int h = 0; h < HN; h++) acc[j][h] += o[h] + o[8 + h];
         }
         tc_fence_before();
         nbk++;
@@ -1309,7 +1338,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   if (warp == NG * 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
 }
 
-template <int D, bool ARGMAX, bool I8, bool APPEND, int BITS>
+template <int D, bool ARGMAX, bool I8, bool APPEND, int BITS, int HN>
 static cudaError_t launch_one(const DecodeParams& p, cudaStream_t stream) {
   using L = DecLayout<D, BITS>;
   static bool configured[64] = {};
@@ -1318,7 +1347,7 @@ static cudaError_t launch_one(const DecodeParams& p, cudaStream_t stream) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  auto kern = decode_kernel<D, ARGMAX, I8, APPEND, BITS>;
+  auto kern = decode_kernel<D, ARGMAX, I8, APPEND, BITS, HN>;
   if (!configured[dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM_BYTES);
     if (e != cudaSuccess) return e;
@@ -1347,15 +1376,19 @@ static cudaError_t launch_one(const DecodeParams& p, cudaStream_t stream) {
   return launch_after_predecessor(kern, dim3((unsigned)ctas), dim3(L::THREADS), L::SMEM_BYTES, stream, p);
 }
 
+template <int D, bool APPEND, int BITS, int HN>
+static cudaError_t launch_decode_heads(const DecodeParams& p, cudaStream_t stream) {
+  const bool am = p.part_argmax != nullptr;
+  if (p.use_i8)  // levels on an 8-bit grid: int8 operands, int32 accumulation
+    return am ? launch_one<D, true, true, APPEND, BITS, HN>(p, stream) : launch_one<D, false, true, APPEND, BITS, HN>(p, stream);
+  return am ? launch_one<D, true, false, APPEND, BITS, HN>(p, stream) : launch_one<D, false, false, APPEND, BITS, HN>(p, stream);
+}
 template <bool APPEND, int BITS>
 static cudaError_t launch_decode_variant(const DecodeParams& p, int head_dim, cudaStream_t stream) {
-  const bool am = p.part_argmax != nullptr;
-  if (p.use_i8) {  // levels on an 8-bit grid: int8 operands, int32 accumulation
-    if (head_dim == 128) return am ? launch_one<128, true, true, APPEND, BITS>(p, stream) : launch_one<128, false, true, APPEND, BITS>(p, stream);
-    return am ? launch_one<256, true, true, APPEND, BITS>(p, stream) : launch_one<256, false, true, APPEND, BITS>(p, stream);
-  }
-  if (head_dim == 128) return am ? launch_one<128, true, false, APPEND, BITS>(p, stream) : launch_one<128, false, false, APPEND, BITS>(p, stream);
-  return am ? launch_one<256, true, false, APPEND, BITS>(p, stream) : launch_one<256, false, false, APPEND, BITS>(p, stream);
+  // up to 4 query heads per KV head: the score and probability work of four columns fewer
+  if (p.group <= 4)
+    return head_dim == 128 ? launch_decode_heads<128, APPEND, BITS, 4>(p, stream) : launch_decode_heads<256, APPEND, BITS, 4>(p, stream);
+  return head_dim == 128 ? launch_decode_heads<128, APPEND, BITS, DEC_HEADS>(p, stream) : launch_decode_heads<256, APPEND, BITS, DEC_HEADS>(p, stream);
 }
 
 }  // namespace iq
