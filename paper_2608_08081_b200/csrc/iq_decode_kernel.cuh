@@ -471,6 +471,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   int count = 0;  // blocks of this CTA's range (read from shared memory after the set-up barrier)
   bool no_work = false;
   int n_work = n_cta;  // CTAs of the grid that have blocks (they share the slots of the sequences without cached rows)
+  bool aligned = false;  // ranges that end where items do (below)
   if (range_mode) {
     constexpr long long W = DEC_SEG_COST;
     int* cnt_s = scan_s + L::THREADS + L::THREADS / 32;  // [THREADS] non-empty sequences per slice of the batch
@@ -491,12 +492,13 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     }
     __syncthreads();
     long long c_total, n_cols;  // cost of the whole launch; blocks per item column (all sequences)
-    int nb_max = 0;
+    int nb_max = 0, n_seqs;     // blocks of the longest sequence, sequences with rows
     {
       int v = 0, c = 0;
       for (int i = lane; i < L::THREADS; i += 32) { v += scan_s[i]; c += cnt_s[i]; }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) { v += __shfl_xor_sync(FULL, v, o); c += __shfl_xor_sync(FULL, c, o); }
+      n_seqs = c;
       c_total = ((long long)v + W * c) * ips;
       n_cols = v;
       for (int i = 0; i < L::THREADS / 32; i++) nb_max = max(nb_max, scan_s[L::THREADS + i]);
@@ -505,9 +507,50 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     cper = max(cper, (long long)((nb_max + W - 1) / (S / NG - 1) + 1));  // an item then spans at most S / NG ranges
     cper = max(cper, W + 1);                                              // and no range between two ranges of blocks is empty
     const long long t_lo = (long long)cta * cper;
-    if (t_lo >= c_total) no_work = true;
-    n_work = (int)min((long long)n_cta, (c_total + cper - 1) / cper);  // 0: no sequence has a cached row
-    if (tid == 0 && !no_work) {
+    // Little work: every item is cut on its own into equal pieces, one CTA each, where the pieces of all items fit the grid
+    // and the longest is not longer than a share of the partition above (which cannot go below an entry's cost, or below
+    // what an item's slots allow wherever it begins). A piece has a block for every group. One sequence of 1 K rows with
+    // one KV head: two CTAs with 4 blocks each instead of one with 8.
+    const long long items = (long long)n_seqs * ips;
+    int bpp = 0, pieces = 0;  // blocks of the longest piece, pieces of the longest item
+    if (items > 0 && items <= n_cta) {
+      pieces = min(S / NG, (int)(n_cta / items));
+      bpp = max(NG, (nb_max + pieces - 1) / pieces);
+      pieces = (nb_max + bpp - 1) / bpp;
+      aligned = bpp <= cper;
+    }
+    if (aligned) {
+      n_work = (int)items * pieces;
+      if (cta >= n_work) no_work = true;
+      else if (tid == 0) {
+        const int item = cta / pieces, k = cta - item * pieces, j = item / ips;  // piece k of item y of the j-th sequence with rows
+        DecStart s0;
+        s0.y = item - j * ips;
+        int before = 0, i = 0;
+        while (before + cnt_s[i] <= j) before += cnt_s[i++];
+        int b = i * per_thread, nb = nb_of(b);
+        for (;; nb = nb_of(++b)) {
+          if (nb == 0) continue;
+          if (before == j) break;
+          before++;
+        }
+        const int np = (nb + bpp - 1) / bpp;
+        s0.b = b;
+        s0.len = len_of(b);
+        s0.piece = k;
+        s0.item_g = 0;
+        s0.g0 = k < np ? (long long)k * nb / np : 0;
+        s0.count = k < np ? (int)((long long)(k + 1) * nb / np - s0.g0) : 0;  // 0: a shorter item has fewer pieces
+        *start_s = s0;
+        *next_s = 0;
+        pre_tab[0] = make_int2(b, s0.y);
+        *n_pre_s = 1;
+      }
+    } else {
+      if (t_lo >= c_total) no_work = true;
+      n_work = (int)min((long long)n_cta, (c_total + cper - 1) / cper);  // 0: no sequence has a cached row
+    }
+    if (tid == 0 && !no_work && !aligned) {
       // the first block at or after cost position t: its sequence, item, block, and launch-wide block index
       auto locate = [&](long long t, int& b, int& nb, int& y, int& blk, long long& before_nb, long long& c_b) {
         before_nb = 0;  // blocks (per item column) of the sequences before b
