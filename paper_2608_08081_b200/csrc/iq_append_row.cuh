@@ -40,13 +40,12 @@ struct WarpRowQuantizer {
   static constexpr int NB = E / 4;  // SO(4) blocks per lane
   static constexpr int NT = (1 << BITS) - 1;
   const float* qbase;
-  float M[NB][4][4];
+  QuatPairs<E> qp;
   float th[NT];
 
   __device__ __forceinline__ void init(const float* rot_head, const float* thresholds, int lane) {
     qbase = rot_head + (size_t)lane * NB * 8;
-#pragma unroll
-    for (int j = 0; j < NB; j++) so4_matrix<float>(qbase + 8 * j, M[j]);
+    qp.load(rot_head, lane);
 #pragma unroll
     for (int i = 0; i < NT; i++) th[i] = thresholds[i];
   }
@@ -82,7 +81,7 @@ struct WarpRowQuantizer {
 #pragma unroll
     for (int e = 0; e < E; e++) v[e] = x[e];
     wht_warp<float, E>(v, lane);
-    so4_apply<float, E, false>(M, v);
+    qp.template apply<false>(v);
     bool any_near = false;
 #pragma unroll
     for (int e = 0; e < E; e++) {

@@ -32,12 +32,8 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
   const int s0 = WPH == 1 ? 0 : warp;
 
   // the rotation block of this lane first: its loads do not depend on the partials and overlap with theirs
-  float M[E / 4][4][4];
-  if (WPH == 1 || warp == 0) {
-    const float* qb = p.rot + ((size_t)kvh * (D / 4) + (size_t)lane * (E / 4)) * 8;
-#pragma unroll
-    for (int j = 0; j < E / 4; j++) so4_matrix<float>(qb + 8 * j, M[j]);
-  }
+  QuatPairs<E> qp;
+  if (WPH == 1 || warp == 0) qp.load(p.rot + (size_t)kvh * (D / 4) * 8, lane);
 
   float m = -INFINITY;
   int best = -1;
@@ -171,7 +167,7 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
   for (int e = 0; e < E; e++) v[e] *= inv;
 
   // o = H_d * blockdiag(M_b^T) * o~   (H_d symmetric, R^T = H_d^T R_SO4^T)
-  so4_apply<float, E, true>(M, v);
+  qp.template apply<true>(v);
   wht_warp<float, E>(v, lane);
   const float inv_root_d = rsqrtf((float)D);
 #pragma unroll

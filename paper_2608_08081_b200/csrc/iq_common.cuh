@@ -64,16 +64,45 @@ __device__ __forceinline__ void wht_warp(T (&v)[E], int lane) {
       }
     }
   }
+  // (a loop: the kernels that use it run it once or twice per warp, where fetching instructions costs more than a branch)
+#pragma unroll 1
+  for (int b = 1; b < 32; b <<= 1) {
+    const T sgn = (lane & b) ? T(-1) : T(1);  // the upper lane of a pair keeps (other - own)
 #pragma unroll
-  for (int b = 0; b < 5; b++) {
-    const bool upper = (lane >> b) & 1;
-#pragma unroll
-    for (int i = 0; i < E; i++) {
-      T o = shfl_xor_t<T>(v[i], 1 << b);
-      v[i] = upper ? (o - v[i]) : (v[i] + o);
-    }
+    for (int i = 0; i < E; i++) v[i] = sgn * v[i] + shfl_xor_t<T>(v[i], b);  // one fused multiply-add, exact product
   }
 }
+
+// The E/4 SO(4) blocks a lane owns as their quaternion pairs, applied by two Hamilton products per block, q_L v conj(q_R)
+// (or the inverse, conj(q_L) v q_R), and one factor 1 / (|q_L| |q_R|): half the instructions of building the 4x4 matrix
+// and multiplying by it, for the places that rotate one vector.
+template <int E>
+struct QuatPairs {
+  float4 l[E / 4], r[E / 4];
+  __device__ __forceinline__ void load(const float* rot_head, int lane) {
+    const float4* q = reinterpret_cast<const float4*>(rot_head) + (size_t)lane * (E / 2);
+#pragma unroll
+    for (int j = 0; j < E / 4; j++) { l[j] = q[2 * j]; r[j] = q[2 * j + 1]; }
+  }
+  template <bool INVERSE>
+  __device__ __forceinline__ void apply(float (&v)[E]) const {
+#pragma unroll
+    for (int j = 0; j < E / 4; j++) {
+      const float sl = INVERSE ? -1.f : 1.f, sr = INVERSE ? 1.f : -1.f;  // the conjugated side
+      const float a = l[j].x, b = sl * l[j].y, c = sl * l[j].z, d = sl * l[j].w;
+      const float e = r[j].x, f = sr * r[j].y, g = sr * r[j].z, h = sr * r[j].w;
+      const float n2l = a * a + b * b + c * c + d * d, n2r = e * e + f * f + g * g + h * h;
+      const float n = (1.f / sqrtf(n2l)) * (1.f / sqrtf(n2r));
+      const float x0 = v[4 * j], x1 = v[4 * j + 1], x2 = v[4 * j + 2], x3 = v[4 * j + 3];
+      const float t0 = a * x0 - b * x1 - c * x2 - d * x3, t1 = a * x1 + b * x0 + c * x3 - d * x2;
+      const float t2 = a * x2 - b * x3 + c * x0 + d * x1, t3 = a * x3 + b * x2 - c * x1 + d * x0;
+      v[4 * j] = (t0 * e - t1 * f - t2 * g - t3 * h) * n;
+      v[4 * j + 1] = (t0 * f + t1 * e + t2 * h - t3 * g) * n;
+      v[4 * j + 2] = (t0 * g - t1 * h + t2 * e + t3 * f) * n;
+      v[4 * j + 3] = (t0 * h + t1 * g - t2 * f + t3 * e) * n;
+    }
+  }
+};
 
 // y = M x (or M^T x) for the E/4 blocks a lane owns.
 template <typename T, int E, bool TRANSPOSE>

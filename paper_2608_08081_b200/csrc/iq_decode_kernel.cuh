@@ -232,15 +232,24 @@ static __device__ __noinline__ DecHeadCoords<D> dec_rotate_head(const __half* q_
     for (int e = 0; e < E; e++) r.v[e] = 0.f;
     return r;
   }
-  float M[E / 4][4][4];
-  const float* qb = rot_head + (size_t)lane * (E / 4) * 8;
+  QuatPairs<E> qp;
+  qp.load(rot_head, lane);
+  uint32_t raw[E / 2];
+  if constexpr (E == 4) {
+    const uint2 t = *reinterpret_cast<const uint2*>(q_head + lane * E);
+    raw[0] = t.x; raw[1] = t.y;
+  } else {
+    const uint4 t = *reinterpret_cast<const uint4*>(q_head + lane * E);
+    raw[0] = t.x; raw[1] = t.y; raw[E / 2 - 2] = t.z; raw[E / 2 - 1] = t.w;
+  }
 #pragma unroll
-  for (int j = 0; j < E / 4; j++) so4_matrix<float>(qb + 8 * j, M[j]);
-  const __half* src = q_head + lane * E;
-#pragma unroll
-  for (int e = 0; e < E; e++) r.v[e] = __half2float(src[e]);
+  for (int e = 0; e < E / 2; e++) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&raw[e]));
+    r.v[2 * e] = f.x;
+    r.v[2 * e + 1] = f.y;
+  }
   wht_warp<float, E>(r.v, lane);
-  so4_apply<float, E, false>(M, r.v);
+  qp.template apply<false>(r.v);
   const float inv_root_d = rsqrtf((float)D);
 #pragma unroll
   for (int e = 0; e < E; e++) r.v[e] *= inv_root_d;
