@@ -38,6 +38,7 @@
 #include "iq_append_row.cuh"
 #include "iq_decode_common.cuh"
 #include "iq_kernels.h"
+#include "iq_tile_mma.cuh"
 
 namespace iq {
 
@@ -55,7 +56,7 @@ struct BulkLayout {
   static constexpr int NG = 4 / NJ;               // packing groups: their accumulators fill the tensor memory
   static constexpr int PACK = GT * NG;            // 512 packing threads
   static constexpr int THREADS = PACK + 32 * NG;  // + a control warp per group
-  static constexpr int OPERAND = 128 * 128 * 2;   // a 128 x 128 binary16 operand: two slabs of [128][64], 128-byte swizzle
+  static constexpr int OPERAND = TILE_OPERAND;
   static constexpr int W_BYTES = NJ * 2 * OPERAND;
   static constexpr int LIST = 48;                 // undecided coordinates a warp collects ...
   static constexpr int LIST_FLUSH = 32;           // ... and decides in fp64 after a tile that left it with this many, or at the end
@@ -93,18 +94,6 @@ struct BulkWarp {       // a packing warp's list
 };
 static_assert(sizeof(BulkWarp) == 32, "list state");
 
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,"
-      "%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-        "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]),
-        "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr)
-      : "memory");
-  tc_wait_ld();
-}
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -112,22 +101,6 @@ __device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                : "memory");
   tc_wait_ld();
 }
-// D[tmem] (+)= A[smem] * B[smem], binary16 operands, fp32 accumulation.
-__device__ __forceinline__ void tc_mma_f16_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(0), "r"(0), "r"(0), "r"(0)
-      : "memory");
-}
-// K-major operand, 128-byte swizzle: rows of 128 bytes (64 binary16 contraction steps), 8 rows = 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc_k128(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-// fp32 result, binary16 operands, both K-major, N = 128, M = 128; bit 13 negates A.
-constexpr uint32_t BULK_IDESC = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr uint32_t BULK_IDESC_NEG = BULK_IDESC | (1u << 13);
-
 __device__ __forceinline__ double half_to_double(uint32_t bits) {
   double d;
   asm("cvt.f64.f16 %0, %1;" : "=d"(d) : "h"((uint16_t)bits));
@@ -243,18 +216,6 @@ static __device__ __noinline__ void bulk_redo_rows(const QuantizeParams& p, cons
   }
 }
 
-// The blocks M_b of one head in fp64, one thread each.
-template <int D>
-static __device__ __noinline__ void bulk_build_m(const float* rot_head, double* m_s, int tid) {
-  if (tid < D / 4) {
-    double M[4][4];
-    so4_matrix<double>(rot_head + (size_t)tid * 8, M);
-#pragma unroll
-    for (int r = 0; r < 4; r++)
-#pragma unroll
-      for (int c = 0; c < 4; c++) m_s[16 * tid + 4 * r + c] = M[r][c];
-  }
-}
 // W of one head into shared memory: thread = (row i, part of the row's quads). W[i][4l + e] = +-V4[e] with
 // V4[e] = sum_c M[i%4][c] (-1)^popc(c & e), the sign (-1)^popc(b & l) with b the 4-block of i inside its 128-row half.
 template <int D>
@@ -519,7 +480,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
 #pragma unroll
                 for (int k = 0; k < 8; k++) {  // 16 contraction steps each: 32 bytes inside a 128-byte row, 4 per slab
                   const uint64_t step = (uint64_t)((k >> 2) * (L::OPERAND / 2) + (k & 3) * 32) >> 4;
-                  tc_mma_f16_ss(tmem_base + grp * GT + 128 * j, a0 + step, b0 + step, (j & hf) ? BULK_IDESC_NEG : BULK_IDESC, (hf | hl | k) != 0);
+                  tc_mma_f16_ss(tmem_base + grp * GT + 128 * j, a0 + step, b0 + step, (j & hf) ? TILE_IDESC | TILE_IDESC_NEG_A : TILE_IDESC, (hf | hl | k) != 0);
                 }
               }
             tc_commit(full_bar);
@@ -588,7 +549,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
       BulkTile* t = describe();
       int kind = failed ? -1 : t->kind;
       if (kind >= 0) load_half(*t, 0);
-      bulk_build_m<D>(rot_head, m_s, tid);
+      tile_build_m<D>(rot_head, m_s, tid);
       cta_bar_sync_n(1, L::PACK);
       bulk_build_w<D>(m_s, smem, tid);
       fence_proxy_async();

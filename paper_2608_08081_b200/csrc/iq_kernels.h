@@ -154,6 +154,8 @@ struct ReconstructParams {
   float levels_k[16], levels_v[16];
 };
 cudaError_t launch_reconstruct_rows(const ReconstructParams& p, int head_dim, int batch, cudaStream_t stream);
+// The same on the tensor cores; false: the levels are not binary16 values times one factor per side.
+bool launch_reconstruct_tiles(const ReconstructParams& p, int head_dim, int batch, cudaStream_t stream, cudaError_t& e);
 
 // ---- rotation parameters
 cudaError_t launch_make_rotation(float* rot, int n_quats, uint64_t seed, cudaStream_t stream);

@@ -125,6 +125,9 @@ static cudaError_t launch_reconstruct_bits(const ReconstructParams& p, int head_
 }
 cudaError_t launch_reconstruct_rows(const ReconstructParams& p, int head_dim, int batch, cudaStream_t stream) {
   if (batch <= 0 || p.t_cap <= 0 || p.out_rows <= 0) return cudaSuccess;
+  // the library's codebooks (levels on an 8-bit grid, or exact binary16) go to the tensor cores; this kernel takes any levels
+  cudaError_t e = cudaSuccess;
+  if (launch_reconstruct_tiles(p, head_dim, batch, stream, e)) return e;
   dim3 grid((unsigned)((min(p.t_cap, p.out_rows) + 127) / 128), (unsigned)p.n_kv_heads, (unsigned)batch);
   if (p.bits == 2) return launch_reconstruct_bits<2>(p, head_dim, grid, stream);
   if (p.bits == 4) return launch_reconstruct_bits<4>(p, head_dim, grid, stream);

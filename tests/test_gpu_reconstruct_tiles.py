@@ -1,0 +1,46 @@
+"""Reconstruction on the tensor cores (levels that are binary16 values times one factor per side) and by the general kernel
+(any other levels) against the oracle's dense R^T: block edges, every bit width, a K and a V codebook of different forms,
+an output shorter than the longest sequence."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+from helpers import cache_to_numpy
+from test_gpu_bits import iq, torch, two_codebooks  # noqa: F401 (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("form", ["8-bit grid", "binary16 keys, 8-bit grid values", "other levels"])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("d", [128, 256])
+def test_reconstructed_rows_at_block_edges(iq, torch, d, bits, form):  # noqa: F811
+    lens, T_out, H = np.array([1, 127, 0, 128, 129, 300], np.int32), 290, 3
+    w = workloads.tiny(860 + bits, len(lens), H, H, d, 300, lens=lens)
+    lv, th, lvv, thv = two_codebooks(d, bits, "int8")
+    if form.startswith("binary16"):
+        lv, th = two_codebooks(d, bits, "fp16", False)[:2]
+    if form.startswith("other"):
+        lvv = (lvv.astype(np.float64) * 1.0001 + 1e-3).astype(np.float32)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)), tuple(map(float, lvv)), tuple(map(float, thv)))
+    shape = iq.Shape(len(lens), H, H, d, w.t_cap, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 0, np.ascontiguousarray(w.quats), rot)
+    cache = iq.new_cache(shape)
+    lens_dev = torch.from_numpy(lens).cuda()
+    iq.iq_quantize_append(shape, rot, cb, torch.from_numpy(w.k).cuda(), torch.from_numpy(w.v).cuda(),
+                          torch.zeros(len(lens), dtype=torch.int32, device="cuda"), lens_dev, 300, cache)
+    kv = torch.full((len(lens), T_out, H, 2 * d), 7.0, dtype=torch.float16, device="cuda")
+    iq.iq_reconstruct_rows(shape, rot, cb, cache, lens_dev, kv[..., :d], kv[..., d:])
+    torch.cuda.synchronize()
+    K, V = oracle.reconstruct_rows(w.quats, lv, cache_to_numpy(cache), lens, H, levels_v=lvv, d=d)
+    for got, ref in ((kv[..., :d].cpu().numpy().astype(np.float64), K), (kv[..., d:].cpu().numpy().astype(np.float64), V)):
+        for b in range(len(lens)):
+            n = min(int(lens[b]), T_out)
+            assert np.all(got[b, n:] == 7.0)
+            if n:
+                r = ref[b, :n]   # one rounding to binary16 and fp32 sums: the bound of the parity test of the general kernel
+                assert np.all(np.abs(got[b, :n] - r) <= 2.0 ** -11 * 1.001 * np.abs(r) + 1e-5 * np.abs(r).max(axis=-1, keepdims=True) + 2.0 ** -25)
