@@ -184,7 +184,7 @@ static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const dou
       ss += __shfl_xor_sync(FULL, ss, o);
     }
     const double* m = m_s + 4 * coord;
-    const double u = (m[0] * z[0] + m[1] * z[1] + m[2] * z[2] + m[3] * z[3]) * (1.0 / sqrt(ss));  // (rows of norm zero are not listed)
+    const double u = (m[0] * z[0] + m[1] * z[1] + m[2] * z[2] + m[3] * z[3]) * inv_sqrt(ss);  // (rows of norm zero are not listed)
     const float th = ((info >> 20) & 1u) ? p.thresholds_v[lower] : p.thresholds_k[lower];
     if (act && li == 0) patch_code<BITS>(dst_s[ee], entry, lower + (u > (double)th ? 1 : 0));
   }
@@ -546,10 +546,10 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         return t;
       };
 
+      tile_build_m<D>(rot_head, m_s, tid);  // (while the control warps find the first tiles)
       BulkTile* t = describe();
       int kind = failed ? -1 : t->kind;
       if (kind >= 0) load_half(*t, 0);
-      tile_build_m<D>(rot_head, m_s, tid);
       cta_bar_sync_n(1, L::PACK);
       bulk_build_w<D>(m_s, smem, tid);
       fence_proxy_async();

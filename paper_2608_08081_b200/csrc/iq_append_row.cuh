@@ -94,7 +94,7 @@ struct WarpRowQuantizer {
 #pragma unroll
       for (int e = 0; e < E; e++) vd[e] = (double)x[e];
       wht_warp<double, E>(vd, lane);
-      const double inv_sd = (ss > 0.0) ? 1.0 / sqrt(ss) : 0.0;
+      const double inv_sd = (ss > 0.0) ? inv_sqrt(ss) : 0.0;
 #pragma unroll
       for (int j = 0; j < NB; j++) {
         double Md[1][4][4];

@@ -17,12 +17,16 @@ constexpr unsigned FULL = 0xffffffffu;
 // of q_L and the right-multiplication matrix of conj(q_R) (Section 3.3, "SO(4) parameterization").
 // q8 = (q_L.wxyz, q_R.wxyz); both are rescaled to unit length in the working precision T.
 // ------------------------------------------------------------------------------------------------
+// 1 / sqrt(x); in fp64 by the library's reciprocal root (1 ulp), a fraction of a root and a division.
+__device__ __forceinline__ float inv_sqrt(float x) { return 1.f / sqrtf(x); }
+__device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
+
 template <typename T>
 __device__ __forceinline__ void so4_matrix(const float* q8, T (&M)[4][4]) {
   T a = q8[0], b = q8[1], c = q8[2], d = q8[3];
   T e = q8[4], f = q8[5], g = q8[6], h = q8[7];
-  T nl = T(1) / sqrt(a * a + b * b + c * c + d * d);
-  T nr = T(1) / sqrt(e * e + f * f + g * g + h * h);
+  T nl = inv_sqrt(a * a + b * b + c * c + d * d);
+  T nr = inv_sqrt(e * e + f * f + g * g + h * h);
   a *= nl; b *= nl; c *= nl; d *= nl;
   e *= nr; f *= nr; g *= nr; h *= nr;
   const T L[4][4] = {{a, -b, -c, -d}, {b, a, -d, c}, {c, d, a, -b}, {d, -c, b, a}};
@@ -92,7 +96,7 @@ struct QuatPairs {
       const float a = l[j].x, b = sl * l[j].y, c = sl * l[j].z, d = sl * l[j].w;
       const float e = r[j].x, f = sr * r[j].y, g = sr * r[j].z, h = sr * r[j].w;
       const float n2l = a * a + b * b + c * c + d * d, n2r = e * e + f * f + g * g + h * h;
-      const float n = (1.f / sqrtf(n2l)) * (1.f / sqrtf(n2r));
+      const float n = inv_sqrt(n2l) * inv_sqrt(n2r);
       const float x0 = v[4 * j], x1 = v[4 * j + 1], x2 = v[4 * j + 2], x3 = v[4 * j + 3];
       const float t0 = a * x0 - b * x1 - c * x2 - d * x3, t1 = a * x1 + b * x0 + c * x3 - d * x2;
       const float t2 = a * x2 - b * x3 + c * x0 + d * x1, t3 = a * x3 + b * x2 - c * x1 + d * x0;
