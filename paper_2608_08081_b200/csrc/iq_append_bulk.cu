@@ -31,8 +31,8 @@
 // the others, which is what bounds the kernel (about 11 instructions per coordinate).
 //
 // Measured (K and V rows of 8 KV heads, Gaussian with outlier channels), against one row in 8 or 16 lanes with butterflies
-// by shuffle and a kernel per tensor: 1.6 M rows, d = 128, 3 bits: 279 us instead of 491 (1.8 TB/s of rows in and codes
-// out); 262 k rows, d = 256, 4 bits: 171 instead of 457; 50 k rows in chunks of 500 per sequence: 29.6 instead of 54.5.
+// by shuffle and a kernel per tensor: 1.6 M rows, d = 128, 3 bits: 278 us instead of 491 (1.8 TB/s of rows in and codes
+// out); 262 k rows, d = 256, 4 bits: 169 instead of 457; 50 k rows in chunks of 500 per sequence: 28.2 instead of 54.5.
 #include <cmath>
 
 #include "iq_append_row.cuh"
