@@ -24,9 +24,10 @@
  *     `status_dev` array of 4 uint32 (zeroed by the caller): [0] bit mask of IQ_STATUS_* flags,
  *     [1] rows with codes re-decided in fp64 (see iq_quantize_append; a row may count once per 32 coordinates), [2] rows skipped because
  *     they fell outside the cache, [3] reserved. Nothing on the device traps or spins without a bound: the waits of the
- *     decode and bulk append kernels on asynchronous copies and tensor-core results give up after 65536 polls of at most
- *     20 us each (about a second at worst; a wait that works lasts microseconds), flag IQ_STATUS_WAIT_TIMEOUT and
- *     the kernel returns with invalid results.
+ *     decode, bulk append and reconstruction kernels on asynchronous copies and tensor-core results give up after 65536 polls
+ *     of at most 20 us each (about a second at worst; a wait that works lasts microseconds). Decode and append then flag
+ *     IQ_STATUS_WAIT_TIMEOUT and return with invalid results; iq_reconstruct_rows, which has no status array, writes NaN
+ *     to the rows concerned.
  *
  * Rotation (Eq. 2, Section 3.3 "SO(4) parameterization", Appendix B)
  *   R = R_SO4 o H_d. H_d is the normalised Walsh-Hadamard matrix in natural (Sylvester) order,
@@ -286,6 +287,13 @@ int iq_combine_splits_sharded(const iq_shape* shape, const float* rot_dev, int32
 int iq_reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
                         const iq_cache* cache, const int32_t* seq_lens_dev, void* k_out, void* v_out,
                         int32_t out_rows, int64_t stride_b, int64_t stride_t, int64_t stride_h, void* stream);
+/* Diagnostic: the same call with `polls` (0 .. 65536) as the limit of its waits for tensor-core results. 0: every wait
+ * gives up at once, the MMAs in flight are waited for before the kernel returns, and every row it owes is NaN. (Codebooks
+ * that do not take the tensor cores have no such wait.) */
+int iq_selftest_reconstruct_wait(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
+                                 const iq_cache* cache, const int32_t* seq_lens_dev, void* k_out, void* v_out,
+                                 int32_t out_rows, int64_t stride_b, int64_t stride_t, int64_t stride_h, uint32_t polls,
+                                 void* stream);
 
 /*
  * Calibration of the codebook on data (Section 3.2, Step 3: "Lloyd-Max for the post-rotation distribution"; the paper

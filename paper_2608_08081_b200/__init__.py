@@ -35,6 +35,7 @@ from .binding import (  # noqa: F401
     iq_fit_rotation,
     iq_format_version,
     iq_selftest_bounded_wait,
+    iq_selftest_reconstruct_wait,
     iq_version,
     iq_wht_coordinates,
     lib_path,

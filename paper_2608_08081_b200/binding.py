@@ -83,6 +83,7 @@ def _load():
     lib.iq_wht_coordinates.argtypes = [ctypes.POINTER(_IqShape), _vp, _i64, _i64, _i64, _vp, _i32, _vp, _vp]
     lib.iq_fit_rotation.argtypes = [_vp, _i32, _i64, _i32, ctypes.POINTER(_IqCodebook), _vp, _vp]
     lib.iq_selftest_bounded_wait.argtypes = [_vp, ctypes.c_uint32, _vp]
+    lib.iq_selftest_reconstruct_wait.argtypes = lib.iq_reconstruct_rows.argtypes[:-1] + [ctypes.c_uint32, _vp]
     lib.iq_decode_step_workspace_bytes.argtypes = [ctypes.POINTER(_IqShape), _i32]
     lib.iq_decode_step_workspace_bytes.restype = ctypes.c_size_t
     lib.iq_decode_step_fused.argtypes = [ctypes.POINTER(_IqShape), _vp, ctypes.POINTER(_IqCodebook), _vp, _vp, _vp,
@@ -429,6 +430,13 @@ def iq_fit_rotation(z_rows, head_dim: int, codebook: Codebook, quats):
     _check(_lib.iq_fit_rotation(z.ctypes.data, z.shape[0], z.shape[1], head_dim, ctypes.byref(cb), q.ctypes.data,
                                 ctypes.cast(dist, ctypes.c_void_p)), "iq_fit_rotation")
     return q, float(dist[0]), float(dist[1])
+
+
+def iq_selftest_reconstruct_wait(shape: Shape, rot_dev, codebook: Codebook, cache: Cache, seq_lens_dev, k_out, v_out, polls: int, stream=None) -> None:
+    cs, cb, cc = shape.c(), codebook.c(), cache.c()
+    _check(_lib.iq_selftest_reconstruct_wait(ctypes.byref(cs), _ptr(rot_dev), ctypes.byref(cb), ctypes.byref(cc), _ptr(seq_lens_dev),
+                                             _ptr(k_out), _ptr(v_out), k_out.shape[1], k_out.stride(0), k_out.stride(1), k_out.stride(2),
+                                             int(polls), _stream(stream)), "iq_selftest_reconstruct_wait")
 
 
 def iq_selftest_bounded_wait(status, polls: int, stream=None) -> None:

@@ -622,9 +622,9 @@ int iq_combine_splits(const iq_shape* shape, const float* rot_dev, int32_t num_s
                                    lse_out, argmax_out, stream);
 }
 
-int iq_reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const iq_cache* cache,
-                        const int32_t* seq_lens_dev, void* k_out, void* v_out, int32_t out_rows, int64_t stride_b,
-                        int64_t stride_t, int64_t stride_h, void* stream) {
+static int reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const iq_cache* cache,
+                            const int32_t* seq_lens_dev, void* k_out, void* v_out, int32_t out_rows, int64_t stride_b,
+                            int64_t stride_t, int64_t stride_h, uint32_t wait_polls, void* stream) {
   int rc = check_shape(shape);
   if (rc) return rc;
   if (!rot_dev || !seq_lens_dev || !k_out || !v_out) return IQ_ERR_NULL;
@@ -652,13 +652,27 @@ int iq_reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_co
   p.t_cap = shape->t_cap;
   p.pm = page_map(cache, shape);
   p.scale_f16 = cache->scales_fp16 ? 1 : 0;
-  p.status = nullptr;
+  p.wait_polls = wait_polls;
   p.out_rows = out_rows;
   p.bits = shape->bits;
   std::memcpy(p.levels_k, side_levels(codebook, 0), sizeof(p.levels_k));
   std::memcpy(p.levels_v, side_levels(codebook, 1), sizeof(p.levels_v));
   const cudaError_t e = iq::launch_reconstruct_rows(p, shape->head_dim, shape->batch, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? IQ_OK : IQ_ERR_CUDA;
+}
+
+int iq_reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const iq_cache* cache,
+                        const int32_t* seq_lens_dev, void* k_out, void* v_out, int32_t out_rows, int64_t stride_b,
+                        int64_t stride_t, int64_t stride_h, void* stream) {
+  return reconstruct_rows(shape, rot_dev, codebook, cache, seq_lens_dev, k_out, v_out, out_rows, stride_b, stride_t, stride_h,
+                          iq::DEC_WAIT_LIMIT, stream);
+}
+
+int iq_selftest_reconstruct_wait(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const iq_cache* cache,
+                                 const int32_t* seq_lens_dev, void* k_out, void* v_out, int32_t out_rows, int64_t stride_b,
+                                 int64_t stride_t, int64_t stride_h, uint32_t polls, void* stream) {
+  if (polls > iq::DEC_WAIT_LIMIT) return IQ_ERR_LIMIT;
+  return reconstruct_rows(shape, rot_dev, codebook, cache, seq_lens_dev, k_out, v_out, out_rows, stride_b, stride_t, stride_h, polls, stream);
 }
 
 int iq_decode_step_host(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const void* inputs_host,
@@ -793,7 +807,7 @@ int iq_fit_rotation(const float* z_host, int32_t n_rows, int64_t row_stride, int
 
 int iq_selftest_bounded_wait(uint32_t* status_dev, uint32_t polls, void* stream) {
   if (!status_dev) return IQ_ERR_NULL;
-  if (polls > 65536u) return IQ_ERR_LIMIT;
+  if (polls > iq::DEC_WAIT_LIMIT) return IQ_ERR_LIMIT;
   return iq::launch_bounded_wait_selftest(status_dev, polls, static_cast<cudaStream_t>(stream)) == cudaSuccess ? IQ_OK : IQ_ERR_CUDA;
 }
 

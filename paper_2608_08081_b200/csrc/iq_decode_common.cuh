@@ -5,12 +5,6 @@
 
 namespace iq {
 
-// Polls one mbarrier wait of the decode kernel may take before the kernel gives up (IQ_STATUS_WAIT_TIMEOUT): with the
-// 20 us suspend hint of a poll that is at most 65536 * 20 us = 1.3 s (and a few milliseconds at least). Waits that
-// work last microseconds. A thread that has given up skips every later wait, so a CTA returns within about that time
-// after its first failed wait.
-constexpr uint32_t DEC_WAIT_LIMIT = 1u << 16;
-
 // ---------------------------------------------------------------------------------------------- tcgen05 wrappers
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -209,6 +203,13 @@ __device__ __forceinline__ bool group_bar_or(int id, bool pred) {
 }
 // Barrier 0 over the whole CTA, for the places where the control and the compute warps arrive from different code.
 __device__ __forceinline__ void cta_bar_sync() { asm volatile("barrier.sync 0;" ::: "memory"); }
+// The same over `count` threads.
+__device__ __forceinline__ bool cta_bar_or_n(int id, int count, bool pred) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %3, 0;\n\tbarrier.red.or.pred p, %1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(r) : "r"(id), "r"(count), "r"((uint32_t)pred) : "memory");
+  return r != 0;
+}
 // Named barrier `id` over `count` threads (a multiple of 32).
 __device__ __forceinline__ void cta_bar_sync_n(int id, int count) { asm volatile("barrier.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
 __device__ __forceinline__ void group_bar_sync(int id) { asm volatile("barrier.sync %0, 128;" ::"r"(id) : "memory"); }

@@ -6,6 +6,12 @@
 
 namespace iq {
 
+// Polls one mbarrier wait of a kernel may take before it gives up (IQ_STATUS_WAIT_TIMEOUT; the reconstruction: rows of NaN):
+// with the 20 us suspend hint of a poll that is at most 65536 * 20 us = 1.3 s (and a few milliseconds at least). Waits that
+// work last microseconds. A thread that has given up skips every later wait, so a CTA returns within about that time
+// after its first failed wait.
+constexpr uint32_t DEC_WAIT_LIMIT = 1u << 16;
+
 // Addressing of the cache arrays: contiguous per sequence (table == nullptr) or a pool of pages with a block table
 // (see cache_row in iq_common.cuh).
 struct PageMap {
@@ -149,9 +155,9 @@ struct ReconstructParams {
   int n_kv_heads, t_cap, out_rows;
   PageMap pm;
   int scale_f16;
-  uint32_t* status;
   int bits;
   float levels_k[16], levels_v[16];
+  uint32_t wait_polls;  // limit of the waits for tensor-core results: DEC_WAIT_LIMIT, or what the self-test asks for
 };
 cudaError_t launch_reconstruct_rows(const ReconstructParams& p, int head_dim, int batch, cudaStream_t stream);
 // The same on the tensor cores; false: the levels are not binary16 values times one factor per side.

@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(RC_WARPS * 32) reconstruct_kernel(const Recons
   const int r_begin = blockIdx.x * TB;
   if (r_begin >= len) return;
   const int n = min(TB, len - r_begin);
-  const size_t row0 = cache_row(p.pm, b, g, r_begin, p.status);  // the block's first row in the cache arrays
+  const size_t row0 = cache_row(p.pm, b, g, r_begin, nullptr);  // the block's first row in the cache arrays
 
   {  // stage the block: n packed K rows, the whole V record set of the block (128 * ROWB = D * 16 b bytes), the scales
     const uint4* ksrc = reinterpret_cast<const uint4*>(p.k_codes + row0 * ROWB);

@@ -27,6 +27,8 @@ struct ReconstructTileParams {
   float factor[2];              // level = binary16 value * factor
 };
 
+constexpr uint32_t HALF2_NAN = 0x7FFF7FFFu;
+
 template <int D>
 struct ReconLayout {
   static constexpr int NJ = D / 128, GT = 128 * NJ, NG = 4 / NJ, THREADS = GT * NG;
@@ -35,8 +37,8 @@ struct ReconLayout {
   static constexpr int OFF_T = OFF_M + D * 32;                       // [lo, hi][NJ][4][128] binary16: the magnitudes of W
   static constexpr int OFF_PRE = OFF_T + 2 * D * 8;                  // [THREADS + 1] int64 block counts before a slice of the batch
   static constexpr int OFF_WSUM = OFF_PRE + 8 * (THREADS + 2);
-  static constexpr int OFF_BAR = OFF_WSUM + 8 * 16;                  // [NG] mbarriers: MMAs done
-  static constexpr int OFF_MISC = OFF_BAR + 8 * NG;
+  static constexpr int OFF_BAR = OFF_WSUM + 8 * 16;                  // [NG][2] mbarriers: MMAs done; all MMAs of a group that gave up
+  static constexpr int OFF_MISC = OFF_BAR + 16 * NG;
   static constexpr int SMEM = OFF_MISC + 16 + 1024;
 };
 static_assert(ReconLayout<128>::SMEM <= 227 * 1024 && ReconLayout<256>::SMEM <= 227 * 1024, "shared memory overflow");
@@ -58,7 +60,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
   __half* t_s = reinterpret_cast<__half*>(smem + L::OFF_T);
   long long* pre_s = reinterpret_cast<long long*>(smem + L::OFF_PRE);
   long long* wsum_s = reinterpret_cast<long long*>(smem + L::OFF_WSUM);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR) + grp;
+  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR) + 2 * grp;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
 
   if (warp == 0) {
@@ -67,6 +69,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
   }
   if (gt == 0) {
     mbar_init(bar, 1);
+    mbar_init(bar + 1, 1);
     fence_mbar_init();
   }
   grid_dependency_wait();
@@ -97,7 +100,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
   const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
   const uint32_t tmem_g = tmem_base + (uint32_t)(grp * GT);
   const uint32_t tmem_t = tmem_g + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * 128);
-  bool failed = false;
+  bool failed = false;  // a bounded wait gave up (the whole group knows from its next barrier on): the rows it still owes become NaN
   uint32_t phase = 0;
 
   long long item = lo;
@@ -172,6 +175,15 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
 
     while (have) {
       const int is_v = w_v, b = w_b, row_base = blk * 128, n_rows = min(128, w_len - row_base);
+      __half* const out = (is_v ? p.v_out : p.k_out) + (size_t)b * p.stride_b + (size_t)row_base * p.stride_t + (size_t)h * p.stride_h;
+      if (failed) {  // no more MMAs
+        for (int i = gt; i < n_rows * (D / 8); i += GT)
+          *reinterpret_cast<uint4*>(out + (long long)(i / (D / 8)) * p.stride_t + 8 * (i % (D / 8))) = make_uint4(HALF2_NAN, HALF2_NAN, HALF2_NAN, HALF2_NAN);
+        it += NG;
+        have = it < seg_hi;
+        if (have) fetch();
+        continue;
+      }
       const float f = scale * q.factor[is_v] * (1.0f / (float)D);  // 1/sqrt(d) of the dequantisation times 1/sqrt(d) of H_d
       uint32_t l_lo[4], l_hi[4];
 #pragma unroll
@@ -216,13 +228,12 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
           have = it < seg_hi;
           if (have) fetch();
         }
-        if (!failed) failed = !mbar_wait_bounded(bar, phase, DEC_WAIT_LIMIT);
+        if (!failed) failed = !mbar_wait_bounded(bar, phase, p.wait_polls);
         phase ^= 1u;
       }
       tc_fence_after();
 
       // ---- this thread's 128 columns of row r: scale, round, through the operand's buffer (256 bytes per row and round)
-      __half* const out = (is_v ? p.v_out : p.k_out) + (size_t)b * p.stride_b + (size_t)row_base * p.stride_t + (size_t)h * p.stride_h;
 #pragma unroll
       for (int rd = 0; rd < NJ; rd++) {
         if (rd > 0) cta_bar_sync_n(bar_id, GT);  // the round before has left the buffer
@@ -239,13 +250,14 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
             *reinterpret_cast<uint4*>(xs + r * 256 + ((c ^ (r & 7)) * 16)) = make_uint4(o[0], o[1], o[2], o[3]);
           }
         }
-        cta_bar_sync_n(bar_id, GT);
+        failed = cta_bar_or_n(bar_id, GT, failed);
         const int c = gt & 15;  // piece of the row; its coordinate
         const int coord = (c / (16 / NJ)) * 128 + rd * (128 / NJ) + (c % (16 / NJ)) * 8;
 #pragma unroll
         for (int i = 0; i < 2048 / GT; i++) {
           const int row = (gt >> 4) + i * (GT / 16);
-          const uint4 v = *reinterpret_cast<const uint4*>(xs + row * 256 + ((c ^ (row & 7)) * 16));
+          uint4 v = *reinterpret_cast<const uint4*>(xs + row * 256 + ((c ^ (row & 7)) * 16));
+          if (failed) v = make_uint4(HALF2_NAN, HALF2_NAN, HALF2_NAN, HALF2_NAN);
           if (row < n_rows) *reinterpret_cast<uint4*>(out + (long long)row * p.stride_t + coord) = v;
         }
       }
@@ -256,6 +268,11 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
     __syncthreads();  // W^T is rebuilt for the next head
   }
   allow_dependent_launch();
+  if (failed && gt < 32) {  // MMAs may still be running: they are waited for, again with a limit, before the tensor memory goes
+    if (elect_one()) tc_commit(bar + 1);
+    __syncwarp();
+    mbar_wait_bounded(bar + 1, 0u, DEC_WAIT_LIMIT);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));

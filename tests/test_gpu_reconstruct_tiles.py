@@ -44,3 +44,33 @@ def test_reconstructed_rows_at_block_edges(iq, torch, d, bits, form):  # noqa: F
             if n:
                 r = ref[b, :n]   # one rounding to binary16 and fp32 sums: the bound of the parity test of the general kernel
                 assert np.all(np.abs(got[b, :n] - r) <= 2.0 ** -11 * 1.001 * np.abs(r) + 1e-5 * np.abs(r).max(axis=-1, keepdims=True) + 2.0 ** -25)
+
+
+@pytest.mark.parametrize("d", [128, 256])
+def test_a_wait_that_gives_up_leaves_no_ordinary_rows(iq, torch, d):  # noqa: F811
+    """A limit of 0 polls: every group gives up on its first tile and owes the rest of its share. The rows are NaN and not
+    the numbers of an unfinished product, rows past the lengths stay, the next call is an ordinary one."""
+    lens, H = [3000, 0, 129, 1500], 4
+    B, T = len(lens), max(lens)
+    shape = iq.Shape(B, H, H, d, 3072)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 5, None, rot)
+    cb, cache = iq.iq_lloyd_max_codebook(d, 3, "int8"), iq.new_cache(shape)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    lens_dev = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    iq.iq_quantize_append(shape, rot, cb, k, v, torch.zeros_like(lens_dev), lens_dev, T, cache)
+    outs = {}
+    for polls in (65536, 0, None):
+        ko, vo = (torch.full((B, T, H, d), 7.0, dtype=torch.float16, device="cuda") for _ in range(2))
+        if polls is None:
+            iq.iq_reconstruct_rows(shape, rot, cb, cache, lens_dev, ko, vo)
+        else:
+            iq.iq_selftest_reconstruct_wait(shape, rot, cb, cache, lens_dev, ko, vo, polls)
+        outs[polls] = (ko, vo)
+    torch.cuda.synchronize()
+    for side in range(2):
+        for b, n in enumerate(lens):
+            assert torch.isnan(outs[0][side][b, :n]).all() and (outs[0][side][b, n:] == 7.0).all()
+        assert torch.equal(outs[65536][side], outs[None][side]) and not torch.isnan(outs[None][side]).any()
