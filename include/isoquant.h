@@ -282,7 +282,10 @@ int iq_combine_splits_sharded(const iq_shape* shape, const float* rot_dev, int32
  *                  elements, multiples of 8; pointers 16-byte aligned), out_rows rows per sequence. Rows
  *                  t >= min(seq_lens[b], out_rows) are not written.
  *   codebook       only the levels are used (any fp32 values).
- * fp32 arithmetic, one rounding to binary16 at the end.
+ * fp32 arithmetic, one rounding to binary16 at the end. Levels on an 8-bit grid, or binary16 values that are integers of up
+ * to 15 bits in units of a power of two (the library's codebooks are one or the other), go through the tensor cores, with
+ * the rotation as two binary16 terms arranged so that the sums lose no more than fp32 butterflies do (an element is off by
+ * at most 2^-22 of itself plus 6e-7 of its row's rms before the rounding, as measured); any others do not.
  */
 int iq_reconstruct_rows(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
                         const iq_cache* cache, const int32_t* seq_lens_dev, void* k_out, void* v_out,

@@ -3,16 +3,27 @@
 //
 // Tile = (tensor, KV head, sequence, 128-row block). D[row][coordinate]: A = L, written into shared memory by the threads that
 // look the codes up -- K: thread = row, K-major; V: thread = coordinate of the token-transposed records, MN-major --
-// B = W^T in two binary16 terms (see iq_append_bulk.cu; W^T instead of W), fp32 accumulation, the small terms first. A
-// thread then holds a whole row (half a row at d = 256): scale, one rounding to binary16, through shared memory so that
-// rows leave in whole 256-byte pieces. d = 256: H_256 = [[H, H], [H, -H]], the halves of the contraction one after
-// the other through the same buffer, the operand of the last quarter negated by the instruction.
+// B = W^T in two binary16 terms. A thread then holds a whole row (half a row at d = 256): scale, one rounding to binary16,
+// through shared memory so that rows leave in whole pieces. d = 256: H_256 = [[H, H], [H, -H]], so the contraction is two of
+// 128 steps, one after the other through the same buffer, and the last stage of the butterfly, a sum and a difference in fp32.
+//
+// Precision. The instruction aligns its 16 products and the accumulator to the largest of them, keeps two bits below the fp32
+// last place, and cuts; the sum is cut to fp32 again (read off in-bounds sums of known terms). Sixteen such cuts of running
+// sums would cost more than the fp32 butterflies of iq_reconstruct.cu do. So the upper term of W is W rounded to a multiple of 2^-10
+// and the levels are integers of up to 7 bits and a sign times one factor: every partial sum of their products is a multiple
+// of 2^-10 below 128 * 128 (Cauchy-Schwarz: the columns of W have norm sqrt(128) per half), i.e. exact in fp32. The lower
+// term (|W - hi| <= 2^-11, rounded to binary16: off by at most 2^-23) goes first, where cuts are 2^-11 as large, and is then
+// cut once per doubling of the sum. Levels that are binary16 values of up to 15 bits are split in two such
+// integers, 256 h + m, and take three passes through the buffer: level x lower term, m x upper, h x upper. Error against
+// an fp64 evaluation before the rounding to binary16, relative to the row's rms: 0.9e-7 rms (two terms of 11 free bits each, all
+// products into one sum: 1.3e-7 to 1.9e-7 at d = 128, 3e-7 with binary16 levels, 4e-7 to 7e-7 at d = 256).
 //
 // One persistent CTA per SM, equal contiguous shares of the tiles ordered by head; groups of 128 threads (256 at d = 256)
 // take them in turn and request the next tile's codes while they work on the present one. About 20 warp instructions
 // per row for the lookups, 20 for the rest; its memory traffic would take 19 us where it takes 45: the groups' barriers and
-// the latency of each step bound it. Measured: 4 x 8 K rows, 8 KV heads, d = 128, 3 bits (407 k K and V rows): 45.0 us
-// instead of 101 with butterflies by shuffle and codes picked one by one (iq_reconstruct.cu, which takes any levels).
+// the latency of each step bound it. Measured: 4 x 8 K rows, 8 KV heads, d = 128, 3 bits (407 k K and V rows): 44.6 us
+// instead of 101 with butterflies by shuffle and codes picked one by one (iq_reconstruct.cu, which takes any levels). Three
+// passes, 4 sequences of up to 8 K rows at d = 128 (4 K at 256), 3 bits: 52 us (65) where one takes 39 (49) and that kernel 88 (134).
 #include <cmath>
 
 #include "iq_kernels.h"
@@ -23,8 +34,9 @@ namespace iq {
 struct ReconstructTileParams {
   ReconstructParams r;
   int batch;
-  uint32_t lo[2][4], hi[2][4];  // low / high bytes of the binary16 levels, K and V (4 per register)
-  float factor[2];              // level = binary16 value * factor
+  uint32_t lo[2][3][4], hi[2][3][4];  // K and V: low / high bytes of the binary16 operand values of each pass (4 per register)
+  int passes[2];                      // 1: the values with both terms of W; 3: with the lower, the upper, the upper term
+  float factor[2];                    // level = (sum of the passes that meet the upper term) * factor
 };
 
 constexpr uint32_t HALF2_NAN = 0x7FFF7FFFu;
@@ -43,7 +55,8 @@ struct ReconLayout {
 };
 static_assert(ReconLayout<128>::SMEM <= 227 * 1024 && ReconLayout<256>::SMEM <= 227 * 1024, "shared memory overflow");
 
-template <int D, int BITS>
+// SPLIT: some side takes three passes (an instance of its own: the loop over one pass costs 3 % at d = 128).
+template <int D, int BITS, bool SPLIT>
 __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_kernel(const __grid_constant__ ReconstructTileParams q) {
   using L = ReconLayout<D>;
   constexpr int NJ = L::NJ, NG = L::NG, GT = L::GT;
@@ -99,7 +112,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
   const long long nb = pre_s[L::THREADS], total = 2 * nb * p.n_kv_heads;  // tiles of a tensor of a head, all tiles
   const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
   const uint32_t tmem_g = tmem_base + (uint32_t)(grp * GT);
-  const uint32_t tmem_t = tmem_g + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * 128);
+  const uint32_t tmem_t = tmem_g + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(part * 64);
   bool failed = false;  // a bounded wait gave up (the whole group knows from its next barrier on): the rows it still owes become NaN
   uint32_t phase = 0;
 
@@ -155,7 +168,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
       const double v4[4] = {(m[0] + m[1]) + (m[2] + m[3]), (m[0] - m[1]) + (m[2] - m[3]), (m[0] + m[1]) - (m[2] + m[3]), (m[0] - m[1]) - (m[2] - m[3])};
 #pragma unroll
       for (int e = 0; e < 4; e++) {
-        const __half x = __double2half(v4[e]);
+        const __half x = __double2half(rint(v4[e] * 1024.0) * (1.0 / 1024.0));  // |V4| <= 2: exact in binary16
         t_s[((NJ + (tid >> 7)) * 4 + e) * 128 + (tid & 127)] = x;
         t_s[((tid >> 7) * 4 + e) * 128 + (tid & 127)] = __double2half(v4[e] - (double)__half2float(x));
       }
@@ -175,8 +188,9 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
 
     while (have) {
       const int is_v = w_v, b = w_b, row_base = blk * 128, n_rows = min(128, w_len - row_base);
-      __half* const out = (is_v ? p.v_out : p.k_out) + (size_t)b * p.stride_b + (size_t)row_base * p.stride_t + (size_t)h * p.stride_h;
+      auto out_rows = [&]() { return (is_v ? p.v_out : p.k_out) + (size_t)b * p.stride_b + (size_t)row_base * p.stride_t + (size_t)h * p.stride_h; };
       if (failed) {  // no more MMAs
+        __half* const out = out_rows();
         for (int i = gt; i < n_rows * (D / 8); i += GT)
           *reinterpret_cast<uint4*>(out + (long long)(i / (D / 8)) * p.stride_t + 8 * (i % (D / 8))) = make_uint4(HALF2_NAN, HALF2_NAN, HALF2_NAN, HALF2_NAN);
         it += NG;
@@ -185,11 +199,14 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
         continue;
       }
       const float f = scale * q.factor[is_v] * (1.0f / (float)D);  // 1/sqrt(d) of the dequantisation times 1/sqrt(d) of H_d
-      uint32_t l_lo[4], l_hi[4];
+      const int passes = SPLIT ? q.passes[is_v] : 1;
 #pragma unroll
-      for (int i = 0; i < 4; i++) { l_lo[i] = q.lo[is_v][i]; l_hi[i] = q.hi[is_v][i]; }
+      for (int hf = 0; hf < NJ; hf++)
+#pragma unroll 1
+      for (int ps = 0; ps < passes; ps++) {
+        uint32_t l_lo[4], l_hi[4];
 #pragma unroll
-      for (int hf = 0; hf < NJ; hf++) {
+        for (int i = 0; i < 4; i++) { l_lo[i] = q.lo[is_v][ps][i]; l_hi[i] = q.hi[is_v][ps][i]; }
 #pragma unroll
         for (int u = 0; u < UPH; u++) {  // 32 entries -> four 16-byte pieces of the operand
           uint32_t lv[16];
@@ -208,22 +225,21 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
         if (gt < 32 && elect_one()) {
           tc_fence_after();
           const uint64_t ad0 = is_v ? smem_desc_mn(smem_u32(xs), 128, 2048) : smem_desc_k128(smem_u32(xs));
+          const uint32_t idesc = TILE_IDESC | (is_v ? TILE_IDESC_MN_A : 0u);
 #pragma unroll
-          for (int j = 0; j < NJ; j++)
+          for (int hl = 0; hl < 2; hl++) {  // W_lo, then W_hi
+            if (passes > 1 && hl != (ps > 0)) continue;
+            const uint64_t bd0 = smem_desc_k128(smem_u32(smem + (2 * hf + hl) * TILE_OPERAND));
 #pragma unroll
-            for (int hl = 0; hl < 2; hl++) {  // W_lo, then W_hi
-              const uint64_t bd0 = smem_desc_k128(smem_u32(smem + (2 * hf + hl) * TILE_OPERAND));
-              const uint32_t idesc = TILE_IDESC | ((j & hf) ? TILE_IDESC_NEG_A : 0u) | (is_v ? TILE_IDESC_MN_A : 0u);
-#pragma unroll
-              for (int k = 0; k < 8; k++) {
-                const uint64_t step = (uint64_t)((k >> 2) * (TILE_OPERAND / 2) + (k & 3) * 32) >> 4;
-                tc_mma_f16_ss(tmem_g + 128 * j, ad0 + (is_v ? (uint64_t)(16 * k) : step), bd0 + step, idesc, (hf | hl | k) != 0);
-              }
+            for (int k = 0; k < 8; k++) {
+              const uint64_t step = (uint64_t)((k >> 2) * (TILE_OPERAND / 2) + (k & 3) * 32) >> 4;
+              tc_mma_f16_ss(tmem_g + 128 * hf, ad0 + (is_v ? (uint64_t)(16 * k) : step), bd0 + step, idesc, (ps | hl | k) != 0);
             }
+          }
           tc_commit(bar);
         }
         __syncwarp();
-        if (hf == NJ - 1) {  // the next tile's codes are on their way during the rest
+        if (hf == NJ - 1 && ps == passes - 1) {  // the next tile's codes are on their way during the rest
           it += NG;
           have = it < seg_hi;
           if (have) fetch();
@@ -232,27 +248,40 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
         phase ^= 1u;
       }
       tc_fence_after();
+      __half* const out = out_rows();
 
-      // ---- this thread's 128 columns of row r: scale, round, through the operand's buffer (256 bytes per row and round)
+      // ---- this thread's columns of row r (d = 256: 64 of each half's result): scale, round, through the operand's buffer
+      // (256 bytes per row and round)
 #pragma unroll
       for (int rd = 0; rd < NJ; rd++) {
         if (rd > 0) cta_bar_sync_n(bar_id, GT);  // the round before has left the buffer
 #pragma unroll
-        for (int ch = 0; ch < UPH; ch++) {
-          uint32_t xr[32];
-          tc_ld32(tmem_t + 32 * (UPH * rd + ch), xr);
+        for (int ch = 0; ch < UPH / NJ; ch++) {  // 32 columns (d = 256: of both halves, which make 64 coordinates)
+          uint32_t xr[NJ][32];
+          tc_ld32(tmem_t + 32 * (NJ == 1 ? ch : rd), xr[0]);
+          if constexpr (NJ == 2) tc_ld32(tmem_t + 128 + 32 * rd, xr[1]);
 #pragma unroll
-          for (int k = 0; k < 4; k++) {
-            uint32_t o[4];
+          for (int s = 0; s < NJ; s++)
 #pragma unroll
-            for (int i = 0; i < 4; i++) o[i] = pack_half2(__uint_as_float(xr[8 * k + 2 * i]) * f, __uint_as_float(xr[8 * k + 2 * i + 1]) * f);
-            const int c = part * (16 / NJ) + 4 * ch + k;
-            *reinterpret_cast<uint4*>(xs + r * 256 + ((c ^ (r & 7)) * 16)) = make_uint4(o[0], o[1], o[2], o[3]);
-          }
+            for (int k = 0; k < 4; k++) {
+              uint32_t o[4];
+#pragma unroll
+              for (int i = 0; i < 4; i++) {
+                float y[2];
+#pragma unroll
+                for (int e = 0; e < 2; e++) {
+                  y[e] = __uint_as_float(xr[0][8 * k + 2 * i + e]);
+                  if constexpr (NJ == 2) y[e] = s ? y[e] - __uint_as_float(xr[1][8 * k + 2 * i + e]) : y[e] + __uint_as_float(xr[1][8 * k + 2 * i + e]);
+                }
+                o[i] = pack_half2(y[0] * f, y[1] * f);
+              }
+              const int c = NJ == 1 ? 4 * ch + k : 8 * part + 4 * s + k;
+              *reinterpret_cast<uint4*>(xs + r * 256 + ((c ^ (r & 7)) * 16)) = make_uint4(o[0], o[1], o[2], o[3]);
+            }
         }
         failed = cta_bar_or_n(bar_id, GT, failed);
         const int c = gt & 15;  // piece of the row; its coordinate
-        const int coord = (c / (16 / NJ)) * 128 + rd * (128 / NJ) + (c % (16 / NJ)) * 8;
+        const int coord = NJ == 1 ? 8 * c : 128 * ((c >> 2) & 1) + 64 * (c >> 3) + 32 * rd + 8 * (c & 3);
 #pragma unroll
         for (int i = 0; i < 2048 / GT; i++) {
           const int row = (gt >> 4) + i * (GT / 16);
@@ -278,7 +307,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
 }
 
-template <int D, int BITS>
+template <int D, int BITS, bool SPLIT>
 static cudaError_t launch_one(const ReconstructTileParams& q, cudaStream_t stream) {
   using L = ReconLayout<D>;
   static bool configured[64] = {};
@@ -287,7 +316,7 @@ static cudaError_t launch_one(const ReconstructTileParams& q, cudaStream_t strea
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  auto kern = reconstruct_tile_kernel<D, BITS>;
+  auto kern = reconstruct_tile_kernel<D, BITS, SPLIT>;
   if (!configured[dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
     if (e != cudaSuccess) return e;
@@ -301,36 +330,57 @@ static cudaError_t launch_one(const ReconstructTileParams& q, cudaStream_t strea
   return launch_after_predecessor(kern, dim3((unsigned)ctas), dim3(L::THREADS), L::SMEM, stream, q);
 }
 
-// The levels of one side as binary16 values times a factor: 1 (exact binary16 levels), else 1/127 of the largest (the 8-bit
-// grid, whose multiples are exact binary16). A product may differ from the level by its own fp32 rounding only.
-static bool binary16_levels(const float* lv, int n, uint32_t (&lo)[4], uint32_t (&hi)[4], float& factor) {
+template <bool SPLIT>
+static cudaError_t launch_bits(const ReconstructTileParams& q, int head_dim, cudaStream_t stream) {
+  const int bits = q.r.bits;
+  if (head_dim == 128) return bits == 2 ? launch_one<128, 2, SPLIT>(q, stream) : (bits == 3 ? launch_one<128, 3, SPLIT>(q, stream) : launch_one<128, 4, SPLIT>(q, stream));
+  return bits == 2 ? launch_one<256, 2, SPLIT>(q, stream) : (bits == 3 ? launch_one<256, 3, SPLIT>(q, stream) : launch_one<256, 4, SPLIT>(q, stream));
+}
+
+// The operand values of one side's levels, and how many passes they take. On the 8-bit grid (factor 1/127 of the largest level) a
+// level is an integer of 7 bits and a sign: one pass. Binary16 levels that are integers of 15 bits and a sign in units of a
+// power of two: three. A product with the factor may differ from the level by its own fp32 rounding only.
+static bool operand_levels(const float* lv, int n, uint32_t (&lo)[3][4], uint32_t (&hi)[3][4], int& passes, float& factor) {
+  for (int t = 0; t < 3; t++)
+    for (int i = 0; i < 4; i++) lo[t][i] = hi[t][i] = 0u;
+  auto put = [&](int t, int i, float v) {  // false: not a binary16 value
+    const __half hv = __float2half_rn(v);
+    const uint32_t bits = __half_as_ushort(hv);
+    lo[t][i >> 2] |= (bits & 0xffu) << (8 * (i & 3));
+    hi[t][i >> 2] |= (bits >> 8) << (8 * (i & 3));
+    return fabsf(v) <= 65504.f && __half2float(hv) == v;
+  };
   float mx = 0.f;
   for (int i = 0; i < n; i++) mx = fmaxf(mx, fabsf(lv[i]));
-  for (const float f : {1.0f, mx / 127.0f}) {
-    if (!(f > 0.f)) continue;
-    bool ok = true;
-    for (int i = 0; i < 4; i++) lo[i] = hi[i] = 0u;
-    for (int i = 0; i < n; i++) {
-      const float v = f == 1.0f ? lv[i] : nearbyintf(lv[i] / f);
-      const __half hv = __float2half_rn(v);
-      ok &= fabsf(v) <= 65504.f && __half2float(hv) == v && fabsf(v * f - lv[i]) <= 2.4e-7f * fabsf(lv[i]);
-      const uint32_t bits = __half_as_ushort(hv);
-      lo[i >> 2] |= (bits & 0xffu) << (8 * (i & 3));
-      hi[i >> 2] |= (bits >> 8) << (8 * (i & 3));
-    }
+  const float f = mx / 127.0f;
+  bool grid = f > 0.f;
+  for (int i = 0; i < n; i++) grid = grid && fabsf(nearbyintf(lv[i] / f) * f - lv[i]) <= 2.4e-7f * fabsf(lv[i]);
+  if (grid) {
+    for (int i = 0; i < n; i++) put(0, i, nearbyintf(lv[i] / f));
+    passes = 1;
     factor = f;
-    if (ok) return true;
+    return true;
   }
-  return false;
+  float unit = 1.f;  // the largest power of two (at most 1) that all levels are multiples of
+  for (int i = 0; i < n; i++)
+    while (unit > 1e-9f && fmodf(lv[i], unit) != 0.f) unit *= 0.5f;
+  bool ok = mx / unit <= 32767.f;
+  for (int i = 0; i < n && ok; i++) {
+    const float h = nearbyintf(lv[i] / unit / 256.f) * 256.f * unit;
+    ok = put(0, i, lv[i]) && put(1, i, lv[i] - h) && put(2, i, h);
+  }
+  passes = 3;
+  factor = 1.f;
+  return ok;
 }
 
 bool launch_reconstruct_tiles(const ReconstructParams& p, int head_dim, int batch, cudaStream_t stream, cudaError_t& e) {
   ReconstructTileParams q;
   q.r = p;
   q.batch = batch;
-  if (!binary16_levels(p.levels_k, 1 << p.bits, q.lo[0], q.hi[0], q.factor[0]) || !binary16_levels(p.levels_v, 1 << p.bits, q.lo[1], q.hi[1], q.factor[1])) return false;
-  if (head_dim == 128) e = p.bits == 2 ? launch_one<128, 2>(q, stream) : (p.bits == 3 ? launch_one<128, 3>(q, stream) : launch_one<128, 4>(q, stream));
-  else e = p.bits == 2 ? launch_one<256, 2>(q, stream) : (p.bits == 3 ? launch_one<256, 3>(q, stream) : launch_one<256, 4>(q, stream));
+  if (!operand_levels(p.levels_k, 1 << p.bits, q.lo[0], q.hi[0], q.passes[0], q.factor[0])) return false;
+  if (!operand_levels(p.levels_v, 1 << p.bits, q.lo[1], q.hi[1], q.passes[1], q.factor[1])) return false;
+  e = q.passes[0] + q.passes[1] > 2 ? launch_bits<true>(q, head_dim, stream) : launch_bits<false>(q, head_dim, stream);
   return true;
 }
 

@@ -74,3 +74,35 @@ def test_a_wait_that_gives_up_leaves_no_ordinary_rows(iq, torch, d):  # noqa: F8
         for b, n in enumerate(lens):
             assert torch.isnan(outs[0][side][b, :n]).all() and (outs[0][side][b, n:] == 7.0).all()
         assert torch.equal(outs[65536][side], outs[None][side]) and not torch.isnan(outs[None][side]).any()
+
+
+@pytest.mark.parametrize("form", ["int8", "fp16"])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("d", [128, 256])
+def test_error_before_the_rounding_is_that_of_fp32(iq, torch, d, bits, form):  # noqa: F811
+    """Rows with outlier channels: beyond the rounding to binary16 an element is off by the fp32 operations on it (the cuts of
+    the sum as it grows, the factors: 2^-22 of it) and by the lower term of W, rounded at 2^-23: sigma 2^-23 / sqrt(3) of the
+    row's rms, 6e-7 is more than eight sigma."""
+    B, H, T = 1, 2, 1024
+    shape = iq.Shape(B, H, H, d, T, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 3, None, rot)
+    cb, cache = iq.iq_lloyd_max_codebook(d, bits, form), iq.new_cache(shape)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits)
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    k[..., :4] *= 20
+    v[..., 7:11] *= 20
+    lens = torch.full((B,), T, dtype=torch.int32, device="cuda")
+    iq.iq_quantize_append(shape, rot, cb, k, v, torch.zeros_like(lens), None, T, cache)
+    ko, vo = torch.empty_like(k), torch.empty_like(v)
+    iq.iq_reconstruct_rows(shape, rot, cb, cache, lens, ko, vo)
+    torch.cuda.synchronize()
+    refs = oracle.reconstruct_rows(rot.cpu().numpy().reshape(H, d // 4, 8), np.array(cb.levels, np.float32), cache_to_numpy(cache),
+                                   np.array([T], np.int32), H, d=d)
+    for got, ref in zip((ko, vo), refs):
+        r = np.asarray(ref)[:, :T]
+        err = np.abs(got.cpu().numpy().astype(np.float64) - r)
+        rms = np.sqrt((r ** 2).mean(axis=-1, keepdims=True))
+        beyond = err - 0.5 * np.spacing(np.abs(r).astype(np.float16)).astype(np.float64)
+        assert np.all(beyond <= 2.0 ** -22 * np.abs(r) + 6e-7 * rms), float((beyond / (2.0 ** -22 * np.abs(r) + 6e-7 * rms)).max())
