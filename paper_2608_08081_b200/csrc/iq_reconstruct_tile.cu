@@ -36,7 +36,7 @@ struct ReconstructTileParams {
   int batch;
   uint32_t lo[2][3][4], hi[2][3][4];  // K and V: low / high bytes of the binary16 operand values of each pass (4 per register)
   int passes[2];                      // 1: the values with both terms of W; 3: with the lower, the upper, the upper term
-  float factor[2];                    // level = (sum of the passes that meet the upper term) * factor
+  float factor[2];                    // level = factor * the value of the one pass, or the values of the two that meet the upper term
 };
 
 constexpr uint32_t HALF2_NAN = 0x7FFF7FFFu;
@@ -338,8 +338,9 @@ static cudaError_t launch_bits(const ReconstructTileParams& q, int head_dim, cud
 }
 
 // The operand values of one side's levels, and how many passes they take. On the 8-bit grid (factor 1/127 of the largest level) a
-// level is an integer of 7 bits and a sign: one pass. Binary16 levels that are integers of 15 bits and a sign in units of a
-// power of two: three. A product with the factor may differ from the level by its own fp32 rounding only.
+// level is an integer of 7 bits and a sign: one pass, if its product with the factor rounds to the level in fp32; levels
+// that are off the grid by an fp32 place or two take three, with the difference as the middle one (rounded to 11 bits, 2^-33 of the
+// level). Binary16 levels that are integers of 15 bits and a sign in units of a power of two: three.
 static bool operand_levels(const float* lv, int n, uint32_t (&lo)[3][4], uint32_t (&hi)[3][4], int& passes, float& factor) {
   for (int t = 0; t < 3; t++)
     for (int i = 0; i < 4; i++) lo[t][i] = hi[t][i] = 0u;
@@ -352,13 +353,23 @@ static bool operand_levels(const float* lv, int n, uint32_t (&lo)[3][4], uint32_
   };
   float mx = 0.f;
   for (int i = 0; i < n; i++) mx = fmaxf(mx, fabsf(lv[i]));
-  const float f = mx / 127.0f;
-  bool grid = f > 0.f;
-  for (int i = 0; i < n; i++) grid = grid && fabsf(nearbyintf(lv[i] / f) * f - lv[i]) <= 2.4e-7f * fabsf(lv[i]);
-  if (grid) {
-    for (int i = 0; i < n; i++) put(0, i, nearbyintf(lv[i] / f));
-    passes = 1;
-    factor = f;
+  const float f0 = mx / 127.0f;
+  bool near_grid = f0 > 0.f;
+  for (int i = 0; i < n; i++) near_grid = near_grid && fabsf(nearbyintf(lv[i] / f0) * f0 - lv[i]) <= 2.4e-7f * fabsf(lv[i]);
+  if (near_grid) {
+    passes = 3;
+    factor = f0;
+    for (const float f : {f0, nextafterf(f0, 0.f), nextafterf(f0, INFINITY)}) {
+      bool grid = true;
+      for (int i = 0; i < n; i++) grid = grid && nearbyintf(lv[i] / f) * f == lv[i];
+      if (grid) { passes = 1; factor = f; break; }
+    }
+    for (int i = 0; i < n; i++) {
+      const float v = nearbyintf(lv[i] / factor);
+      put(0, i, v);
+      put(1, i, (float)(((double)lv[i] - (double)v * factor) / factor));
+      put(2, i, v);
+    }
     return true;
   }
   float unit = 1.f;  // the largest power of two (at most 1) that all levels are multiples of

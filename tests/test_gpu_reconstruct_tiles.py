@@ -106,3 +106,25 @@ def test_error_before_the_rounding_is_that_of_fp32(iq, torch, d, bits, form):  #
         rms = np.sqrt((r ** 2).mean(axis=-1, keepdims=True))
         beyond = err - 0.5 * np.spacing(np.abs(r).astype(np.float16)).astype(np.float64)
         assert np.all(beyond <= 2.0 ** -22 * np.abs(r) + 6e-7 * rms), float((beyond / (2.0 ** -22 * np.abs(r) + 6e-7 * rms)).max())
+
+
+@pytest.mark.parametrize("d", [128, 256])
+def test_levels_off_the_grid_by_an_fp32_place_are_used_as_they_are(iq, torch, d):  # noqa: F811
+    """Identity blocks and a row of equal codes: its first element is scale * level. The level 1 + 2^-11 + 2^-23 is one place
+    above a multiple of the grid and rounds to 1 + 2^-10 in binary16, the multiple (a tie) to 1."""
+    f = np.float32(2049 / 2 ** 17)
+    level = np.float32(1 + 2.0 ** -11 + 2.0 ** -23)
+    lv = (-127 * float(f), 3 * float(f), float(level), 127 * float(f))
+    cb = iq.Codebook(lv, (-1.0, 0.5, 1.5))
+    shape = iq.Shape(1, 1, 1, d, 128, bits=2)
+    rot = torch.empty(iq.iq_rotation_floats(d, 1), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, 1, 0, np.tile(np.array([1, 0, 0, 0, 1, 0, 0, 0], np.float32), (1, d // 4, 1)), rot)
+    cache = iq.new_cache(shape)
+    for codes, scales in ((cache.k_codes, cache.k_scales), (cache.v_codes, cache.v_scales)):
+        codes.fill_(0xAA)   # code 2 everywhere
+        scales.fill_(1.0)
+    ko, vo = (torch.zeros((1, 128, 1, d), dtype=torch.float16, device="cuda") for _ in range(2))
+    iq.iq_reconstruct_rows(shape, rot, cb, cache, torch.tensor([128], dtype=torch.int32, device="cuda"), ko, vo)
+    torch.cuda.synchronize()
+    for o in (ko, vo):
+        assert (o[..., 0] == 1 + 2.0 ** -10).all() and (o[..., 1:] == 0).all()
