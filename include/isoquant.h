@@ -206,6 +206,13 @@ int iq_quantize_append(const iq_shape* shape, const float* rot_dev, const iq_cod
                        const void* k_new, const void* v_new, int64_t stride_b, int64_t stride_t,
                        int64_t stride_h, const int32_t* append_pos_dev, const int32_t* n_new_dev,
                        int32_t n_new_max, const iq_cache* cache, uint32_t* status_dev, void* stream);
+/* Diagnostic: the same call with `polls` (0 .. 65536) as the limit of the bulk kernel's waits for tensor-core results. 0:
+ * they give up at once, IQ_STATUS_WAIT_TIMEOUT is set, the MMAs in flight are waited for before the kernel returns; the
+ * rows that the call was to append are invalid, others are left as they are. */
+int iq_selftest_append_wait(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
+                            const void* k_new, const void* v_new, int64_t stride_b, int64_t stride_t,
+                            int64_t stride_h, const int32_t* append_pos_dev, const int32_t* n_new_dev,
+                            int32_t n_new_max, const iq_cache* cache, uint32_t* status_dev, uint32_t polls, void* stream);
 
 /*
  * Fused decode step on the packed cache (Appendix A; Table 2, kernels A-C), split over the context.

@@ -34,6 +34,7 @@ from .binding import (  # noqa: F401
     iq_suggest_splits,
     iq_fit_rotation,
     iq_format_version,
+    iq_selftest_append_wait,
     iq_selftest_bounded_wait,
     iq_selftest_reconstruct_wait,
     iq_version,

@@ -83,6 +83,7 @@ def _load():
     lib.iq_wht_coordinates.argtypes = [ctypes.POINTER(_IqShape), _vp, _i64, _i64, _i64, _vp, _i32, _vp, _vp]
     lib.iq_fit_rotation.argtypes = [_vp, _i32, _i64, _i32, ctypes.POINTER(_IqCodebook), _vp, _vp]
     lib.iq_selftest_bounded_wait.argtypes = [_vp, ctypes.c_uint32, _vp]
+    lib.iq_selftest_append_wait.argtypes = lib.iq_quantize_append.argtypes[:-1] + [ctypes.c_uint32, _vp]
     lib.iq_selftest_reconstruct_wait.argtypes = lib.iq_reconstruct_rows.argtypes[:-1] + [ctypes.c_uint32, _vp]
     lib.iq_decode_step_workspace_bytes.argtypes = [ctypes.POINTER(_IqShape), _i32]
     lib.iq_decode_step_workspace_bytes.restype = ctypes.c_size_t
@@ -430,6 +431,15 @@ def iq_fit_rotation(z_rows, head_dim: int, codebook: Codebook, quats):
     _check(_lib.iq_fit_rotation(z.ctypes.data, z.shape[0], z.shape[1], head_dim, ctypes.byref(cb), q.ctypes.data,
                                 ctypes.cast(dist, ctypes.c_void_p)), "iq_fit_rotation")
     return q, float(dist[0]), float(dist[1])
+
+
+def iq_selftest_append_wait(shape: Shape, rot_dev, codebook: Codebook, k_new, v_new, append_pos_dev, n_new_dev, n_new_max: int, cache: Cache,
+                            status_dev, polls: int, stream=None) -> None:
+    sb, st, sh = k_new.stride(0), k_new.stride(1), k_new.stride(2)
+    cs, cb, cc = shape.c(), codebook.c(), cache.c()
+    _check(_lib.iq_selftest_append_wait(ctypes.byref(cs), _ptr(rot_dev), ctypes.byref(cb), _ptr(k_new), _ptr(v_new), sb, st, sh,
+                                        _ptr(append_pos_dev), _ptr(n_new_dev), n_new_max, ctypes.byref(cc), _ptr(status_dev),
+                                        int(polls), _stream(stream)), "iq_selftest_append_wait")
 
 
 def iq_selftest_reconstruct_wait(shape: Shape, rot_dev, codebook: Codebook, cache: Cache, seq_lens_dev, k_out, v_out, polls: int, stream=None) -> None:

@@ -380,10 +380,10 @@ int iq_make_rotation(int32_t head_dim, int32_t n_kv_heads, uint64_t seed, const 
   return e == cudaSuccess ? IQ_OK : IQ_ERR_CUDA;
 }
 
-int iq_quantize_append(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const void* k_new,
-                       const void* v_new, int64_t stride_b, int64_t stride_t, int64_t stride_h,
-                       const int32_t* append_pos_dev, const int32_t* n_new_dev, int32_t n_new_max,
-                       const iq_cache* cache, uint32_t* status_dev, void* stream) {
+static int quantize_append(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const void* k_new,
+                           const void* v_new, int64_t stride_b, int64_t stride_t, int64_t stride_h,
+                           const int32_t* append_pos_dev, const int32_t* n_new_dev, int32_t n_new_max,
+                           const iq_cache* cache, uint32_t* status_dev, uint32_t wait_polls, void* stream) {
   int rc = check_shape(shape);
   if (rc) return rc;
   if (!rot_dev || !append_pos_dev) return IQ_ERR_NULL;
@@ -418,8 +418,26 @@ int iq_quantize_append(const iq_shape* shape, const float* rot_dev, const iq_cod
   p.t_cap = shape->t_cap;
   p.pm = page_map(cache, shape);
   p.scale_f16 = cache->scales_fp16 ? 1 : 0;
+  p.wait_polls = wait_polls;
   const cudaError_t e = iq::launch_quantize_append(p, shape->head_dim, shape->batch, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? IQ_OK : IQ_ERR_CUDA;
+}
+
+int iq_quantize_append(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const void* k_new,
+                       const void* v_new, int64_t stride_b, int64_t stride_t, int64_t stride_h,
+                       const int32_t* append_pos_dev, const int32_t* n_new_dev, int32_t n_new_max,
+                       const iq_cache* cache, uint32_t* status_dev, void* stream) {
+  return quantize_append(shape, rot_dev, codebook, k_new, v_new, stride_b, stride_t, stride_h, append_pos_dev, n_new_dev, n_new_max,
+                         cache, status_dev, iq::DEC_WAIT_LIMIT, stream);
+}
+
+int iq_selftest_append_wait(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook, const void* k_new,
+                            const void* v_new, int64_t stride_b, int64_t stride_t, int64_t stride_h,
+                            const int32_t* append_pos_dev, const int32_t* n_new_dev, int32_t n_new_max,
+                            const iq_cache* cache, uint32_t* status_dev, uint32_t polls, void* stream) {
+  if (polls > iq::DEC_WAIT_LIMIT) return IQ_ERR_LIMIT;
+  return quantize_append(shape, rot_dev, codebook, k_new, v_new, stride_b, stride_t, stride_h, append_pos_dev, n_new_dev, n_new_max,
+                         cache, status_dev, polls, stream);
 }
 
 // Validation and kernel parameters shared by the decode entry points.

@@ -72,8 +72,8 @@ struct BulkLayout {
   static constexpr int OFF_PRE = OFF_WARP + (PACK / 32) * 32;           // [THREADS + 1] int64 block counts before a slice of the batch
   static constexpr int OFF_WSUM = OFF_PRE + 8 * (THREADS + 2);
   static constexpr int OFF_TAU = OFF_WSUM + 8 * 32;                     // [2][16] BIG * threshold, K and V
-  static constexpr int OFF_BAR = OFF_TAU + 128;                         // [NG][4] mbarriers: tile described, copied in, norms, accumulator
-  static constexpr int OFF_MISC = OFF_BAR + 8 * (4 * NG);
+  static constexpr int OFF_BAR = OFF_TAU + 128;                         // [NG][5] mbarriers: tile described, copied in, norms, accumulator, drained
+  static constexpr int OFF_MISC = OFF_BAR + 8 * (5 * NG + (NG & 1));
   static constexpr int SMEM = OFF_MISC + 32 + 1024;                     // + alignment of the swizzle atoms
 };
 static_assert(BulkLayout<128>::SMEM <= 227 * 1024 && BulkLayout<256>::SMEM <= 227 * 1024, "shared memory overflow");
@@ -327,10 +327,11 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   const bool control = tid >= L::PACK;
   const int grp = control ? warp - L::PACK / 32 : tid / GT;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::OFF_BAR);
-  uint64_t* tile_bar = bars + 4 * grp;      // the next tile has been described
-  uint64_t* copy_bar = bars + 4 * grp + 1;  // the tile (half) is in the buffer, the accumulator has been read
-  uint64_t* norm_bar = bars + 4 * grp + 2;  // the norms are in shared memory, the buffer has been read
-  uint64_t* full_bar = bars + 4 * grp + 3;  // the MMAs are done
+  uint64_t* tile_bar = bars + 5 * grp;       // the next tile has been described
+  uint64_t* copy_bar = bars + 5 * grp + 1;   // the tile (half) is in the buffer, the accumulator has been read
+  uint64_t* norm_bar = bars + 5 * grp + 2;   // the norms are in shared memory, the buffer has been read
+  uint64_t* full_bar = bars + 5 * grp + 3;   // the MMAs are done
+  uint64_t* drain_bar = bars + 5 * grp + 4;  // (after a wait that gave up) all MMAs of the group are done
   BulkTile* tiles = reinterpret_cast<BulkTile*>(smem + L::OFF_TILE) + 2 * grp;
   uint8_t* xs = smem + L::OFF_X + grp * L::OPERAND;
   long long* pre_s = reinterpret_cast<long long*>(smem + L::OFF_PRE);
@@ -351,6 +352,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
     mbar_init(copy_bar, GT);
     mbar_init(norm_bar, GT);
     mbar_init(full_bar, 1);
+    mbar_init(drain_bar, 1);
     fence_mbar_init();
   }
   if (tid == L::PACK) {
@@ -570,7 +572,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           mbar_arrive(norm_bar);  // everybody has read the first half ...
           if (!failed) failed = !mbar_wait_bounded(norm_bar, n_norm & 1u, DEC_WAIT_LIMIT);
           n_norm++;
-          if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, DEC_WAIT_LIMIT);  // ... the MMAs too
+          if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, p.wait_polls);  // ... the MMAs too
           load_half(*t, 1);
           copied_in();
           n_half++;
@@ -611,7 +613,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         mbar_arrive(norm_bar);
         if (!failed) failed = !mbar_wait_bounded(norm_bar, n_norm & 1u, DEC_WAIT_LIMIT);
         n_norm++;
-        if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, DEC_WAIT_LIMIT);
+        if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, p.wait_polls);
         tc_fence_after();
         const bool special = t->special != 0;
         // the next tile's copy runs under the packing of this one
@@ -737,6 +739,11 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   if (n_redone && p.status) atomicAdd(&p.status[1], n_redone);
   if (failed && tid == 0 && p.status) atomicOr(&p.status[0], IQ_STATUS_WAIT_TIMEOUT);
   cp_async_wait_all();
+  if (failed && control) {  // MMAs may still be running: they are waited for, again with a limit, before the tensor memory goes
+    if (elect_one()) tc_commit(drain_bar);
+    __syncwarp();
+    mbar_wait_bounded(drain_bar, 0u, DEC_WAIT_LIMIT);
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));

@@ -102,3 +102,40 @@ def test_codebook_with_close_thresholds_keeps_its_path(iq, torch):  # noqa: F811
     a, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], T, 0, torch.float32)
     b, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], 4, 0, torch.float32)
     assert torch.equal(a.k_codes, b.k_codes) and torch.equal(a.v_codes, b.v_codes)
+
+
+@pytest.mark.parametrize("d", [128, 256])
+def test_a_wait_that_gives_up_is_reported(iq, torch, d):  # noqa: F811
+    """A limit of 0 polls for the tensor-core results: the flag is set, the call returns within the limit of the other waits,
+    rows that it was not to append stay, and the next call over the same rows is an ordinary one."""
+    B, H, T = 3, 2, 700
+    shape = iq.Shape(B, H, H, d, 1024)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 5, None, rot)
+    cb = iq.iq_lloyd_max_codebook(d, 3, "int8")
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    caches = [iq.new_cache(shape) for _ in range(2)]
+    for c in caches:
+        c.k_codes.fill_(0x5A)
+        c.k_scales.fill_(3.0)
+    pos = torch.tensor([0, 100, 250], dtype=torch.int32, device="cuda")
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    iq.iq_selftest_append_wait(shape, rot, cb, k, v, pos, None, T, caches[0], status, 0)
+    torch.cuda.synchronize()
+    assert int(status[0]) == 2
+    for b, p in enumerate(pos.tolist()):
+        for a in (caches[0].k_codes, caches[0].k_scales):
+            outside = torch.cat([a[b, :, :p], a[b, :, p + T:]], dim=1)
+            assert (outside == (0x5A if a is caches[0].k_codes else 3.0)).all()
+    status.zero_()
+    for c in caches:
+        iq.iq_quantize_append(shape, rot, cb, k, v, pos, None, T, c, status)
+    torch.cuda.synchronize()
+    assert int(status[0]) == 0
+    assert torch.equal(caches[0].k_codes, caches[1].k_codes) and torch.equal(caches[0].k_scales, caches[1].k_scales)
+    for b, p in enumerate(pos.tolist()):   # whole new blocks of V
+        lo, hi = (p + 127) // 128, (p + T) // 128
+        va, vb = (c.v_codes.reshape(B, H, 8, -1)[b, :, lo:hi] for c in caches)
+        assert torch.equal(va, vb)
