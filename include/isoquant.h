@@ -200,7 +200,8 @@ int iq_make_rotation(int32_t head_dim, int32_t n_kv_heads, uint64_t seed, const 
  * tensor-core contraction with the rotation as two binary16 terms); a coordinate closer than 2^-15 (2^-16) to a
  * decision threshold is re-decided in fp64 inside the kernel, so the codes equal those of an fp64
  * evaluation except for ties at the fp64 rounding level. The stored scale is sqrt(sum x^2) accumulated
- * in fp64 and rounded to fp32. A zero row stores scale 0 and the code of u = 0 everywhere.
+ * in fp64 and rounded to fp32. A zero row stores scale 0 and the code of u = 0 everywhere; a row with an infinity or a NaN
+ * stores its norm (inf or NaN) and code 0 everywhere: u is not a number, and not above any threshold.
  */
 int iq_quantize_append(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
                        const void* k_new, const void* v_new, int64_t stride_b, int64_t stride_t,

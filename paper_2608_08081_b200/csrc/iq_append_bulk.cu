@@ -649,9 +649,9 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
                 const uint32_t cb = __float_as_uint(bulk_decide<BITS, SYM, NS>(x, b, off));
                 uint32_t code = ((cb + 0x0003FFFFu) >> 19) & 15u;
                 const bool odd_c = (cb & 0x0007FFFFu) != 0u;
-                if (b == 0.f) {  // a row of norm zero: u = 0; one whose norm is not finite: not a number
+                if (b == 0.f) {  // a row of norm zero: u = 0; one whose norm is not finite: not a number, above no threshold
                   const float z = x * 0.f;
-                  code = z != z ? (SYM && BITS == 3 ? 3u : 0u) : (uint32_t)zero_code_s[is_v ? 1 : 0];
+                  code = z != z ? 0u : (uint32_t)zero_code_s[is_v ? 1 : 0];
                 } else if (odd_c && row >= c_lo && row < c_hi) {
                   near_m |= 1u << i;
                 }

@@ -139,3 +139,44 @@ def test_a_wait_that_gives_up_is_reported(iq, torch, d):  # noqa: F811
         lo, hi = (p + 127) // 128, (p + T) // 128
         va, vb = (c.v_codes.reshape(B, H, 8, -1)[b, :, lo:hi] for c in caches)
         assert torch.equal(va, vb)
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("grid", ["symmetric", "shifted"])
+def test_rows_that_are_not_finite(iq, torch, bits, d, grid):  # noqa: F811
+    """Rows with an infinity or a NaN in a prompt: code 0 everywhere and a norm that is not finite, as in calls of up to four
+    rows; the rows next to them in the same tile as if they were not there."""
+    B, H, T = 1, 2, 260
+    lv, th, _, _ = two_codebooks(d, bits, "int8", False)
+    if grid == "shifted":
+        th = (th.astype(np.float64) + 0.01 * ((np.arange(len(th)) * 7) % 5 - 2)).astype(np.float32)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)))
+    shape = iq.Shape(B, H, H, d, 384, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 2, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits)
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    bad = {0: float("inf"), 5: float("nan"), 64: float("-inf"), 127: float("nan"), 128: float("inf"), 259: float("-inf")}
+    plain_k, plain_v = k.clone(), v.clone()
+    for r, x in bad.items():
+        for a in (k, v):
+            a[:, r, :, r % d] = x
+        if r == 64:
+            k[:, r, :, 1] = float("inf")   # two infinities of opposite sign
+    whole, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], T, 0, torch.float32)
+    rows, _ = _append(iq, torch, shape, rot, cb, k, v, [0], [T], 4, 0, torch.float32)
+    plain, _ = _append(iq, torch, shape, rot, cb, plain_k, plain_v, [0], [T], T, 0, torch.float32)
+    good = [r for r in range(T) if r not in bad]
+    for h in range(H):
+        for name in ("k_codes", "v_codes", "k_scales", "v_scales"):
+            a, b, c = (cache_to_numpy(x)[name][0, h] for x in (whole, rows, plain))
+            if name.endswith("scales"):
+                assert np.array_equal(a.view(np.int32)[good], c.view(np.int32)[good]) and not np.isfinite(a[list(bad)]).any()
+                assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b))
+                continue
+            codes = [[oracle.unpack_row(d, x[r], bits) if name == "k_codes" else oracle.v_row_codes(d, x, r, bits) for r in range(T)] for x in (a, b, c)]
+            codes = np.array(codes)
+            assert np.array_equal(codes[0][good], codes[2][good]) and np.array_equal(codes[0], codes[1])
+            assert (codes[0][list(bad)] == 0).all()
