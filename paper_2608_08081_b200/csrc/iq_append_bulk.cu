@@ -16,7 +16,10 @@
 // fraction inside a band of +-GUARD around the threshold. The code is the sum; a sum that is not a whole number (16 + code
 // is kept, so its fraction bits are the same for all codes; they are OR-ed over 8 coordinates) marks a coordinate too
 // close to call, which is put on a list and decided again in fp64 by eight lanes (exact +-1 sums, the norm and the block
-// in fp64). So the codes are those of an fp64 evaluation. GUARD covers the error of the fp32 sums near a threshold: W
+// in fp64). Where 8 columns of a warp have many, or the list is full (rows with ties throughout: constant rows, rows whose
+// Walsh-Hadamard coordinates vanish), the rows are marked instead; the group's warps share the marked rows of a tile when
+// the next one has been copied in, a row at a time by a warp. 4 x 8 K constant rows, d = 128, 3 bits: 0.77 ms, every 13th row
+// constant 0.28 (ordinary rows 0.081); with every warp of a V tile deciding all rows, code by code: 8.8 and 0.9. So the codes are those of an fp64 evaluation. GUARD covers the error of the fp32 sums near a threshold: W
 // (2^-22 sqrt(d)) and one cut of the running sum per instruction -- a sum that ends near a threshold stays below
 // sqrt(d) / 2 + 2.8 on the way (Cauchy-Schwarz on the two parts), so 8 cuts of 2^-21 at d = 128, 16 of 2^-20 at d = 256:
 // 6.5e-6 and 1.9e-5. Measured over 16 M coordinates each of Gaussian, outlier, heavy-tailed and cancelling rows: no code
@@ -59,7 +62,9 @@ struct BulkLayout {
   static constexpr int OPERAND = TILE_OPERAND;
   static constexpr int W_BYTES = NJ * 2 * OPERAND;
   static constexpr int LIST = 48;                 // undecided coordinates a warp collects ...
+  static constexpr int LIST_STEP = 12;            // ... unless 8 columns have more: rows with ties throughout, decided as a whole
   static constexpr int LIST_FLUSH = 32;           // ... and decides in fp64 after a tile that left it with this many, or at the end
+  static constexpr int TILES = 4;                 // tile descriptors kept: the next, the present, and the one before (its rows are redone late)
   // shared memory: W, the groups' tile buffers (128 contraction steps), the warps' lists, the rest
   static constexpr int OFF_X = W_BYTES;
   static constexpr int OFF_LIST = OFF_X + NG * OPERAND;
@@ -67,9 +72,10 @@ struct BulkLayout {
   static constexpr int OFF_BINV = OFF_LIST + (PACK / 32) * LIST_BYTES;  // [NG][128] BIG / s of the rows of a group's tile
   static constexpr int OFF_SS = OFF_BINV + NG * 512;                    // [NG][2][128] fp64 partial square sums (d = 256)
   static constexpr int OFF_M = OFF_SS + (NJ > 1 ? NG * 2048 : 0);       // [D][4] fp64 rows of the blocks M_b
-  static constexpr int OFF_TILE = OFF_M + D * 32;                       // [NG][2] tile descriptors
-  static constexpr int OFF_WARP = OFF_TILE + NG * 2 * 48;               // [16] the warps' list state
-  static constexpr int OFF_PRE = OFF_WARP + (PACK / 32) * 32;           // [THREADS + 1] int64 block counts before a slice of the batch
+  static constexpr int OFF_TILE = OFF_M + D * 32;                       // [NG][TILES] tile descriptors
+  static constexpr int OFF_ROWS = OFF_TILE + NG * TILES * 48;           // [NG] rows to be decided again
+  static constexpr int OFF_WARP = OFF_ROWS + NG * 32;                   // [16] coordinates on the warps' lists
+  static constexpr int OFF_PRE = OFF_WARP + (PACK / 32) * 4;            // [THREADS + 1] int64 block counts before a slice of the batch
   static constexpr int OFF_WSUM = OFF_PRE + 8 * (THREADS + 2);
   static constexpr int OFF_TAU = OFF_WSUM + 8 * 32;                     // [2][16] BIG * threshold, K and V
   static constexpr int OFF_BAR = OFF_TAU + 128;                         // [NG][5] mbarriers: tile described, copied in, norms, accumulator, drained
@@ -87,12 +93,9 @@ struct BulkTile {       // a tile, as the control warp hands it to its group
   int pad[4];
 };
 static_assert(sizeof(BulkTile) == 48, "tile descriptor");
-struct BulkWarp {       // a packing warp's list
-  int n;                // coordinates put on it (beyond LIST: only their rows are remembered, in `full`)
-  uint32_t full[4];     // rows of the tile that are decided again as a whole
-  int pad[3];
+struct BulkRows {       // rows of a tile that are decided again as a whole: of the group's present tile and of the one before, by its
+  uint32_t full[2][4];  // parity. Set by all warps at the end of a tile, read by all when the next one is copied in
 };
-static_assert(sizeof(BulkWarp) == 32, "list state");
 
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -190,28 +193,133 @@ static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const dou
   }
 }
 
-// Whole rows again (rows of which the list could not take every undecided coordinate), one after the other by the warp.
-// All codes of the row are set, also those that other warps of the group pack: a warp that stores its own later stores
-// codes that are either these or on its own list.
+// The codes of a row in fp64 throughout (exact +-1 sums, the blocks from shared memory): lane l those of coordinates l E ...
 template <int D, int BITS>
-static __device__ __noinline__ void bulk_redo_rows(const QuantizeParams& p, const float* rot_head, const uint32_t* full, const __half* src0,
-                                                   size_t row0, int is_v, int lane) {
-  constexpr int E = D / 32;
-  WarpRowQuantizer<D, BITS> rq;
-  rq.init(rot_head, is_v ? p.thresholds_v : p.thresholds_k, lane);
-  for (int r = 0; r < 128; r++) {
-    if (!((full[r >> 5] >> (r & 31)) & 1u)) continue;
-    const __half2* src = reinterpret_cast<const __half2*>(src0 + (long long)r * p.stride_t + lane * E);
-    __half2 raw[E / 2];
+static __device__ __forceinline__ void bulk_exact_row(const __half* src_row, const double* m_s, const float (&th)[(1 << BITS) - 1], int lane, int (&code)[D / 32]) {
+  constexpr int E = D / 32, NT = (1 << BITS) - 1;
+  const __half2* src = reinterpret_cast<const __half2*>(src_row + lane * E);
+  double v[E], ss = 0.0;
 #pragma unroll
-    for (int k = 0; k < E / 2; k++) raw[k] = src[k];
-    int code[E];
-    rq.run(raw, lane, code, nullptr);
+  for (int k = 0; k < E / 2; k++) {
+    const float2 f = __half22float2(src[k]);
+    v[2 * k] = (double)f.x;
+    v[2 * k + 1] = (double)f.y;
+    ss += (double)(f.x * f.x) + (double)(f.y * f.y);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(FULL, ss, o);
+  wht_warp<double, E>(v, lane);
+  const double inv = ss > 0.0 ? inv_sqrt(ss) : 0.0;
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const double* m = m_s + 4 * (lane * E + e);
+    const double* z = v + (e & ~3);
+    bool nb;
+    code[e] = decide_code_n<double, NT>((m[0] * z[0] + m[1] * z[1] + m[2] * z[2] + m[3] * z[3]) * inv, th, nb, 0.0);
+  }
+}
+
+// 8 mask bits -> the lowest bits of the 8 nibbles of a word.
+__device__ __forceinline__ uint32_t spread8(uint32_t b) {
+  b &= 0xffu;
+  b = (b | (b << 12)) & 0x000F000Fu;
+  b = (b | (b << 6)) & 0x03030303u;
+  return (b | (b << 3)) & 0x11111111u;
+}
+// The packed words of 32 entries from their codes as four words of nibbles.
+template <int BITS>
+__device__ __forceinline__ void pack_nibbles(const uint32_t (&nib)[4], uint32_t* word) {
+  if constexpr (BITS == 4) {
+#pragma unroll
+    for (int q = 0; q < 4; q++) word[q] = nib[q];
+  } else if constexpr (BITS == 3) {  // entries 24..31: bit k of the code into the top bits of word k's nibbles
+    word[0] = nib[0] | ((nib[3] & 0x11111111u) << 3);
+    word[1] = nib[1] | ((nib[3] & 0x22222222u) << 2);
+    word[2] = nib[2] | ((nib[3] & 0x44444444u) << 1);
+  } else {
+    word[0] = nib[0] | (nib[1] << 2);
+    word[1] = nib[2] | (nib[3] << 2);
+  }
+}
+// The bits of packed word k that belong to the entries of vm (32 bits, one per entry).
+template <int BITS>
+__device__ __forceinline__ uint32_t packed_mask(uint32_t vm, int k) {
+  if constexpr (BITS == 4) return spread8(vm >> (8 * k)) * 15u;
+  else if constexpr (BITS == 3) return spread8(vm >> (8 * k)) * 7u + spread8(vm >> 24) * 8u;
+  else return spread8(vm >> (16 * k)) * 3u + spread8(vm >> (16 * k + 8)) * 12u;
+}
+// Which of the 32 rows from 32 u on are new, rows [c_lo, c_hi) of the block being so.
+__device__ __forceinline__ uint32_t new_rows(int c_lo, int c_hi, int u) {
+  const int a = min(max(c_lo - 32 * u, 0), 32), z = min(max(c_hi - 32 * u, 0), 32);
+  if (a >= z) return 0u;
+  return (z == 32 ? 0xFFFFFFFFu : (1u << z) - 1u) & ~((1u << a) - 1u);
+}
+
+// Rows of which the lists did not take every undecided coordinate, again as a whole, by one warp: the rows `m` of the 32 from
+// 32 u on (V, d = 256: those of the 16 that are this warp's, `part`). Stores and changes that other warps make to the same
+// codes are of the same values, or are changed to these by their lists; words of V have other rows' codes too, which the
+// lists may be changing, so bits of part of a word are set one way and the other by atomics.
+template <int D, int BITS>
+static __device__ __noinline__ void bulk_redo_rows(const QuantizeParams& p, const double* m_s, const BulkTile* t, uint32_t m, int u, int part, int lane) {
+  constexpr int E = D / 32, NT = (1 << BITS) - 1, NJ = D / 128;
+  const bool is_v = t->kind != 0;
+  float th[NT];
+#pragma unroll
+  for (int i = 0; i < NT; i++) th[i] = is_v ? p.thresholds_v[i] : p.thresholds_k[i];
+  const uint32_t vm = m & new_rows(t->c_lo, t->c_hi, u) & (NJ == 1 || !is_v ? 0xFFFFFFFFu : (part ? 0xFFFF0000u : 0x0000FFFFu));
+  const __half* src0 = t->src + (long long)(32 * u) * p.stride_t;
+  int code[E];
+  if (!is_v) {
+    const RowSink sink{p.k_codes, p.k_scales, p.v_codes, p.v_scales, p.status, p.scale_f16};
+    m = vm;
+#pragma unroll 1
+    while (m) {
+      const int r = __ffs(m) - 1;
+      m &= m - 1u;
+      bulk_exact_row<D, BITS>(src0 + (long long)r * p.stride_t, m_s, th, lane, code);
+      warp_store_k_row<D, BITS, false>(sink, t->row0 + 32 * u + r, code, 0.f, lane);
+    }
+  } else if (vm) {
+    constexpr int Q = 4 / NJ;  // groups of 8 rows
+    const int q0 = NJ == 1 ? 0 : 2 * part;
+    uint32_t nib[E][Q];
+#pragma unroll 1
+    for (int q = 0; q < Q; q++) {
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+#pragma unroll
+        for (int i = 0; i < Q - 1; i++) nib[e][i] = nib[e][i + 1];
+        nib[e][Q - 1] = 0u;
+      }
+#pragma unroll 1
+      for (int i = 0; i < 8; i++) {
+        const int r = 8 * (q0 + q) + i;
+        if (!((vm >> r) & 1u)) continue;
+        bulk_exact_row<D, BITS>(src0 + (long long)r * p.stride_t, m_s, th, lane, code);
+#pragma unroll
+        for (int e = 0; e < E; e++) nib[e][Q - 1] |= (uint32_t)code[e] << (4 * i);
+      }
+    }
 #pragma unroll
     for (int e = 0; e < E; e++) {
-      const int c = lane * E + e;
-      if (is_v) patch_code<BITS>(reinterpret_cast<uint32_t*>(p.v_codes + ((row0 / 128) * D + c) * (size_t)(16 * BITS)), r, code[e]);
-      else patch_code<BITS>(reinterpret_cast<uint32_t*>(p.k_codes + (row0 + r) * (size_t)(BITS * D / 8)), c, code[e]);
+      uint32_t word[BITS];
+      if constexpr (NJ == 1) {
+        pack_nibbles<BITS>(nib[e], word);
+      } else {
+        const uint32_t n4[4] = {part ? 0u : nib[e][0], part ? 0u : nib[e][1], part ? nib[e][0] : 0u, part ? nib[e][1] : 0u};
+        pack_nibbles<BITS>(n4, word);
+      }
+      uint32_t* d = reinterpret_cast<uint32_t*>(p.v_codes + ((t->row0 / 128) * D + lane * E + e) * (size_t)(16 * BITS)) + BITS * u;
+#pragma unroll
+      for (int k = 0; k < BITS; k++) {
+        const uint32_t wm = packed_mask<BITS>(vm, k);
+        if (wm == 0xFFFFFFFFu) {
+          d[k] = word[k];
+        } else if (wm) {
+          atomicAnd(d + k, ~wm);
+          atomicOr(d + k, word[k]);
+        }
+      }
     }
   }
 }
@@ -249,14 +357,6 @@ static __device__ __noinline__ void bulk_build_w(const double* m_s, uint8_t* w_s
     *reinterpret_cast<uint4*>(base_hi + off) = make_uint4(hi[0] ^ s0, hi[1] ^ s0, hi[0] ^ s1, hi[1] ^ s1);
     *reinterpret_cast<uint4*>(base_lo + off) = make_uint4(lo[0] ^ s0, lo[1] ^ s0, lo[0] ^ s1, lo[1] ^ s1);
   }
-}
-
-// 8 mask bits -> the lowest bits of the 8 nibbles of a word.
-__device__ __forceinline__ uint32_t spread8(uint32_t b) {
-  b &= 0xffu;
-  b = (b | (b << 12)) & 0x000F000Fu;
-  b = (b | (b << 6)) & 0x03030303u;
-  return (b | (b << 3)) & 0x11111111u;
 }
 
 // A group's position in the tiles of a head: K tiles of all sequences, then V tiles, each sequence's blocks in order.
@@ -332,7 +432,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   uint64_t* norm_bar = bars + 5 * grp + 2;   // the norms are in shared memory, the buffer has been read
   uint64_t* full_bar = bars + 5 * grp + 3;   // the MMAs are done
   uint64_t* drain_bar = bars + 5 * grp + 4;  // (after a wait that gave up) all MMAs of the group are done
-  BulkTile* tiles = reinterpret_cast<BulkTile*>(smem + L::OFF_TILE) + 2 * grp;
+  BulkTile* tiles = reinterpret_cast<BulkTile*>(smem + L::OFF_TILE) + L::TILES * grp;
   uint8_t* xs = smem + L::OFF_X + grp * L::OPERAND;
   long long* pre_s = reinterpret_cast<long long*>(smem + L::OFF_PRE);
   long long* wsum_s = reinterpret_cast<long long*>(smem + L::OFF_WSUM);
@@ -363,7 +463,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
     for (int g = 0; g < NG; g++) started_s[g] = 0;
   }
   if (tid < 32) tau_s[tid] = (tid & 15) < NT ? BIG * (tid < 16 ? p.thresholds_k[tid & 15] : p.thresholds_v[tid & 15]) : 0.f;
-  if (tid < (L::PACK / 32) * 8) reinterpret_cast<int*>(smem + L::OFF_WARP)[tid] = 0;
+  if (tid < L::PACK / 32) reinterpret_cast<int*>(smem + L::OFF_WARP)[tid] = 0;
   grid_dependency_wait();
 
   // ---- blocks of every sequence; this CTA's share of the tiles
@@ -454,7 +554,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           BulkTile d = nt;
           d.special = 0;
           if (!found) d.kind = -1;
-          tiles[n_tile & 1u] = d;
+          tiles[n_tile % L::TILES] = d;
           mbar_arrive(tile_bar);
         }
         __syncwarp();
@@ -489,7 +589,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           }
           __syncwarp();
         }
-        have = describe_next();  // (into the slot of the tile before: the group was done with it when it had this one copied in)
+        have = describe_next();  // (into the slot of the tile four before: the group was done with it when it had the one before this copied in)
       }
     } else {
       // ================================================================ packing group: thread = tensor-memory lane (and 128-column half)
@@ -501,7 +601,8 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
       const __half** src_s = reinterpret_cast<const __half**>(list);
       uint32_t** dst_s = reinterpret_cast<uint32_t**>(list + 8 * L::LIST);
       uint32_t* info_s = reinterpret_cast<uint32_t*>(list + 16 * L::LIST);
-      BulkWarp* wl = reinterpret_cast<BulkWarp*>(smem + L::OFF_WARP) + warp;
+      int* const n_list_s = reinterpret_cast<int*>(smem + L::OFF_WARP) + warp;
+      BulkRows* rows_s = reinterpret_cast<BulkRows*>(smem + L::OFF_ROWS) + grp;
       double* m_s = reinterpret_cast<double*>(smem + L::OFF_M);
 
       // 128-coordinate half hf of a tile's rows into the group's buffer; rows that are not new repeat the nearest one that
@@ -543,10 +644,22 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
       };
       auto describe = [&]() -> BulkTile* {  // the group's next tile, or none
         if (!failed) failed = !mbar_wait_bounded(tile_bar, n_tile & 1u, DEC_WAIT_LIMIT);
-        BulkTile* t = &tiles[n_tile & 1u];
+        BulkTile* t = &tiles[n_tile % L::TILES];
         n_tile++;
         return t;
       };
+
+      // Warp w of the group decides the rows of its quarter again that are marked in tile number `no`. d = 256 has two warps per
+      // quarter: K rows go to the one or the other by turns, V rows by halves.
+      auto redo_marked = [&](uint32_t no) {
+        uint32_t m = __shfl_sync(FULL, rows_s->full[no & 1u][warp & 3], 0);
+        if (m == 0u) return;
+        const BulkTile* t = &tiles[no % L::TILES];
+        if (NJ == 2 && t->kind == 0) m &= part ? 0xAAAAAAAAu : 0x55555555u;
+        if (m != 0u) bulk_redo_rows<D, BITS>(p, m_s, t, m, warp & 3, part, lane);
+        __syncwarp();
+      };
+      if (gt < 8) reinterpret_cast<uint32_t*>(rows_s)[gt] = 0u;
 
       tile_build_m<D>(rot_head, m_s, tid);  // (while the control warps find the first tiles)
       BulkTile* t = describe();
@@ -560,6 +673,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
       while (!__any_sync(FULL, failed || kind < 0)) {
         copied_in();
         n_half++;
+        redo_marked(n_tile - 2u);  // the tile before this one, number n_tile - 1
         if (first) {  // the groups' first norms one after the other: the conversions of all groups at once would keep one
                       // pipe busy and the others idle, tile after tile
           for (int i = 0; i < 64 && grp > 0 && started_s[grp - 1] == 0; i++) __nanosleep(64);
@@ -613,6 +727,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         mbar_arrive(norm_bar);
         if (!failed) failed = !mbar_wait_bounded(norm_bar, n_norm & 1u, DEC_WAIT_LIMIT);
         n_norm++;
+        if (gt < 4) rows_s->full[n_tile & 1u][gt] = 0u;  // (everybody has read the marks of the tile before; the next tile sets its own there)
         if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, p.wait_polls);
         tc_fence_after();
         const bool special = t->special != 0;
@@ -662,35 +777,28 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
               for (int k = 0; k < 4; k++) nib[k] = (k == q) ? nw : nib[k];
               const uint32_t rows = is_v ? __reduce_or_sync(FULL, near_m) : __ballot_sync(FULL, near_m != 0u);
               if (lane == 0) n_redone += __popc(rows);
+              const int n_list = *n_list_s, n_near = (int)__reduce_add_sync(FULL, (unsigned)__popc(near_m));
+              if (n_near > L::LIST_STEP || n_list + n_near > L::LIST) {  // their rows again as a whole (the tile's number is n_tile - 2)
+                const uint32_t marked = is_v ? rows << (8 * q) : rows;
+                if (lane == 0) atomicOr(&rows_s->full[n_tile & 1u][is_v ? ch : warp & 3], marked);
+                near_m = 0u;
+              }
+              __syncwarp();
               while (near_m) {
                 const int i = __ffs(near_m) - 1, col = 32 * ch + 8 * q + i;
                 near_m &= near_m - 1u;
                 const int row = is_v ? col : r, coord = is_v ? gt : part * 128 + col;
-                const int k = atomicAdd(&wl->n, 1);
-                if (k < L::LIST) {
-                  src_s[k] = src0 + (long long)row * p.stride_t;
-                  dst_s[k] = is_v ? dst : dst - part * (4 * BITS);
-                  info_s[k] = (uint32_t)coord | ((uint32_t)(is_v ? row : coord) << 8) | (((low >> (4 * i)) & 15u) << 16) | (is_v ? 1u << 20 : 0u);
-                } else {
-                  atomicOr(&wl->full[row >> 5], 1u << (row & 31));
-                }
+                const int k = atomicAdd(n_list_s, 1);
+                src_s[k] = src0 + (long long)row * p.stride_t;
+                dst_s[k] = is_v ? dst : dst - part * (4 * BITS);
+                info_s[k] = (uint32_t)coord | ((uint32_t)(is_v ? row : coord) << 8) | (((low >> (4 * i)) & 15u) << 16) | (is_v ? 1u << 20 : 0u);
               }
               __syncwarp();
             }
           }
 #pragma unroll
           for (int i = 0; i < 3 * BITS; i++) word[i] = word[i + BITS];
-          if constexpr (BITS == 4) {
-#pragma unroll
-            for (int q = 0; q < 4; q++) word[12 + q] = nib[q];
-          } else if constexpr (BITS == 3) {  // entries 24..31: bit k of the code into the top bits of word k's nibbles
-            word[9] = nib[0] | ((nib[3] & 0x11111111u) << 3);
-            word[10] = nib[1] | ((nib[3] & 0x22222222u) << 2);
-            word[11] = nib[2] | ((nib[3] & 0x44444444u) << 1);
-          } else {
-            word[6] = nib[0] | (nib[1] << 2);
-            word[7] = nib[2] | (nib[3] << 2);
-          }
+          pack_nibbles<BITS>(nib, word + 3 * BITS);
         }
         if (is_v ? (c_lo == 0 && c_hi == 128) : (r >= c_lo && r < c_hi)) {
 #pragma unroll
@@ -699,15 +807,11 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         } else if (is_v) {  // a partly new block: the other rows' codes stay
 #pragma unroll
           for (int u = 0; u < 4; u++) {
-            const int a = min(max(c_lo - 32 * u, 0), 32), z = min(max(c_hi - 32 * u, 0), 32);
-            if (a >= z) continue;
-            const uint32_t vm = (z == 32 ? 0xFFFFFFFFu : (1u << z) - 1u) & ~((1u << a) - 1u);  // (a < 32)
+            const uint32_t vm = new_rows(c_lo, c_hi, u);
+            if (vm == 0u) continue;
 #pragma unroll
             for (int k = 0; k < BITS; k++) {
-              uint32_t m;
-              if constexpr (BITS == 4) m = spread8(vm >> (8 * k)) * 15u;
-              else if constexpr (BITS == 3) m = spread8(vm >> (8 * k)) * 7u + spread8(vm >> 24) * 8u;
-              else m = spread8(vm >> (16 * k)) * 3u + spread8(vm >> (16 * k + 8)) * 12u;
+              const uint32_t m = packed_mask<BITS>(vm, k);
               if (m == 0u) continue;
               uint32_t* d = dst + BITS * u + k;
               *d = m == 0xFFFFFFFFu ? word[BITS * u + k] : ((*d & ~m) | (word[BITS * u + k] & m));
@@ -715,21 +819,22 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           }
         }
         __syncwarp();  // the warp's stores come before the changes made to them below
-        const int n_list = wl->n;
+        const int n_list = *n_list_s;
         if (n_list >= L::LIST_FLUSH) {
-          bulk_redo<D, BITS>(p, m_s, src_s, dst_s, info_s, min(n_list, L::LIST), lane);
-          if (n_list > L::LIST) bulk_redo_rows<D, BITS>(p, rot_head, wl->full, src0, row0, is_v ? 1 : 0, lane);
+          bulk_redo<D, BITS>(p, m_s, src_s, dst_s, info_s, n_list, lane);
           __syncwarp();
-          if (lane < 5) reinterpret_cast<int*>(wl)[lane] = 0;
+          if (lane == 0) *n_list_s = 0;
           __syncwarp();
         }
       }
-      if (wl->n > 0) {
-        bulk_redo<D, BITS>(p, m_s, src_s, dst_s, info_s, wl->n, lane);
+      const int n_list = *n_list_s;
+      if (n_list > 0) {
+        bulk_redo<D, BITS>(p, m_s, src_s, dst_s, info_s, n_list, lane);
         __syncwarp();
-        if (lane == 0) wl->n = 0;
-        __syncwarp();
+        if (lane == 0) *n_list_s = 0;
       }
+      cta_bar_sync_n(2 + grp, GT);  // the marks of the group's last tile, and the stores to it, are in place
+      if (!__any_sync(FULL, failed)) redo_marked(n_tile - 2u);
     }
     item = head0 + seg_hi;
     if (__syncthreads_or(failed)) { failed = true; break; }  // (W is rebuilt for the next head)

@@ -123,8 +123,8 @@ struct RowSink {
   int scale_f16;
 };
 
-// K row `row` (index into the cache arrays): lane l holds the codes of coordinates l E .. l E + E - 1.
-template <int D, int BITS = 3>
+// K row `row` (index into the cache arrays): lane l holds the codes of coordinates l E .. l E + E - 1. SCALE: and its norm s.
+template <int D, int BITS = 3, bool SCALE = true>
 __device__ __forceinline__ void warp_store_k_row(const RowSink& c, size_t row, const int (&code)[D / 32], float s, int lane) {
   constexpr int E = D / 32;
   if constexpr (BITS != 3) {
@@ -141,7 +141,7 @@ __device__ __forceinline__ void warp_store_k_row(const RowSink& c, size_t row, c
     for (int o = 1; o < LPW; o <<= 1) w |= __shfl_xor_sync(FULL, w, o);
     uint32_t* row_words = reinterpret_cast<uint32_t*>(c.k_codes + row * (size_t)(BITS * D / 8));
     if (lane % LPW == 0) row_words[lane * E / EPW] = w;
-    if (lane == 0) store_scale(c.k_scales, row, s, c.scale_f16, c.status);
+    if (SCALE && lane == 0) store_scale(c.k_scales, row, s, c.scale_f16, c.status);
     return;
   }
   constexpr int LPU = 32 / E;  // lanes per 32-coordinate packing unit
@@ -170,7 +170,7 @@ __device__ __forceinline__ void warp_store_k_row(const RowSink& c, size_t row, c
   const int k = lane % LPU;
   uint32_t* row_words = reinterpret_cast<uint32_t*>(c.k_codes + row * (size_t)(3 * D / 8));
   if (k < 3) row_words[3 * (lane / LPU) + k] = (k == 0) ? w[0] : (k == 1 ? w[1] : w[2]);
-  if (lane == 0) store_scale(c.k_scales, row, s, c.scale_f16, c.status);
+  if (SCALE && lane == 0) store_scale(c.k_scales, row, s, c.scale_f16, c.status);
 }
 
 // V row t of its sequence (at `row` in the cache arrays) into the token-transposed records: row t is entry r = t % 32
