@@ -22,8 +22,8 @@
  *     before anything is launched; on an error nothing has been enqueued.
  *   - Device-side conditions that cannot be known on the host are reported through an optional
  *     `status_dev` array of 4 uint32 (zeroed by the caller): [0] bit mask of IQ_STATUS_* flags,
- *     [1] rows with codes re-decided in fp64 (see iq_quantize_append; a row may count once per 32 coordinates), [2] rows skipped because
- *     they fell outside the cache, [3] reserved. Nothing on the device traps or spins without a bound: the waits of the
+ *     [1] rows whose codes were re-decided in fp64 (see iq_quantize_append), [2] rows skipped because they fell outside the
+ *     cache, [3] reserved. Nothing on the device traps or spins without a bound: the waits of the
  *     decode, bulk append and reconstruction kernels on asynchronous copies and tensor-core results give up after 65536 polls
  *     of at most 20 us each (about a second at worst; a wait that works lasts microseconds). Decode and append then flag
  *     IQ_STATUS_WAIT_TIMEOUT and return with invalid results; iq_reconstruct_rows, which has no status array, writes NaN

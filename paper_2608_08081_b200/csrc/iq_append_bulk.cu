@@ -74,7 +74,7 @@ struct BulkLayout {
   static constexpr int OFF_M = OFF_SS + (NJ > 1 ? NG * 2048 : 0);       // [D][4] fp64 rows of the blocks M_b
   static constexpr int OFF_TILE = OFF_M + D * 32;                       // [NG][TILES] tile descriptors
   static constexpr int OFF_ROWS = OFF_TILE + NG * TILES * 48;           // [NG] rows to be decided again
-  static constexpr int OFF_WARP = OFF_ROWS + NG * 32;                   // [16] coordinates on the warps' lists
+  static constexpr int OFF_WARP = OFF_ROWS + NG * 64;                   // [16] coordinates on the warps' lists
   static constexpr int OFF_PRE = OFF_WARP + (PACK / 32) * 4;            // [THREADS + 1] int64 block counts before a slice of the batch
   static constexpr int OFF_WSUM = OFF_PRE + 8 * (THREADS + 2);
   static constexpr int OFF_TAU = OFF_WSUM + 8 * 32;                     // [2][16] BIG * threshold, K and V
@@ -93,8 +93,9 @@ struct BulkTile {       // a tile, as the control warp hands it to its group
   int pad[4];
 };
 static_assert(sizeof(BulkTile) == 48, "tile descriptor");
-struct BulkRows {       // rows of a tile that are decided again as a whole: of the group's present tile and of the one before, by its
-  uint32_t full[2][4];  // parity. Set by all warps at the end of a tile, read by all when the next one is copied in
+struct BulkRows {       // rows of the group's present tile and of the one before, by its parity; set by all warps at the end of a tile
+  uint32_t full[2][4];  // decided again as a whole: read by all warps when the next tile is copied in
+  uint32_t near[2][4];  // with a coordinate that is decided again: counted then
 };
 
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -438,7 +439,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   long long* wsum_s = reinterpret_cast<long long*>(smem + L::OFF_WSUM);
   float* tau_s = reinterpret_cast<float*>(smem + L::OFF_TAU);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_MISC);
-  int* zero_code_s = reinterpret_cast<int*>(smem + L::OFF_MISC + 8);    // [2] code of u = 0, K and V
+  int* zero_code_s = reinterpret_cast<int*>(smem + L::OFF_MISC + 8);    // [2] code of u = 0, K and V (+ 16: it is near a threshold)
 
   volatile int* started_s = reinterpret_cast<volatile int*>(smem + L::OFF_MISC + 16);  // [NG]
 
@@ -457,7 +458,10 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   }
   if (tid == L::PACK) {
     int zk = 0, zv = 0;
-    for (int j = 0; j < NT; j++) { zk += 0.f > p.thresholds_k[j] ? 1 : 0; zv += 0.f > p.thresholds_v[j] ? 1 : 0; }
+    for (int j = 0; j < NT; j++) {
+      zk = (zk + (0.f > p.thresholds_k[j] ? 1 : 0)) | (fabsf(p.thresholds_k[j]) <= GUARD_BAND ? 16 : 0);
+      zv = (zv + (0.f > p.thresholds_v[j] ? 1 : 0)) | (fabsf(p.thresholds_v[j]) <= GUARD_BAND ? 16 : 0);
+    }
     zero_code_s[0] = zk;
     zero_code_s[1] = zv;
     for (int g = 0; g < NG; g++) started_s[g] = 0;
@@ -503,7 +507,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   const long long total = 2 * nb * p.n_kv_heads;
   const long long lo = total * blockIdx.x / gridDim.x, hi = total * (blockIdx.x + 1) / gridDim.x;
   bool failed = false;      // a bounded wait gave up: the CTA leaves at the end of the head
-  uint32_t n_redone = 0;    // (lane 0 of a packing warp) rows on its list
+  uint32_t n_redone = 0;    // (the first four threads of a group) rows with coordinates decided again
   // phases, kept over the heads: tiles described, halves copied in (= MMA batches), tiles whose norms are done
   uint32_t n_tile = 0, n_half = 0, n_norm = 0;
   bool first = true;
@@ -659,7 +663,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         if (m != 0u) bulk_redo_rows<D, BITS>(p, m_s, t, m, warp & 3, part, lane);
         __syncwarp();
       };
-      if (gt < 8) reinterpret_cast<uint32_t*>(rows_s)[gt] = 0u;
+      if (gt < 16) reinterpret_cast<uint32_t*>(rows_s)[gt] = 0u;
 
       tile_build_m<D>(rot_head, m_s, tid);  // (while the control warps find the first tiles)
       BulkTile* t = describe();
@@ -698,9 +702,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           ss = ss_s[r] + ss_s[128 + r];
         }
         const bool is_v = kind != 0;
-        const int c_lo = t->c_lo, c_hi = t->c_hi;
-        const __half* const src0 = t->src;
-        const size_t row0 = t->row0;
+        const BulkTile* const cur = t;  // (read where it is needed: its slot is kept, registers are short)
         float binv = 0.f;
         if (NJ == 1 || part == 0 || !is_v) {
           float s = sqrtf((float)ss);
@@ -715,9 +717,9 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           binv = ordinary ? BIG * __frcp_rn(s) : 0.f;
           if (part == 0) {
             if (is_v) binv_s[r] = binv;
-            if (r >= c_lo && r < c_hi) {
+            if (r >= cur->c_lo && r < cur->c_hi) {
               if (!ordinary) t->special = 1;
-              store_scale(is_v ? p.v_scales : p.k_scales, row0 + r, s, p.scale_f16, p.status);
+              store_scale(is_v ? p.v_scales : p.k_scales, cur->row0 + r, s, p.scale_f16, p.status);
             }
           }
         }
@@ -727,7 +729,10 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         mbar_arrive(norm_bar);
         if (!failed) failed = !mbar_wait_bounded(norm_bar, n_norm & 1u, DEC_WAIT_LIMIT);
         n_norm++;
-        if (gt < 4) rows_s->full[n_tile & 1u][gt] = 0u;  // (everybody has read the marks of the tile before; the next tile sets its own there)
+        if (gt < 4) {  // everybody has read the marks of the tile before; the next tile sets its own there
+          n_redone += __popc(rows_s->near[n_tile & 1u][gt]);
+          rows_s->full[n_tile & 1u][gt] = rows_s->near[n_tile & 1u][gt] = 0u;
+        }
         if (!failed) failed = !mbar_wait_bounded(full_bar, (n_half - 1) & 1u, p.wait_polls);
         tc_fence_after();
         const bool special = t->special != 0;
@@ -737,9 +742,10 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
         if (kind >= 0) load_half(*t, 0);
 
         // ---- decisions and packing: 128 columns of this thread's lane, 32 at a time
-        uint32_t* const dst = reinterpret_cast<uint32_t*>(
-            is_v ? p.v_codes + ((row0 / 128) * D + gt) * (size_t)(16 * BITS)
-                 : p.k_codes + (row0 + r) * (size_t)(BITS * D / 8) + part * (16 * BITS));
+        auto run_of = [&]() {  // the record (V) or packed row (K) of this thread
+          return reinterpret_cast<uint32_t*>(is_v ? p.v_codes + ((cur->row0 / 128) * D + gt) * (size_t)(16 * BITS)
+                                                  : p.k_codes + (cur->row0 + r) * (size_t)(BITS * D / 8));
+        };
         uint32_t word[4 * BITS];
 #pragma unroll
         for (int i = 0; i < 4 * BITS; i++) word[i] = 0u;
@@ -752,10 +758,11 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
             // some coordinate of the warp lies in a band (or the tile has rows to be treated apart): the words in question
             // again, with the nearest codes, and the coordinates of new rows go on the list
             const uint32_t odd_words = (odd[0] ? 1u : 0u) | (odd[1] ? 2u : 0u) | (odd[2] ? 4u : 0u) | (odd[3] ? 8u : 0u);
+            const int c_lo = cur->c_lo, c_hi = cur->c_hi;
 #pragma unroll 1
             for (int q = 0; q < 4; q++) {
               if (!special && !__any_sync(FULL, (odd_words >> q) & 1u)) continue;
-              uint32_t x8[8], nw = 0u, low = 0u, near_m = 0u;  // the nearest codes, the codes below, which of them are undecided
+              uint32_t x8[8], nw = 0u, low = 0u, near_m = 0u;  // the nearest codes, the codes below, which of them are undecided (+ 8: of a zero row, at a threshold)
               tc_ld8(tmem_t + 32 * ch + 8 * q, x8);
 #pragma unroll
               for (int i = 0; i < 8; i++) {
@@ -766,7 +773,9 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
                 const bool odd_c = (cb & 0x0007FFFFu) != 0u;
                 if (b == 0.f) {  // a row of norm zero: u = 0; one whose norm is not finite: not a number, above no threshold
                   const float z = x * 0.f;
-                  code = z != z ? 0u : (uint32_t)zero_code_s[is_v ? 1 : 0];
+                  const uint32_t zc = (uint32_t)zero_code_s[is_v ? 1 : 0];
+                  code = z != z ? 0u : zc & 15u;
+                  if (z == z && zc >= 16u && row >= c_lo && row < c_hi) near_m |= 256u << i;  // (only counted)
                 } else if (odd_c && row >= c_lo && row < c_hi) {
                   near_m |= 1u << i;
                 }
@@ -775,12 +784,18 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
               }
 #pragma unroll
               for (int k = 0; k < 4; k++) nib[k] = (k == q) ? nw : nib[k];
-              const uint32_t rows = is_v ? __reduce_or_sync(FULL, near_m) : __ballot_sync(FULL, near_m != 0u);
-              if (lane == 0) n_redone += __popc(rows);
+              uint32_t rows;
+              if (is_v) {
+                rows = __reduce_or_sync(FULL, near_m);
+                rows = ((rows | rows >> 8) & 255u) << (8 * q);
+              } else {
+                rows = __ballot_sync(FULL, near_m != 0u);
+              }
+              if (lane == 0) atomicOr(&rows_s->near[n_tile & 1u][is_v ? ch : warp & 3], rows);
+              near_m &= 255u;
               const int n_list = *n_list_s, n_near = (int)__reduce_add_sync(FULL, (unsigned)__popc(near_m));
               if (n_near > L::LIST_STEP || n_list + n_near > L::LIST) {  // their rows again as a whole (the tile's number is n_tile - 2)
-                const uint32_t marked = is_v ? rows << (8 * q) : rows;
-                if (lane == 0) atomicOr(&rows_s->full[n_tile & 1u][is_v ? ch : warp & 3], marked);
+                if (lane == 0) atomicOr(&rows_s->full[n_tile & 1u][is_v ? ch : warp & 3], rows);
                 near_m = 0u;
               }
               __syncwarp();
@@ -789,8 +804,8 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
                 near_m &= near_m - 1u;
                 const int row = is_v ? col : r, coord = is_v ? gt : part * 128 + col;
                 const int k = atomicAdd(n_list_s, 1);
-                src_s[k] = src0 + (long long)row * p.stride_t;
-                dst_s[k] = is_v ? dst : dst - part * (4 * BITS);
+                src_s[k] = cur->src + (long long)row * p.stride_t;
+                dst_s[k] = run_of();
                 info_s[k] = (uint32_t)coord | ((uint32_t)(is_v ? row : coord) << 8) | (((low >> (4 * i)) & 15u) << 16) | (is_v ? 1u << 20 : 0u);
               }
               __syncwarp();
@@ -800,6 +815,8 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
           for (int i = 0; i < 3 * BITS; i++) word[i] = word[i + BITS];
           pack_nibbles<BITS>(nib, word + 3 * BITS);
         }
+        const int c_lo = cur->c_lo, c_hi = cur->c_hi;
+        uint32_t* const dst = run_of() + (is_v ? 0 : part * (4 * BITS));
         if (is_v ? (c_lo == 0 && c_hi == 128) : (r >= c_lo && r < c_hi)) {
 #pragma unroll
           for (int i = 0; i < BITS; i++)
@@ -835,6 +852,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
       }
       cta_bar_sync_n(2 + grp, GT);  // the marks of the group's last tile, and the stores to it, are in place
       if (!__any_sync(FULL, failed)) redo_marked(n_tile - 2u);
+      if (gt < 4) n_redone += __popc(rows_s->near[n_tile & 1u][gt]);
     }
     item = head0 + seg_hi;
     if (__syncthreads_or(failed)) { failed = true; break; }  // (W is rebuilt for the next head)

@@ -180,3 +180,39 @@ def test_rows_that_are_not_finite(iq, torch, bits, d, grid):  # noqa: F811
             codes = np.array(codes)
             assert np.array_equal(codes[0][good], codes[2][good]) and np.array_equal(codes[0], codes[1])
             assert (codes[0][list(bad)] == 0).all()
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_each_row_that_is_decided_again_counts_once(iq, torch, bits, d):  # noqa: F811
+    """status[1] of a prompt: the rows with a coordinate at a threshold (here: constant rows, 0 everywhere but in one block,
+    and zero rows), one each per KV head and tensor, as calls of four rows count them. Other rows have no coordinate within
+    2e-4 of a threshold, more than any band."""
+    B, H, T = 2, 2, 700
+    lv, th, _, _ = two_codebooks(d, bits, "int8", False)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)))
+    shape = iq.Shape(B, H, H, d, 768, bits=bits)
+    rng = np.random.default_rng(d + bits)
+    q8 = rng.standard_normal((H, d // 4, 8)).astype(np.float32)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 0, q8, rot)
+    W = [oracle.rotation_matrix(d, q) * np.sqrt(d) for q in q8]
+    x = rng.standard_normal((2, B, T, H, d)).astype(np.float16)
+    near = np.zeros((2, B, T, H), bool)
+    for h in range(H):
+        for _ in range(400):   # rows with a coordinate near a threshold are drawn again
+            u = x[:, :, :, h].astype(np.float64) @ W[h].T / np.linalg.norm(x[:, :, :, h].astype(np.float64), axis=-1, keepdims=True)
+            bad = np.zeros(u.shape[:-1], bool)
+            for t in th:
+                bad |= (np.abs(u - float(t)) < 2e-4).any(axis=-1)
+            if not bad.any():
+                break
+            x[:, :, :, h][bad] = rng.standard_normal((int(bad.sum()), d)).astype(np.float16)
+        assert not bad.any()
+    x[:, :, 3::50] = 1
+    x[:, :, 7::90] = 0
+    near[:, :, 3::50] = near[:, :, 7::90] = True
+    k, v = (torch.from_numpy(a).cuda() for a in x)
+    _, whole = _append(iq, torch, shape, rot, cb, k, v, [0, 30], [T, T], T, 0, torch.float32)
+    _, rows = _append(iq, torch, shape, rot, cb, k, v, [0, 30], [T, T], 4, 0, torch.float32)
+    assert whole[0] == rows[0] == 0 and whole[1] == rows[1] == int(near.sum())
