@@ -6,24 +6,30 @@
 // two operands are chosen so that a thread reads from its tensor-memory lane what it has to pack next to each other:
 //   K: D[row][coordinate]  = X W^T   thread = row,        the words of its packed row
 //   V: D[coordinate][row]  = W X^T   thread = coordinate, the words of its token-transposed record
-// W is split into two binary16 terms, W_hi + W_lo (|W - W_hi - W_lo| <= 2^-22 |W|), the products with binary16 rows are
-// exact and summed in fp32, the small terms first. W has only 4 distinct magnitudes per row (M_b times a 4-point
+// W is split into two binary16 terms, W_hi + W_lo (|W - W_hi - W_lo| <= 2^-22 |W|, or 2^-25 where W_lo is subnormal), the
+// products with binary16 rows are exact and summed in fp32, the small terms first. W has only 4 distinct magnitudes per row (M_b times a 4-point
 // transform; the rest of H_d is signs), so a CTA builds it in about a microsecond per head. d = 256: H_256 is
 // [[H, H], [H, -H]], so the operand of the second half of the contraction is that of the first, negated where both
 // halves are the upper ones by the instruction's negate bit: 2 x 64 KB of W instead of 256.
 //
-// Decision. Per threshold one fused multiply-add with saturation, sat(B x + o_j), B = BIG / s: 0 below, 1 above, and a
+// Decision. Per threshold one fused multiply-add with saturation, sat(B x + o_j), B = 0.5 / (GUARD s): 0 below, 1 above, and a
 // fraction inside a band of +-GUARD around the threshold. The code is the sum; a sum that is not a whole number (16 + code
 // is kept, so its fraction bits are the same for all codes; they are OR-ed over 8 coordinates) marks a coordinate too
 // close to call, which is put on a list and decided again in fp64 by eight lanes (exact +-1 sums, the norm and the block
 // in fp64). Where 8 columns of a warp have many, or the list is full (rows with ties throughout: constant rows, rows whose
 // Walsh-Hadamard coordinates vanish), the rows are marked instead; the group's warps share the marked rows of a tile when
 // the next one has been copied in, a row at a time by a warp. 4 x 8 K constant rows, d = 128, 3 bits: 0.77 ms, every 13th row
-// constant 0.28 (ordinary rows 0.081); with every warp of a V tile deciding all rows, code by code: 8.8 and 0.9. So the codes are those of an fp64 evaluation. GUARD covers the error of the fp32 sums near a threshold: W
-// (2^-22 sqrt(d)) and one cut of the running sum per instruction -- a sum that ends near a threshold stays below
-// sqrt(d) / 2 + 2.8 on the way (Cauchy-Schwarz on the two parts), so 8 cuts of 2^-21 at d = 128, 16 of 2^-20 at d = 256:
-// 6.5e-6 and 1.9e-5. Measured over 16 M coordinates each of Gaussian, outlier, heavy-tailed and cancelling rows: no code
-// differs with a band of 2^-20 at d = 128, of 2^-16 at d = 256; the bands are 2^-16 and 2^-15.
+// constant 0.28 (ordinary rows 0.081); with every warp of a V tile deciding all rows, code by code: 8.8 and 0.9.
+//
+// GUARD bounds the error of a sum that ends near a threshold t, so the codes are those of an fp64 evaluation. An instruction
+// (16 products) aligns its products and the running sum to the largest of them, keeps two bits below the fp32 last
+// place, and cuts; the result is cut to fp32 (an emulation of just this gives the same bits as the tensor core on sums of
+// all kinds). So it loses at most 17 x 2^-25 of the larger of the running sum and its products, and 2^-23 of its result. The
+// running sums S_i of a row of norm 1 that end at t are bounded together, by Cauchy-Schwarz on sum c_i S_i: at d = 128 the
+// cuts are at most 1.9e-5 + 2.3e-6 t, with W's 2^-22 sqrt(d) and the rounding of x B 2.25e-5 + 2.3e-6 t. At d = 256 the second
+// half's lower terms would each cut the sum of the first half; they come last, where it is back at t: 5.5e-5 + 9.8e-6 t
+// (9.1e-5 + 7e-6 t in the other order). Rows built against it (an emulated search over prefixes along W's row, with the low bits of
+// every element chosen for the largest cut) reach 7e-6 and 1.9e-5, Gaussian and outlier rows 1e-6.
 // Symmetric codebooks (t_mid = 0, t_j = -t_-j): the positive thresholds against |x| plus the sign, 4 instead of 7
 // multiply-adds per coordinate at 3 bits, 8 instead of 15 at 4 bits.
 //
@@ -45,12 +51,8 @@
 
 namespace iq {
 
-// Half-width of the band around a threshold in which the tile decision is not trusted (see above).
-template <int D>
-struct BulkGuard {
-  static constexpr float GUARD = D == 128 ? 1.52587890625e-05f : 3.0517578125e-05f;  // 2^-16, 2^-15
-  static constexpr float BIG = 0.5f / GUARD;
-};
+// Half-width of the band around a threshold in which the tile decision is not trusted (see above); t: the largest threshold.
+static float bulk_guard(int head_dim, float t) { return head_dim == 128 ? 2.25e-5f + 2.3e-6f * t : 5.5e-5f + 9.8e-6f * t; }
 
 template <int D>
 struct BulkLayout {
@@ -69,7 +71,7 @@ struct BulkLayout {
   static constexpr int OFF_X = W_BYTES;
   static constexpr int OFF_LIST = OFF_X + NG * OPERAND;
   static constexpr int LIST_BYTES = 20 * LIST;    // source rows (8), destinations (8), (side, code, coordinate, entry) (4)
-  static constexpr int OFF_BINV = OFF_LIST + (PACK / 32) * LIST_BYTES;  // [NG][128] BIG / s of the rows of a group's tile
+  static constexpr int OFF_BINV = OFF_LIST + (PACK / 32) * LIST_BYTES;  // [NG][128] 0.5 / (GUARD s) of the rows of a group's tile
   static constexpr int OFF_SS = OFF_BINV + NG * 512;                    // [NG][2][128] fp64 partial square sums (d = 256)
   static constexpr int OFF_M = OFF_SS + (NJ > 1 ? NG * 2048 : 0);       // [D][4] fp64 rows of the blocks M_b
   static constexpr int OFF_TILE = OFF_M + D * 32;                       // [NG][TILES] tile descriptors
@@ -77,7 +79,7 @@ struct BulkLayout {
   static constexpr int OFF_WARP = OFF_ROWS + NG * 64;                   // [16] coordinates on the warps' lists
   static constexpr int OFF_PRE = OFF_WARP + (PACK / 32) * 4;            // [THREADS + 1] int64 block counts before a slice of the batch
   static constexpr int OFF_WSUM = OFF_PRE + 8 * (THREADS + 2);
-  static constexpr int OFF_TAU = OFF_WSUM + 8 * 32;                     // [2][16] BIG * threshold, K and V
+  static constexpr int OFF_TAU = OFF_WSUM + 8 * 32;                     // [2][16] 0.5 / GUARD * threshold, K and V
   static constexpr int OFF_BAR = OFF_TAU + 128;                         // [NG][5] mbarriers: tile described, copied in, norms, accumulator, drained
   static constexpr int OFF_MISC = OFF_BAR + 8 * (5 * NG + (NG & 1));
   static constexpr int SMEM = OFF_MISC + 32 + 1024;                     // + alignment of the swizzle atoms
@@ -370,7 +372,7 @@ struct BulkWalk {
 };
 
 // 16 + code of one coordinate as a float, with a fraction where it lies in the band of a threshold. x: the coordinate of
-// W x, b = BIG / s, off[j] = 0.5 - BIG t_j.
+// W x, b = big / s, off[j] = 0.5 - big t_j, big = 0.5 / GUARD.
 template <int BITS, bool SYM, int NS>
 __device__ __forceinline__ float bulk_decide(float x, float b, const float (&off)[NS]) {
   if constexpr (SYM) {
@@ -420,7 +422,6 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   constexpr int NJ = L::NJ, NG = L::NG, GT = L::GT;
   constexpr int NT = (1 << BITS) - 1;                   // thresholds
   constexpr int NS = SYM ? (1 << (BITS - 1)) - 1 : NT;  // those compared one by one (besides zero)
-  constexpr float BIG = BulkGuard<D>::BIG;
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -466,7 +467,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
     zero_code_s[1] = zv;
     for (int g = 0; g < NG; g++) started_s[g] = 0;
   }
-  if (tid < 32) tau_s[tid] = (tid & 15) < NT ? BIG * (tid < 16 ? p.thresholds_k[tid & 15] : p.thresholds_v[tid & 15]) : 0.f;
+  if (tid < 32) tau_s[tid] = (tid & 15) < NT ? p.big * (tid < 16 ? p.thresholds_k[tid & 15] : p.thresholds_v[tid & 15]) : 0.f;
   if (tid < L::PACK / 32) reinterpret_cast<int*>(smem + L::OFF_WARP)[tid] = 0;
   grid_dependency_wait();
 
@@ -580,8 +581,8 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
 #pragma unroll
             for (int j = 0; j < NJ; j++)
 #pragma unroll
-              for (int hl = 0; hl < 2; hl++) {  // W_lo, then W_hi
-                const uint64_t wd = smem_desc_k128(smem_u32(smem + (2 * j + hl) * L::OPERAND));
+              for (int hl = 0; hl < 2; hl++) {  // W_lo, then W_hi; the second half the other way round
+                const uint64_t wd = smem_desc_k128(smem_u32(smem + (2 * j + (hf ? 1 - hl : hl)) * L::OPERAND));
                 const uint64_t a0 = is_v ? wd : xd, b0 = is_v ? xd : wd;
 #pragma unroll
                 for (int k = 0; k < 8; k++) {  // 16 contraction steps each: 32 bytes inside a 128-byte row, 4 per slab
@@ -714,7 +715,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
             else if (s > 0.f && ss < md * md) s = dn;
           }
           const bool ordinary = s > 0.f && s < INFINITY;
-          binv = ordinary ? BIG * __frcp_rn(s) : 0.f;
+          binv = ordinary ? p.big * __frcp_rn(s) : 0.f;
           if (part == 0) {
             if (is_v) binv_s[r] = binv;
             if (r >= cur->c_lo && r < cur->c_hi) {
@@ -912,10 +913,18 @@ static cudaError_t launch_bulk_bits(const QuantizeParams& p, bool sym, int batch
   return sym ? launch_bulk<D, 4, true>(p, batch, stream) : launch_bulk<D, 4, false>(p, batch, stream);
 }
 
+// The largest threshold that a row can come near: |u| <= sqrt(d).
+static float largest_threshold(const QuantizeParams& p, int head_dim) {
+  float m = 0.f;
+  for (const float* t : {p.thresholds_k, p.thresholds_v})
+    for (int j = 0; j < (1 << p.bits) - 1; j++) m = fmaxf(m, fabsf(t[j]));
+  return fminf(m, sqrtf((float)head_dim));
+}
+
 // The codebooks whose thresholds the saturating sums can tell apart: neighbours further apart than the bands around
-// them, and small enough for BIG * t to keep fractions. Lloyd-Max thresholds are 0.1 and more apart.
+// them, and small enough for big * t to keep fractions. Lloyd-Max thresholds are 0.1 and more apart.
 bool append_bulk_takes(const QuantizeParams& p, int head_dim) {
-  const float guard = head_dim == 128 ? BulkGuard<128>::GUARD : BulkGuard<256>::GUARD;
+  const float guard = bulk_guard(head_dim, largest_threshold(p, head_dim));
   const int nt = (1 << p.bits) - 1;
   for (const float* t : {p.thresholds_k, p.thresholds_v})
     for (int j = 0; j < nt; j++) {
@@ -925,7 +934,9 @@ bool append_bulk_takes(const QuantizeParams& p, int head_dim) {
   return true;
 }
 
-cudaError_t launch_append_bulk(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream) {
+cudaError_t launch_append_bulk(const QuantizeParams& params, int head_dim, int batch, cudaStream_t stream) {
+  QuantizeParams p = params;
+  p.big = 0.5f / bulk_guard(head_dim, largest_threshold(p, head_dim));
   const int nt = (1 << p.bits) - 1, mid = nt / 2;
   bool sym = true;
   for (const float* t : {p.thresholds_k, p.thresholds_v}) {

@@ -42,6 +42,7 @@ struct QuantizeParams {
   int n_kv_heads, t_cap;
   PageMap pm;
   int scale_f16;
+  float big;                // bulk: 0.5 over the band around a threshold (set by the launcher)
   uint32_t wait_polls;      // bulk: limit of the waits for tensor-core results: DEC_WAIT_LIMIT, or what the self-test asks for
 };
 cudaError_t launch_quantize_append(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream);

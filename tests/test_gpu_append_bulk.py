@@ -216,3 +216,44 @@ def test_each_row_that_is_decided_again_counts_once(iq, torch, bits, d):  # noqa
     _, whole = _append(iq, torch, shape, rot, cb, k, v, [0, 30], [T, T], T, 0, torch.float32)
     _, rows = _append(iq, torch, shape, rot, cb, k, v, [0, 30], [T, T], 4, 0, torch.float32)
     assert whole[0] == rows[0] == 0 and whole[1] == rows[1] == int(near.sum())
+
+
+@pytest.mark.parametrize("d,bits", [(128, 2), (128, 3), (128, 4), (256, 2), (256, 3), (256, 4)])
+def test_rows_built_against_the_band(iq, torch, d, bits):  # noqa: F811
+    """Rows along a row of W up to some element and against it from there, so that the running sum is as large as it can be
+    and comes back to a threshold: the nearest of 3000 variants on either side of it, and some a few 1e-6 to 1e-4 away. Every
+    code of every row is that of an fp64 evaluation."""
+    lv, th, _, _ = two_codebooks(d, bits, "int8", False)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)))
+    rng = np.random.default_rng(d + bits)
+    q8 = rng.standard_normal((1, d // 4, 8)).astype(np.float32)
+    W = oracle.rotation_matrix(d, q8[0]) * np.sqrt(d)
+    rows = []
+    for case in range(80):
+        w, t = W[rng.integers(d)], float(th[case % len(th)])
+        m = int(d * rng.uniform(0.3, 0.95))
+        A, Bq, Cq = m + m * m / (d - m), -2 * t * m / (d - m), t * t / (d - m) - 1   # |x| = 1, <w, x> = t
+        a = (-Bq + np.sqrt(Bq * Bq - 4 * A * Cq)) / (2 * A)
+        x = w * np.where(np.arange(d) < m, a, (t - a * m) / (d - m)) * rng.uniform(8, 64)
+        x = (x * (1 + 0.003 * rng.standard_normal((3000, d)))).astype(np.float16)
+        dist = x.astype(np.float64) @ w / np.linalg.norm(x.astype(np.float64), axis=1) - t
+        for side in (1, -1):
+            order = np.argsort(np.where(side * dist > 1e-9, np.abs(dist), np.inf))
+            rows += [x[i] for i in order[:3]]
+            for far in (3e-6, 1e-5, 3e-5, 1e-4):
+                rows.append(x[np.argmin(np.abs(side * dist - far))])
+    x = np.array(rows)
+    T = len(x)
+    shape = iq.Shape(1, 1, 1, d, (T + 127) // 128 * 128, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, 1), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, 1, 0, q8, rot)
+    W = oracle.rotation_matrix(d, rot.cpu().numpy()) * np.sqrt(d)
+    k = torch.from_numpy(x).cuda().reshape(1, T, 1, d)
+    cache, _ = _append(iq, torch, shape, rot, cb, k, k, [0], [T], T, 0, torch.float32)
+    x = x.astype(np.float64)
+    u = x @ W.T / np.linalg.norm(x, axis=1, keepdims=True)
+    gap = u[..., None] - th.astype(np.float64)
+    want, tie = (gap > 0).sum(axis=-1), (np.abs(gap) < 1e-12).any(axis=-1)
+    g = cache_to_numpy(cache)
+    for got in ([oracle.unpack_row(d, g["k_codes"][0, 0, r], bits) for r in range(T)], [oracle.v_row_codes(d, g["v_codes"][0, 0], r, bits) for r in range(T)]):
+        assert np.all((np.array(got) == want) | tie), int(((np.array(got) != want) & ~tie).sum())
