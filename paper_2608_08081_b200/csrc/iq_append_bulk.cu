@@ -146,7 +146,7 @@ __device__ __forceinline__ void patch_code(uint32_t* run, int e, int code) {
 }
 
 // The listed coordinates in fp64, eight lanes each: z = the four outputs of the coordinate's block of H x (exact sums),
-// u = its row of M_b times z, over the exact norm, against the one threshold it lies close to.
+// u = its row of M_b times z, over the exact norm, against the thresholds from the first that it may be above.
 template <int D, int BITS>
 static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const double* m_s, const __half* const* src_s,
                                               uint32_t* const* dst_s, const uint32_t* info_s, int n, int lane) {
@@ -191,8 +191,10 @@ static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const dou
     }
     const double* m = m_s + 4 * coord;
     const double u = (m[0] * z[0] + m[1] * z[1] + m[2] * z[2] + m[3] * z[3]) * inv_sqrt(ss);  // (rows of norm zero are not listed)
-    const float th = ((info >> 20) & 1u) ? p.thresholds_v[lower] : p.thresholds_k[lower];
-    if (act && li == 0) patch_code<BITS>(dst_s[ee], entry, lower + (u > (double)th ? 1 : 0));
+    const float* th = ((info >> 20) & 1u) ? p.thresholds_v : p.thresholds_k;
+    int code = lower;
+    while (code < (1 << BITS) - 1 && u > (double)th[code]) code++;
+    if (act && li == 0) patch_code<BITS>(dst_s[ee], entry, code);
   }
 }
 
@@ -371,11 +373,25 @@ struct BulkWalk {
   int pos0, n_new;
 };
 
+// How a coordinate is decided. CLOSE: thresholds may lie within one another's bands, where two fractions can add up to a
+// whole number, so the thresholds below and above the band are counted; twice the instructions (4 x 32 K rows, d = 128,
+// thresholds 1e-5 apart: 894 us where a warp per row takes 1790).
+enum BulkMode { BULK_PLAIN, BULK_SYMMETRIC, BULK_CLOSE };
+
 // 16 + code of one coordinate as a float, with a fraction where it lies in the band of a threshold. x: the coordinate of
 // W x, b = big / s, off[j] = 0.5 - big t_j, big = 0.5 / GUARD.
-template <int BITS, bool SYM, int NS>
+template <int BITS, int MODE, int NS>
 __device__ __forceinline__ float bulk_decide(float x, float b, const float (&off)[NS]) {
-  if constexpr (SYM) {
+  if constexpr (MODE == BULK_CLOSE) {
+    float lo = 16.0f, hi = 16.0f;
+#pragma unroll
+    for (int j = 0; j < NS; j++) {
+      const float v = fmaf(x, b, off[j]);
+      lo += v >= 1.0f ? 1.0f : 0.0f;
+      hi += v > 0.0f ? 1.0f : 0.0f;
+    }
+    return hi > lo ? lo + 0.5f : lo;
+  } else if constexpr (MODE == BULK_SYMMETRIC) {
     float m = __saturatef(fmaf(fabsf(x), b, off[0]));
 #pragma unroll
     for (int j = 1; j < NS; j++) m += __saturatef(fmaf(fabsf(x), b, off[j]));
@@ -390,7 +406,7 @@ __device__ __forceinline__ float bulk_decide(float x, float b, const float (&off
 
 // 32 columns of a lane: the nibble words of their codes, and per word the fraction bits of its sums OR-ed together.
 // ROWS: a column is a row (V tiles), its b in shared memory; otherwise the lane is one, b0.
-template <int BITS, bool SYM, bool ROWS, int NS>
+template <int BITS, int MODE, bool ROWS, int NS>
 __device__ __forceinline__ void bulk_pack32(uint32_t taddr, const float* b_s, float b0, const float (&off)[NS], uint32_t (&nib)[4], uint32_t (&odd)[4]) {
   constexpr float MAGIC = 8388608.0f - 16.0f * 4369.0f;  // 2^23 - the 16 of four sums, one per nibble
   uint32_t xr[32];
@@ -405,8 +421,8 @@ __device__ __forceinline__ void bulk_pack32(uint32_t taddr, const float* b_s, fl
       if constexpr (ROWS) b4 = *reinterpret_cast<const float4*>(b_s + 8 * q + 4 * hq);
       else b4 = make_float4(b0, b0, b0, b0);
       const uint32_t* x = xr + 8 * q + 4 * hq;
-      const float c0 = bulk_decide<BITS, SYM, NS>(__uint_as_float(x[0]), b4.x, off), c1 = bulk_decide<BITS, SYM, NS>(__uint_as_float(x[1]), b4.y, off);
-      const float c2 = bulk_decide<BITS, SYM, NS>(__uint_as_float(x[2]), b4.z, off), c3 = bulk_decide<BITS, SYM, NS>(__uint_as_float(x[3]), b4.w, off);
+      const float c0 = bulk_decide<BITS, MODE, NS>(__uint_as_float(x[0]), b4.x, off), c1 = bulk_decide<BITS, MODE, NS>(__uint_as_float(x[1]), b4.y, off);
+      const float c2 = bulk_decide<BITS, MODE, NS>(__uint_as_float(x[2]), b4.z, off), c3 = bulk_decide<BITS, MODE, NS>(__uint_as_float(x[3]), b4.w, off);
       tt[hq] = fmaf(c3, 4096.f, fmaf(c2, 256.f, fmaf(c1, 16.f, c0 + MAGIC)));
       acc = (acc | __float_as_uint(c0) | __float_as_uint(c1));
       acc = (acc | __float_as_uint(c2) | __float_as_uint(c3));
@@ -416,11 +432,12 @@ __device__ __forceinline__ void bulk_pack32(uint32_t taddr, const float* b_s, fl
   }
 }
 
-template <int D, int BITS, bool SYM>
+template <int D, int BITS, int MODE>
 __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(const __grid_constant__ QuantizeParams p, const __grid_constant__ int batch) {
   using L = BulkLayout<D>;
   constexpr int NJ = L::NJ, NG = L::NG, GT = L::GT;
   constexpr int NT = (1 << BITS) - 1;                   // thresholds
+  constexpr bool SYM = MODE == BULK_SYMMETRIC;
   constexpr int NS = SYM ? (1 << (BITS - 1)) - 1 : NT;  // those compared one by one (besides zero)
 
   extern __shared__ uint8_t smem_raw[];
@@ -753,8 +770,8 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
 #pragma unroll 1
         for (int ch = 0; ch < 4; ch++) {
           uint32_t nib[4], odd[4];
-          if (is_v) bulk_pack32<BITS, SYM, true, NS>(tmem_t + 32 * ch, binv_s + 32 * ch, 0.f, off, nib, odd);
-          else bulk_pack32<BITS, SYM, false, NS>(tmem_t + 32 * ch, nullptr, binv, off, nib, odd);
+          if (is_v) bulk_pack32<BITS, MODE, true, NS>(tmem_t + 32 * ch, binv_s + 32 * ch, 0.f, off, nib, odd);
+          else bulk_pack32<BITS, MODE, false, NS>(tmem_t + 32 * ch, nullptr, binv, off, nib, odd);
           if (__any_sync(FULL, special || ((odd[0] | odd[1]) | (odd[2] | odd[3])) != 0u)) {
             // some coordinate of the warp lies in a band (or the tile has rows to be treated apart): the words in question
             // again, with the nearest codes, and the coordinates of new rows go on the list
@@ -769,7 +786,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
               for (int i = 0; i < 8; i++) {
                 const int col = 32 * ch + 8 * q + i, row = is_v ? col : r;
                 const float x = __uint_as_float(x8[i]), b = is_v ? binv_s[col] : binv;
-                const uint32_t cb = __float_as_uint(bulk_decide<BITS, SYM, NS>(x, b, off));
+                const uint32_t cb = __float_as_uint(bulk_decide<BITS, MODE, NS>(x, b, off));
                 uint32_t code = ((cb + 0x0003FFFFu) >> 19) & 15u;
                 const bool odd_c = (cb & 0x0007FFFFu) != 0u;
                 if (b == 0.f) {  // a row of norm zero: u = 0; one whose norm is not finite: not a number, above no threshold
@@ -873,7 +890,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
 }
 
-template <int D, int BITS, bool SYM>
+template <int D, int BITS, int MODE>
 static cudaError_t launch_bulk(const QuantizeParams& p, int batch, cudaStream_t stream) {
   using L = BulkLayout<D>;
   static bool configured[64] = {};
@@ -882,7 +899,7 @@ static cudaError_t launch_bulk(const QuantizeParams& p, int batch, cudaStream_t 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  auto kern = append_bulk_kernel<D, BITS, SYM>;
+  auto kern = append_bulk_kernel<D, BITS, MODE>;
   if (!configured[dev]) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM);
     if (e != cudaSuccess) return e;
@@ -907,10 +924,11 @@ static cudaError_t launch_bulk(const QuantizeParams& p, int batch, cudaStream_t 
 }
 
 template <int D>
-static cudaError_t launch_bulk_bits(const QuantizeParams& p, bool sym, int batch, cudaStream_t stream) {
-  if (p.bits == 2) return launch_bulk<D, 2, false>(p, batch, stream);
-  if (p.bits == 3) return sym ? launch_bulk<D, 3, true>(p, batch, stream) : launch_bulk<D, 3, false>(p, batch, stream);
-  return sym ? launch_bulk<D, 4, true>(p, batch, stream) : launch_bulk<D, 4, false>(p, batch, stream);
+static cudaError_t launch_bulk_bits(const QuantizeParams& p, BulkMode mode, int batch, cudaStream_t stream) {
+  if (p.bits == 2) return launch_bulk<D, 2, BULK_PLAIN>(p, batch, stream);
+  if (p.bits == 4) return mode == BULK_SYMMETRIC ? launch_bulk<D, 4, BULK_SYMMETRIC>(p, batch, stream) : launch_bulk<D, 4, BULK_PLAIN>(p, batch, stream);
+  if (mode == BULK_CLOSE) return launch_bulk<D, 3, BULK_CLOSE>(p, batch, stream);
+  return mode == BULK_SYMMETRIC ? launch_bulk<D, 3, BULK_SYMMETRIC>(p, batch, stream) : launch_bulk<D, 3, BULK_PLAIN>(p, batch, stream);
 }
 
 // The largest threshold that a row can come near: |u| <= sqrt(d).
@@ -921,29 +939,34 @@ static float largest_threshold(const QuantizeParams& p, int head_dim) {
   return fminf(m, sqrtf((float)head_dim));
 }
 
-// The codebooks whose thresholds the saturating sums can tell apart: neighbours further apart than the bands around
-// them, and small enough for big * t to keep fractions. Lloyd-Max thresholds are 0.1 and more apart.
-bool append_bulk_takes(const QuantizeParams& p, int head_dim) {
+// No coordinate reaches this (|u| <= 16): thresholds beyond it are held here, where big * t keeps fractions.
+constexpr float BULK_REACH = 32.f;
+
+// Neighbouring thresholds that the saturating sums cannot tell apart (Lloyd-Max thresholds are 0.1 and more apart).
+static bool close_thresholds(const QuantizeParams& p, int head_dim) {
   const float guard = bulk_guard(head_dim, largest_threshold(p, head_dim));
-  const int nt = (1 << p.bits) - 1;
   for (const float* t : {p.thresholds_k, p.thresholds_v})
-    for (int j = 0; j < nt; j++) {
-      if (!(fabsf(t[j]) < 64.f)) return false;
-      if (j > 0 && !(t[j] - t[j - 1] > 8.f * guard)) return false;
-    }
-  return true;
+    for (int j = 1; j < (1 << p.bits) - 1; j++)
+      if (t[j] > -BULK_REACH && t[j - 1] < BULK_REACH && !(t[j] - t[j - 1] > 8.f * guard)) return true;
+  return false;
 }
+
+// 2 and 4 bits: close thresholds stay with a warp per row, which is all that these widths had.
+bool append_bulk_takes(const QuantizeParams& p, int head_dim) { return p.bits == 3 || !close_thresholds(p, head_dim); }
 
 cudaError_t launch_append_bulk(const QuantizeParams& params, int head_dim, int batch, cudaStream_t stream) {
   QuantizeParams p = params;
   p.big = 0.5f / bulk_guard(head_dim, largest_threshold(p, head_dim));
   const int nt = (1 << p.bits) - 1, mid = nt / 2;
-  bool sym = true;
-  for (const float* t : {p.thresholds_k, p.thresholds_v}) {
-    sym &= t[mid] == 0.f;
-    for (int j = 1; j <= mid; j++) sym &= t[mid - j] == -t[mid + j];
+  BulkMode mode = close_thresholds(p, head_dim) ? BULK_CLOSE : BULK_SYMMETRIC;
+  for (float* t : {p.thresholds_k, p.thresholds_v}) {
+    if (mode == BULK_SYMMETRIC && t[mid] != 0.f) mode = BULK_PLAIN;
+    for (int j = 1; j <= mid; j++)
+      if (mode == BULK_SYMMETRIC && t[mid - j] != -t[mid + j]) mode = BULK_PLAIN;
   }
-  return head_dim == 128 ? launch_bulk_bits<128>(p, sym, batch, stream) : launch_bulk_bits<256>(p, sym, batch, stream);
+  for (float* t : {p.thresholds_k, p.thresholds_v})
+    for (int j = 0; j < nt; j++) t[j] = fminf(fmaxf(t[j], -BULK_REACH), BULK_REACH);
+  return head_dim == 128 ? launch_bulk_bits<128>(p, mode, batch, stream) : launch_bulk_bits<256>(p, mode, batch, stream);
 }
 
 }  // namespace iq

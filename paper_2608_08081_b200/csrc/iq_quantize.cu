@@ -320,7 +320,7 @@ static cudaError_t launch_few(const QuantizeParams& p, int batch, cudaStream_t s
 cudaError_t launch_quantize_append(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream) {
   if (p.n_new_max <= 0 || batch <= 0) return cudaSuccess;
   // Up to 4 rows per sequence: a warp per row (5 us for one row; the bulk kernel's set-up alone takes as long). More: the
-  // bulk kernel, unless two thresholds of the codebook are too close together for its decision.
+  // bulk kernel, unless two thresholds of a 2- or 4-bit codebook are too close together for its decision.
   if (p.n_new_max > QA_FEW_ROWS && append_bulk_takes(p, head_dim)) return launch_append_bulk(p, head_dim, batch, stream);
   if (p.bits == 2) return head_dim == 128 ? launch_few<128, 2>(p, batch, stream) : launch_few<256, 2>(p, batch, stream);
   if (p.bits == 4) return head_dim == 128 ? launch_few<128, 4>(p, batch, stream) : launch_few<256, 4>(p, batch, stream);

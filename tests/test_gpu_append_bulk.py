@@ -257,3 +257,32 @@ def test_rows_built_against_the_band(iq, torch, d, bits):  # noqa: F811
     g = cache_to_numpy(cache)
     for got in ([oracle.unpack_row(d, g["k_codes"][0, 0, r], bits) for r in range(T)], [oracle.v_row_codes(d, g["v_codes"][0, 0], r, bits) for r in range(T)]):
         assert np.all((np.array(got) == want) | tie), int(((np.array(got) != want) & ~tie).sum())
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("form", ["a pair", "seven in a band", "across two bands", "out of reach"])
+def test_three_bit_codebooks_with_close_or_far_thresholds(iq, torch, d, form):  # noqa: F811
+    """Thresholds within one another's bands (2e-6 to 1e-4 apart, some of them around 0, where constant rows tie) and
+    thresholds that no coordinate reaches: the bytes of calls of four rows."""
+    B, H, T = 3, 2, 900
+    lv, th, _, _ = two_codebooks(d, 3, "int8", False)
+    th = th.astype(np.float64)
+    if form == "a pair":
+        th[4] = th[3] + 1e-5
+    elif form == "seven in a band":
+        th = 0.4 + 2e-6 * np.arange(7)
+    elif form == "across two bands":
+        th = np.array([-1.0, -2e-5, -1e-5, 0.0, 4e-5, 8e-5, 0.7])
+    else:
+        th = np.array([-1e30, -100.0, -1.0, 0.0, 1.0, 1e5, 3e38])
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th.astype(np.float32))))
+    shape = iq.Shape(B, H, H, d, 1024)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 1, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    k[:, 3::17], v[:, 5::29] = 1, 1
+    a, sa = _append(iq, torch, shape, rot, cb, k, v, [0, 60, 100], [T, T - 1, 300], T, 0, torch.float32)
+    b, sb = _append(iq, torch, shape, rot, cb, k, v, [0, 60, 100], [T, T - 1, 300], 4, 0, torch.float32)
+    assert torch.equal(a.k_codes, b.k_codes) and torch.equal(a.v_codes, b.v_codes) and sa[0] == sb[0] == 0
