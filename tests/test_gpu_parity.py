@@ -1121,3 +1121,30 @@ def test_split_count_does_not_change_the_result(iq, torch, seed):
             assert bool((ws.out[~nz] == 0).all()) and bool(torch.isneginf(ws.lse[~nz]).all()) and bool((ws.argmax[~nz] == -1).all())
         del cache
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("d", [128, 256])
+def test_rotation_buffer_far_from_unit_length(iq, torch, codebooks, d):
+    """The kernels rescale the quaternions of the buffer to unit length. All of them times 2^62 (square sums still in the
+    fp32 range): a step (append of one row, decode, merge) gives what the unit buffer gives, to the bit."""
+    B, H_q, H_kv, T = 2, 8, 2, 300
+    cb = codebook_for(iq, codebooks, d)
+    shape = iq.Shape(B, H_q, H_kv, d, 384)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d)
+    k, v = (torch.randn((B, T, H_kv, d), generator=gen, device="cuda").half() for _ in range(2))
+    q = torch.randn((B, H_q, d), generator=gen, device="cuda").half()
+    unit = torch.empty(iq.iq_rotation_floats(d, H_kv), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H_kv, 9, None, unit)
+    pos = torch.full((B,), T - 1, dtype=torch.int32, device="cuda")
+    results = []
+    for rot in (unit, unit * 2.0 ** 62):
+        cache = iq.new_cache(shape)
+        iq.iq_quantize_append(shape, unit, cb, k[:, :-1], v[:, :-1], torch.zeros_like(pos), None, T - 1, cache)
+        iq.iq_quantize_append(shape, rot, cb, k[:, -1:], v[:, -1:], pos, None, 1, cache)
+        ws = iq.DecodeWorkspace(shape, 1)
+        iq.decode_step(shape, rot, cb, q, cache, pos + 1, ws)
+        results.append((cache.k_codes, cache.v_codes, cache.k_scales, ws.out.clone(), ws.lse.clone()))
+    torch.cuda.synchronize()
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
