@@ -196,9 +196,9 @@ int iq_make_rotation(int32_t head_dim, int32_t n_kv_heads, uint64_t seed, const 
  *                  sequence-length array: the caller advances its lengths. Calls that append to the same
  *                  (sequence, KV head) must be ordered on one stream.
  *   status_dev     optional (see top). Rows with append_pos + i outside [0, t_cap) are skipped and flagged.
- * Arithmetic: fp32 sums (calls of up to 4 rows per sequence: butterfly WHT and 4x4 block products; larger ones: one
+ * Arithmetic: fp32 sums (calls of a few rows per sequence: butterfly WHT and 4x4 block products; larger ones: one
  * tensor-core contraction with the rotation as two binary16 terms); a coordinate closer to a decision threshold than its
- * sum can be off (2^-15 in calls of up to 4 rows; in larger ones 2.25e-5 + 2.3e-6 t at head_dim 128, 5.5e-5 + 9.8e-6 t at 256, t the
+ * sum can be off (2^-15 in calls of a few rows; in larger ones 2.25e-5 + 2.3e-6 t at head_dim 128, 5.5e-5 + 9.8e-6 t at 256, t the
  * largest threshold) is re-decided in fp64 inside the kernel, so the codes equal those of an fp64
  * evaluation except for ties at the fp64 rounding level. The stored scale is sqrt(sum x^2) accumulated
  * in fp64 and rounded to fp32. A zero row stores scale 0 and the code of u = 0 everywhere; a row with an infinity or a NaN

@@ -34,18 +34,37 @@ __device__ __forceinline__ int decide_code_n(T u, const float (&th)[NT], bool& n
   }
 }
 
-template <int D, int BITS = 3>
+// The blocks of the rotation as quaternion pairs (one row per warp), or MANY: as matrices, and the butterfly unrolled, which
+// costs more to set up and less per row (a call of 4 rows, 32 sequences, d = 256, 2 bits: 13.9 us by pairs, 12.4 by matrices; one row
+// 9.3 and 9.8).
+template <int E, bool MANY>
+struct WarpBlocks {
+  float M[E / 4][4][4];
+  __device__ __forceinline__ void load(const float* rot_head, int lane) {
+#pragma unroll
+    for (int j = 0; j < E / 4; j++) so4_matrix<float>(rot_head + (size_t)(lane * (E / 4) + j) * 8, M[j]);
+  }
+  __device__ __forceinline__ void apply(float (&v)[E]) const { so4_apply<float, E, false>(M, v); }
+};
+template <int E>
+struct WarpBlocks<E, false> {
+  QuatPairs<E> qp;
+  __device__ __forceinline__ void load(const float* rot_head, int lane) { qp.load(rot_head, lane); }
+  __device__ __forceinline__ void apply(float (&v)[E]) const { qp.template apply<false>(v); }
+};
+
+template <int D, int BITS = 3, bool MANY = false>
 struct WarpRowQuantizer {
   static constexpr int E = D / 32;  // coordinates per lane
   static constexpr int NB = E / 4;  // SO(4) blocks per lane
   static constexpr int NT = (1 << BITS) - 1;
   const float* qbase;
-  QuatPairs<E> qp;
+  WarpBlocks<E, MANY> blocks;
   float th[NT];
 
   __device__ __forceinline__ void init(const float* rot_head, const float* thresholds, int lane) {
     qbase = rot_head + (size_t)lane * NB * 8;
-    qp.load(rot_head, lane);
+    blocks.load(rot_head, lane);
 #pragma unroll
     for (int i = 0; i < NT; i++) th[i] = thresholds[i];
   }
@@ -80,8 +99,8 @@ struct WarpRowQuantizer {
     float v[E];
 #pragma unroll
     for (int e = 0; e < E; e++) v[e] = x[e];
-    wht_warp<float, E>(v, lane);
-    qp.template apply<false>(v);
+    wht_warp<float, E, MANY>(v, lane);
+    blocks.apply(v);
     bool any_near = false;
 #pragma unroll
     for (int e = 0; e < E; e++) {

@@ -55,7 +55,7 @@ __device__ __forceinline__ double shfl_xor_t<double>(double v, int mask) { retur
 // strides E .. 16E are xor-shuffles (lane bit b <-> stride E << b). d log2 d adds in total (Section 3.2,
 // rotation cost analysis).
 // ------------------------------------------------------------------------------------------------
-template <typename T, int E>
+template <typename T, int E, bool UNROLL = false>
 __device__ __forceinline__ void wht_warp(T (&v)[E], int lane) {
 #pragma unroll
   for (int s = 1; s < E; s <<= 1) {
@@ -68,8 +68,9 @@ __device__ __forceinline__ void wht_warp(T (&v)[E], int lane) {
       }
     }
   }
-  // (a loop: the kernels that use it run it once or twice per warp, where fetching instructions costs more than a branch)
-#pragma unroll 1
+  // (a loop, unless asked otherwise: most kernels run it once or twice per warp, where fetching instructions costs more than a branch)
+  constexpr int STAGES = UNROLL ? 5 : 1;
+#pragma unroll STAGES
   for (int b = 1; b < 32; b <<= 1) {
     const T sgn = (lane & b) ? T(-1) : T(1);  // the upper lane of a pair keeps (other - own)
 #pragma unroll

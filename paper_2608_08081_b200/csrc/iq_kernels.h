@@ -21,7 +21,6 @@ struct PageMap {
 
 // ---- quantize-append
 constexpr int QA_WARPS = 4;
-constexpr int QA_FEW_ROWS = 4;        // calls with at most this many new rows per sequence take the one-warp-per-row latency path
 
 struct QuantizeParams {
   const __half* k_new;

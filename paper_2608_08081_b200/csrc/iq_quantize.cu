@@ -1,5 +1,5 @@
 // Quantize-append for few new rows (Algorithm 1: normalise, WHT, SO(4) blocks, Lloyd-Max, bit-pack; a warp per row: the
-// decode step), the dispatch between it and the bulk kernel (iq_append_bulk.cu), and the calibration kernels. K rows are
+// decode step, the verification of a few drafted rows), the dispatch between it and the bulk kernel (iq_append_bulk.cu), and the calibration kernels. K rows are
 // packed row-major, V rows token-transposed.
 #include "iq_common.cuh"
 #include "iq_kernels.h"
@@ -114,7 +114,7 @@ struct RowQuantizer {
 // blocks), five shuffle stages of the butterfly -- a short instruction stream and no shared memory. The V row goes
 // straight into its transposed records with one read-modify-write per touched word.
 // ---------------------------------------------------------------------------------------------------------
-template <int D, int BITS>
+template <int D, int BITS, bool MANY>
 __global__ void __launch_bounds__(32) quantize_append_few_kernel(const __grid_constant__ QuantizeParams p) {
   constexpr int E = D / 32;
   grid_dependency_wait();
@@ -136,31 +136,37 @@ __global__ void __launch_bounds__(32) quantize_append_few_kernel(const __grid_co
   __half2 raw[E / 2];  // the first row is requested before the rotation blocks are set up: two latencies in one
 #pragma unroll
   for (int k = 0; k < E / 2; k++) raw[k] = reinterpret_cast<const __half2*>(src_base + (size_t)i_lo * p.stride_t)[k];
-  WarpRowQuantizer<D, BITS> rq;
+  WarpRowQuantizer<D, BITS, MANY> rq;
   const RowSink sink{p.k_codes, p.k_scales, p.v_codes, p.v_scales, p.status, p.scale_f16};
   rq.init(p.rot + (size_t)h * (D / 4) * 8, is_v ? p.thresholds_v : p.thresholds_k, lane);
-  // 2 and 4 bits, V rows: the codes of consecutive rows that share a word of the records (8 or 16 rows) are collected in
-  // registers and the word is written once -- whole when every entry of it is new, merged with the old word otherwise --
-  // instead of one read-modify-write per row.
-  uint32_t pend[E];
-  uint32_t pend_mask = 0u;
-  int pend_word = -1;
+  // Several V rows: the codes of consecutive rows that share words of the records (one word of 8 or 16 rows at 4 and 2 bits,
+  // three words of 32 rows at 3) are collected in registers and the words are written once -- whole when every entry is
+  // new, merged with the old word otherwise -- instead of one read-modify-write per row.
+  constexpr int PW = BITS == 3 ? 3 : 1;  // words collected
+  uint32_t pend[E][PW], pend_mask[PW];
+  int pend_word = -1;                    // the first of them within the record
   size_t pend_blk = 0;
 #pragma unroll
-  for (int e = 0; e < E; e++) pend[e] = 0u;
-  auto flush_pending = [&]() {
-    if constexpr (BITS != 3) {
-      if (pend_word >= 0 && pend_mask != 0u) {
+  for (int w = 0; w < PW; w++) {
+    pend_mask[w] = 0u;
 #pragma unroll
-        for (int e = 0; e < E; e++) {
-          uint32_t* dst = reinterpret_cast<uint32_t*>(p.v_codes + (pend_blk * D + lane * E + e) * (size_t)(16 * BITS)) + pend_word;
-          *dst = (pend_mask == 0xFFFFFFFFu) ? pend[e] : ((*dst & ~pend_mask) | pend[e]);
-          pend[e] = 0u;
+    for (int e = 0; e < E; e++) pend[e][w] = 0u;
+  }
+  auto flush_pending = [&]() {
+    if (pend_word >= 0) {
+#pragma unroll
+      for (int e = 0; e < E; e++) {
+        uint32_t* dst = reinterpret_cast<uint32_t*>(p.v_codes + (pend_blk * D + lane * E + e) * (size_t)(16 * BITS)) + pend_word;
+#pragma unroll
+        for (int w = 0; w < PW; w++) {
+          if (pend_mask[w] != 0u) dst[w] = (pend_mask[w] == 0xFFFFFFFFu) ? pend[e][w] : ((dst[w] & ~pend_mask[w]) | pend[e][w]);
+          pend[e][w] = 0u;
         }
       }
-      pend_mask = 0u;
-      pend_word = -1;
     }
+#pragma unroll
+    for (int w = 0; w < PW; w++) pend_mask[w] = 0u;
+    pend_word = -1;
   };
   for (int i = i_lo; i < i_hi; i++) {
     __half2 nxt[E / 2];  // the next row is requested before this one is worked on
@@ -186,19 +192,32 @@ __global__ void __launch_bounds__(32) quantize_append_few_kernel(const __grid_co
       const float s = rq.run(raw, lane, code, p.status);
       if (!is_v) {
         warp_store_k_row<D, BITS>(sink, row, code, s, lane);
-      } else if constexpr (BITS == 3) {
+      } else if constexpr (!MANY) {
         warp_store_v_row<D, BITS>(sink, row, t, code, s, lane);
       } else {
         int word, sh;
-        packed_place<BITS>((int)(t % 128), word, sh);
+        if constexpr (BITS == 3) word = 3 * ((int)(t % 128) / 32);
+        else packed_place<BITS>((int)(t % 128), word, sh);
         if (word != pend_word || row / 128 != pend_blk) {
           flush_pending();
           pend_word = word;
           pend_blk = row / 128;
         }
+        if constexpr (BITS == 3) {  // entry r of the unit: word r / 8, or for the last 8 a bit of each
+          const int r = (int)(t % 32);
+          sh = r < 24 ? 4 * (r & 7) : 4 * (r - 24) + 3;
 #pragma unroll
-        for (int e = 0; e < E; e++) pend[e] |= (uint32_t)code[e] << sh;
-        pend_mask |= ((1u << BITS) - 1u) << sh;
+          for (int w = 0; w < 3; w++) {
+            const uint32_t bits = r < 24 ? (r >> 3 == w ? 7u : 0u) : 1u;
+            pend_mask[w] |= bits << sh;
+#pragma unroll
+            for (int e = 0; e < E; e++) pend[e][w] |= (((uint32_t)code[e] >> (r < 24 ? 0 : w)) & bits) << sh;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < E; e++) pend[e][0] |= (uint32_t)code[e] << sh;
+          pend_mask[0] |= ((1u << BITS) - 1u) << sh;
+        }
         if (lane == 0) store_scale(p.v_scales, row, s, p.scale_f16, p.status);
       }
     }
@@ -207,7 +226,7 @@ __global__ void __launch_bounds__(32) quantize_append_few_kernel(const __grid_co
       for (int k = 0; k < E / 2; k++) raw[k] = nxt[k];
     }
   }
-  flush_pending();
+  if constexpr (MANY) flush_pending();
 }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -309,19 +328,29 @@ cudaError_t launch_wht_coordinates(const WhtParams& p, int head_dim, int batch, 
                          : launch_after_predecessor(wht_coordinates_kernel<256>, grid, dim3(QA_WARPS * 32), 0, stream, p);
 }
 
-template <int D, int BITS>
-static cudaError_t launch_few(const QuantizeParams& p, int batch, cudaStream_t stream) {
+template <int D, int BITS, bool MANY>
+static cudaError_t launch_few_rows(const QuantizeParams& p, int batch, cudaStream_t stream) {
   // x = 2 * chunk + (0: the K rows, 1: the V rows) of (sequence, KV head); a chunk is the part of the new rows inside
   // one 128-row block of the cache (+1: the first row may sit in the middle of a block)
   dim3 grid(2 * ((p.n_new_max + 127) / 128 + 1), p.n_kv_heads, batch);
-  return launch_after_predecessor(quantize_append_few_kernel<D, BITS>, grid, dim3(32), 0, stream, p);
+  return launch_after_predecessor(quantize_append_few_kernel<D, BITS, MANY>, grid, dim3(32), 0, stream, p);
+}
+template <int D, int BITS>
+static cudaError_t launch_few(const QuantizeParams& p, int batch, cudaStream_t stream) {
+  return p.n_new_max > 1 ? launch_few_rows<D, BITS, true>(p, batch, stream) : launch_few_rows<D, BITS, false>(p, batch, stream);
 }
 
 cudaError_t launch_quantize_append(const QuantizeParams& p, int head_dim, int batch, cudaStream_t stream) {
   if (p.n_new_max <= 0 || batch <= 0) return cudaSuccess;
-  // Up to 4 rows per sequence: a warp per row (5 us for one row; the bulk kernel's set-up alone takes as long). More: the
-  // bulk kernel, unless two thresholds of a 2- or 4-bit codebook are too close together for its decision.
-  if (p.n_new_max > QA_FEW_ROWS && append_bulk_takes(p, head_dim)) return launch_append_bulk(p, head_dim, batch, stream);
+  // Few rows per sequence: a warp for the rows that fall into a block, one after the other (5 us for one row, 0.7 - 1.6 us for each
+  // more). More: the bulk kernel, which takes a whole tile for a block however few of its rows are new, unless two thresholds
+  // of a 2- or 4-bit codebook are too close together for its decision. The line lies where the two met at 2, 3 and 4 bits, in us
+  // for 8 rows / at the line (warp per block, bulk), 8 KV heads, 1 - 8 / 32 / 128 sequences:
+  //   d = 128: 10 - 15 / 11 - 15 / 20 - 26 and 13 - 17 at 10 / 23 - 30 at 20 / 49 - 66 at 24; bulk 12 - 26 / 24 - 33 / 53 - 79
+  //   d = 256: 14 - 22 / 17 - 25 / 31 - 45 and 20 - 36 at 14 / 40 - 66 at 28 / 110 - 180 at 42; bulk 20 - 35 / 46 - 68 / 122 - 190
+  const long long pairs = (long long)batch * p.n_kv_heads;
+  const int line = head_dim == 128 ? (pairs < 128 ? 10 : (pairs < 512 ? 20 : 24)) : (pairs < 128 ? 14 : (pairs < 512 ? 28 : 42));
+  if (p.n_new_max > line && append_bulk_takes(p, head_dim)) return launch_append_bulk(p, head_dim, batch, stream);
   if (p.bits == 2) return head_dim == 128 ? launch_few<128, 2>(p, batch, stream) : launch_few<256, 2>(p, batch, stream);
   if (p.bits == 4) return head_dim == 128 ? launch_few<128, 4>(p, batch, stream) : launch_few<256, 4>(p, batch, stream);
   return head_dim == 128 ? launch_few<128, 3>(p, batch, stream) : launch_few<256, 3>(p, batch, stream);

@@ -286,3 +286,28 @@ def test_three_bit_codebooks_with_close_or_far_thresholds(iq, torch, d, form):  
     a, sa = _append(iq, torch, shape, rot, cb, k, v, [0, 60, 100], [T, T - 1, 300], T, 0, torch.float32)
     b, sb = _append(iq, torch, shape, rot, cb, k, v, [0, 60, 100], [T, T - 1, 300], 4, 0, torch.float32)
     assert torch.equal(a.k_codes, b.k_codes) and torch.equal(a.v_codes, b.v_codes) and sa[0] == sb[0] == 0
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("B,H", [(3, 2), (30, 5), (130, 4)])
+def test_calls_on_both_sides_of_the_line_between_the_kernels(iq, torch, bits, d, B, H):  # noqa: F811
+    """2 to 44 rows per sequence (the line lies between 10 and 42, by batch and head size), starting and ending inside words,
+    units and blocks of the V records: the bytes of calls of one row."""
+    lv, th, lvv, thv = two_codebooks(d, bits, "int8", True)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)), tuple(map(float, lvv)), tuple(map(float, thv)))
+    shape = iq.Shape(B, H, H, d, 256, bits=bits)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 4, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits + B)
+    T = 44
+    k, v = (torch.randn((B, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    first = [(37 * b) % 190 for b in range(B)]
+    lens = [T - (b % 5 == 3) * 7 for b in range(B)]
+    ref, _ = _append(iq, torch, shape, rot, cb, k, v, first, lens, 1, 0, torch.float32)
+    for rows in (2, 7, 10, 11, 20, 24, 25, 28, 29, 42, 43, 44):
+        got, status = _append(iq, torch, shape, rot, cb, k, v, first, lens, rows, 0, torch.float32)
+        for name in ("k_codes", "v_codes", "k_scales", "v_scales"):
+            assert torch.equal(getattr(got, name), getattr(ref, name)), (rows, name)
+        assert status[0] == 0 and status[2] == 0
