@@ -146,7 +146,7 @@ __device__ __forceinline__ void patch_code(uint32_t* run, int e, int code) {
 }
 
 // The listed coordinates in fp64, eight lanes each: z = the four outputs of the coordinate's block of H x (exact sums),
-// u = its row of M_b times z, over the exact norm, against the thresholds from the first that it may be above.
+// u = its row of M_b times z, over the exact norm, against the thresholds from the first that it may not be above.
 template <int D, int BITS>
 static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const double* m_s, const __half* const* src_s,
                                               uint32_t* const* dst_s, const uint32_t* info_s, int n, int lane) {
@@ -158,7 +158,7 @@ static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const dou
     const bool act = e < n;
     const int ee = act ? e : n - 1;
     const uint32_t info = info_s[ee];
-    const int coord = info & 0xff, entry = (info >> 8) & 0xff, lower = (info >> 16) & 15;
+    const int coord = info & 0xff, entry = (info >> 8) & 0xff, nearest = (info >> 16) & 15;
     const uint4* src = reinterpret_cast<const uint4*>(src_s[ee] + li * EPL);
     const int blk = coord >> 2;
     double z[4] = {0.0, 0.0, 0.0, 0.0}, ss = 0.0;
@@ -192,7 +192,7 @@ static __device__ __noinline__ void bulk_redo(const QuantizeParams& p, const dou
     const double* m = m_s + 4 * coord;
     const double u = (m[0] * z[0] + m[1] * z[1] + m[2] * z[2] + m[3] * z[3]) * inv_sqrt(ss);  // (rows of norm zero are not listed)
     const float* th = ((info >> 20) & 1u) ? p.thresholds_v : p.thresholds_k;
-    int code = lower;
+    int code = max(nearest - 1, 0);
     while (code < (1 << BITS) - 1 && u > (double)th[code]) code++;
     if (act && li == 0) patch_code<BITS>(dst_s[ee], entry, code);
   }
@@ -776,30 +776,33 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
             // some coordinate of the warp lies in a band (or the tile has rows to be treated apart): the words in question
             // again, with the nearest codes, and the coordinates of new rows go on the list
             const uint32_t odd_words = (odd[0] ? 1u : 0u) | (odd[1] ? 2u : 0u) | (odd[2] ? 4u : 0u) | (odd[3] ? 8u : 0u);
-            const int c_lo = cur->c_lo, c_hi = cur->c_hi;
+            const uint32_t valid = is_v ? new_rows(cur->c_lo, cur->c_hi, ch) : (r >= cur->c_lo && r < cur->c_hi ? 255u : 0u);  // the new rows
 #pragma unroll 1
             for (int q = 0; q < 4; q++) {
               if (!special && !__any_sync(FULL, (odd_words >> q) & 1u)) continue;
-              uint32_t x8[8], nw = 0u, low = 0u, near_m = 0u;  // the nearest codes, the codes below, which of them are undecided (+ 8: of a zero row, at a threshold)
+              uint32_t x8[8], nw = 0u, near_m = 0u;  // the nearest codes, which of them are undecided (+ 8: of a zero row, at a threshold)
+              float b8[8];
               tc_ld8(tmem_t + 32 * ch + 8 * q, x8);
 #pragma unroll
+              for (int i = 0; i < 8; i++) b8[i] = is_v ? binv_s[32 * ch + 8 * q + i] : binv;
+#pragma unroll
               for (int i = 0; i < 8; i++) {
-                const int col = 32 * ch + 8 * q + i, row = is_v ? col : r;
-                const float x = __uint_as_float(x8[i]), b = is_v ? binv_s[col] : binv;
-                const uint32_t cb = __float_as_uint(bulk_decide<BITS, MODE, NS>(x, b, off));
-                uint32_t code = ((cb + 0x0003FFFFu) >> 19) & 15u;
-                const bool odd_c = (cb & 0x0007FFFFu) != 0u;
-                if (b == 0.f) {  // a row of norm zero: u = 0; one whose norm is not finite: not a number, above no threshold
-                  const float z = x * 0.f;
-                  const uint32_t zc = (uint32_t)zero_code_s[is_v ? 1 : 0];
-                  code = z != z ? 0u : zc & 15u;
-                  if (z == z && zc >= 16u && row >= c_lo && row < c_hi) near_m |= 256u << i;  // (only counted)
-                } else if (odd_c && row >= c_lo && row < c_hi) {
-                  near_m |= 1u << i;
-                }
-                nw |= code << (4 * i);
-                low |= ((cb >> 19) & 15u) << (4 * i);
+                const uint32_t cb = __float_as_uint(bulk_decide<BITS, MODE, NS>(__uint_as_float(x8[i]), b8[i], off));
+                nw |= (((cb + 0x0003FFFFu) >> 19) & 15u) << (4 * i);
+                if (cb & 0x0007FFFFu) near_m |= 1u << i;
               }
+              if (special) {
+#pragma unroll
+                for (int i = 0; i < 8; i++) {
+                  if (b8[i] != 0.f) continue;
+                  const float z = __uint_as_float(x8[i]) * 0.f;  // a row of norm zero: u = 0; one whose norm is not finite: not a number, above no threshold
+                  const uint32_t zc = (uint32_t)zero_code_s[is_v ? 1 : 0];
+                  nw = (nw & ~(15u << (4 * i))) | (z != z ? 0u : (zc & 15u) << (4 * i));
+                  near_m &= ~(1u << i);
+                  if (z == z && zc >= 16u) near_m |= 256u << i;  // (only counted)
+                }
+              }
+              near_m &= ((is_v ? valid >> (8 * q) : valid) & 255u) * 257u;
 #pragma unroll
               for (int k = 0; k < 4; k++) nib[k] = (k == q) ? nw : nib[k];
               uint32_t rows;
@@ -824,7 +827,7 @@ __global__ void __launch_bounds__(BulkLayout<D>::THREADS, 1) append_bulk_kernel(
                 const int k = atomicAdd(n_list_s, 1);
                 src_s[k] = cur->src + (long long)row * p.stride_t;
                 dst_s[k] = run_of();
-                info_s[k] = (uint32_t)coord | ((uint32_t)(is_v ? row : coord) << 8) | (((low >> (4 * i)) & 15u) << 16) | (is_v ? 1u << 20 : 0u);
+                info_s[k] = (uint32_t)coord | ((uint32_t)(is_v ? row : coord) << 8) | (((nw >> (4 * i)) & 15u) << 16) | (is_v ? 1u << 20 : 0u);
               }
               __syncwarp();
             }
