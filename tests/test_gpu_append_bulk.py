@@ -311,3 +311,39 @@ def test_calls_on_both_sides_of_the_line_between_the_kernels(iq, torch, bits, d,
         for name in ("k_codes", "v_codes", "k_scales", "v_scales"):
             assert torch.equal(getattr(got, name), getattr(ref, name)), (rows, name)
         assert status[0] == 0 and status[2] == 0
+
+
+@pytest.mark.parametrize("d,bits,variant", [(128, 2, "paged"), (128, 3, "shifted"), (128, 3, "binary16 scales"), (128, 4, "paged"), (128, 4, "shifted"),
+                                            (256, 2, "shifted"), (256, 3, "paged"), (256, 4, "binary16 scales"), (256, 4, "shifted")])
+def test_many_tiles_per_group(iq, torch, bits, d, variant):  # noqa: F811
+    """Enough 128-row tiles that every group of every CTA takes several of a head one after the other and goes on to another
+    head: buffers, accumulators and barrier phases are used again, lists and marks carry over tiles. Rows that tie throughout,
+    rows with one element, zero rows; sequences that start and end inside blocks. Bytes of calls of four rows (the row kernel)."""
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    B, H = 6, 7
+    groups = 4 if d == 128 else 2
+    T = 128 * -(-(4 * groups * sm) // (2 * B * H)) + 77     # at least four tiles per group
+    shape = iq.Shape(B, H, H, d, (T + 300 + 127) // 128 * 128, bits=bits)
+    lv, th, lvv, thv = two_codebooks(d, bits, "int8", True)
+    if variant == "shifted":
+        th = (th.astype(np.float64) + 0.01 * ((np.arange(len(th)) * 7) % 5 - 2)).astype(np.float32)
+    cb = iq.Codebook(tuple(map(float, lv)), tuple(map(float, th)), tuple(map(float, lvv)), tuple(map(float, thv)))
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 21, None, rot)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits)
+    kv = torch.randn((B, T, H, 2 * d), generator=gen, device="cuda").half()
+    kv[..., ::37] *= 20
+    kv[:, 5::43] = 1
+    kv[:, 400:437] = 1                    # a run that fills units and crosses blocks
+    kv[:, 7::91, :, 1:] = 0
+    kv[:, 2::111] = 0
+    k, v = kv[..., :d], kv[..., d:]
+    first, lens = [0, 3, 127, 128, 200, 291], [T, T - 1, T - 100, T, T - 64, T]
+    page_rows, scales = (128 if variant == "paged" else 0), (torch.float16 if variant == "binary16 scales" else torch.float32)
+    bulk, st = _append(iq, torch, shape, rot, cb, k, v, first, lens, T, page_rows, scales)
+    rows, st_rows = _append(iq, torch, shape, rot, cb, k, v, first, lens, 4, page_rows, scales)
+    for name in ("k_codes", "v_codes", "k_scales", "v_scales"):
+        a, b = getattr(bulk, name), getattr(rows, name)
+        assert torch.equal(a, b), f"{name}: {int((a != b).sum())} of {a.numel()} differ"
+    assert st[0] == st_rows[0] == 0 and st[2] == st_rows[2] == 0

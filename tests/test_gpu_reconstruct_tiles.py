@@ -128,3 +128,49 @@ def test_levels_off_the_grid_by_an_fp32_place_are_used_as_they_are(iq, torch, d)
     torch.cuda.synchronize()
     for o in (ko, vo):
         assert (o[..., 0] == 1 + 2.0 ** -10).all() and (o[..., 1:] == 0).all()
+
+
+def _against_the_oracle(iq, torch, d, bits, form, H, T, table_of, lens):  # noqa: F811
+    """Five sequences of T rows in a scattered pool of 128-row pages; sequence b of the call reads the pages of sequence
+    table_of[b], lens[b] rows."""
+    t_cap = (T + 127) // 128 * 128
+    pages = np.random.default_rng(d + bits).permutation(5 * (t_cap // 128)).astype(np.int32).reshape(5, -1)
+    part, shape = (iq.Shape(n, H, H, d, t_cap, bits=bits) for n in (5, len(lens)))
+    cb = iq.iq_lloyd_max_codebook(d, bits, form)
+    rot = torch.empty(iq.iq_rotation_floats(d, H), dtype=torch.float32, device="cuda")
+    iq.iq_make_rotation(d, H, 8, None, rot)
+    pool, whole = iq.new_paged_cache(part, pages.size, 128, torch.from_numpy(pages).cuda()), iq.new_cache(part)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(d + bits)
+    k, v = (torch.randn((5, T, H, d), generator=gen, device="cuda").half() for _ in range(2))
+    for c in (pool, whole):   # (contiguous for the oracle)
+        iq.iq_quantize_append(part, rot, cb, k, v, torch.zeros(5, dtype=torch.int32, device="cuda"), None, T, c)
+    cache = iq.Cache(pool.k_codes, pool.k_scales, pool.v_codes, pool.v_scales, torch.from_numpy(pages[table_of]).cuda(), 128)
+    ko, vo = (torch.full((len(lens), T, H, d), 7.0, dtype=torch.float16, device="cuda") for _ in range(2))
+    iq.iq_reconstruct_rows(shape, rot, cb, cache, torch.tensor(lens, dtype=torch.int32, device="cuda"), ko, vo)
+    torch.cuda.synchronize()
+    refs = oracle.reconstruct_rows(rot.cpu().numpy().reshape(H, d // 4, 8), np.array(cb.levels, np.float32), cache_to_numpy(whole),
+                                   np.full(5, T, np.int32), H, d=d)
+    for out, ref in zip((ko, vo), refs):
+        want = torch.from_numpy(np.ascontiguousarray(np.asarray(ref)[:, :T])).cuda()
+        bound = 2.0 ** -11 * 1.001 * want.abs() + 1e-5 * want.abs().amax(dim=-1, keepdim=True) + 2.0 ** -25
+        for b, n in enumerate(lens):
+            assert (out[b, n:] == 7.0).all()
+            assert ((out[b, :n].double() - want[table_of[b], :n]).abs() <= bound[table_of[b], :n]).all(), b
+
+
+@pytest.mark.parametrize("form", ["int8", "fp16"])
+@pytest.mark.parametrize("d,bits", [(128, 2), (128, 3), (128, 4), (256, 2), (256, 3), (256, 4)])
+def test_many_tiles_per_group(iq, torch, d, bits, form):  # noqa: F811
+    """Enough 128-row tiles that every group of every CTA takes at least four, one after the other, K and then V, and goes on
+    to another head: buffers, accumulators and barrier phases are used again."""
+    groups = (4 if d == 128 else 2) * torch.cuda.get_device_properties(0).multi_processor_count
+    H = 3
+    T = 128 * -(-4 * groups // (2 * H * 4))
+    _against_the_oracle(iq, torch, d, bits, form, H, T, [3, 0, 4, 1, 2], [T, T - 1, T - 127, T - 300, T])
+
+
+@pytest.mark.parametrize("d,bits", [(128, 3), (256, 4)])
+def test_more_sequences_than_threads_of_a_cta(iq, torch, d, bits):  # noqa: F811
+    lens = [(b * 37) % 300 * (b % 3 != 1) for b in range(1100)]
+    _against_the_oracle(iq, torch, d, bits, "int8", 1, 300, [b % 5 for b in range(1100)], lens)
