@@ -37,11 +37,12 @@
 // warps (eight at d = 256), each with a tile buffer and accumulator columns of its own, take the tiles in turn. A group
 // copies its next tile in (cp.async) while it packs the present one; a control warp per group finds the tiles and issues
 // the MMAs. The groups run in different phases, so that copies, norms and contractions of one run under the packing of
-// the others, which is what bounds the kernel (about 11 instructions per coordinate).
+// the others. No pipe is near its limit and issue is at 42 %: what bounds the kernel is that a group's phases run one after the
+// other, and the groups that fit do not cover them.
 //
 // Measured (K and V rows of 8 KV heads, Gaussian with outlier channels), against one row in 8 or 16 lanes with butterflies
-// by shuffle and a kernel per tensor: 1.6 M rows, d = 128, 3 bits: 278 us instead of 491 (1.8 TB/s of rows in and codes
-// out); 262 k rows, d = 256, 4 bits: 169 instead of 457; 50 k rows in chunks of 500 per sequence: 28.2 instead of 54.5.
+// by shuffle and a kernel per tensor: 1.6 M rows, d = 128, 3 bits: 255 us instead of 491 (1.9 TB/s of rows in and codes
+// out); 262 k rows, d = 256, 4 bits: 187 instead of 457; 50 k rows in chunks of 500 per sequence: 26.0 instead of 54.5.
 #include <cmath>
 
 #include "iq_append_row.cuh"

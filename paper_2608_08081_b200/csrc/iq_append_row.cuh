@@ -35,8 +35,8 @@ __device__ __forceinline__ int decide_code_n(T u, const float (&th)[NT], bool& n
 }
 
 // The blocks of the rotation as quaternion pairs (one row per warp), or MANY: as matrices, and the butterfly unrolled, which
-// costs more to set up and less per row (a call of 4 rows, 32 sequences, d = 256, 2 bits: 13.9 us by pairs, 12.4 by matrices; one row
-// 9.3 and 9.8).
+// costs more to set up and less per row (32 sequences, 8 KV heads, d = 256, 2 bits: calls of 2 rows 10.0 us by pairs, 9.6 by
+// matrices, 4 rows 13.8 and 12.3, 32 rows 60 and 47).
 template <int E, bool MANY>
 struct WarpBlocks {
   float M[E / 4][4][4];

@@ -1,4 +1,4 @@
-"""The bulk append kernel (Algorithm 1 on the tensor cores) against the warp-per-row kernel that calls of up to four rows
+"""The bulk append kernel (Algorithm 1 on the tensor cores) against the warp-per-row kernel that calls of a few rows
 take, byte for byte, and against the oracle: tile edges (first and last rows inside 128-row blocks), every bit width, both
 forms of the decision (thresholds symmetric about zero or not), two codebooks, strided inputs, paged caches, binary16
 scales, rows whose coordinates all sit on a threshold, zero rows, rows that end a sequence outside the cache."""
@@ -86,8 +86,8 @@ def test_bulk_append_codes_match_the_oracle(iq, torch, d, bits, n):  # noqa: F81
 
 
 def test_codebook_with_close_thresholds_keeps_its_path(iq, torch):  # noqa: F811
-    """Thresholds 1e-5 apart cannot be told apart by the bulk kernel's decision: such a call takes the row kernel whatever
-    its size and gives what calls of four rows give."""
+    """Thresholds 1e-5 apart cannot be told apart by the bulk kernel's saturating sums: such a call is decided in another way
+    and gives what calls of four rows give."""
     d, T = 128, 200
     lv, th, _, _ = two_codebooks(d, 3, "int8", False)
     th = th.copy()
