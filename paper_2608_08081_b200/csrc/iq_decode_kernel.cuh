@@ -97,7 +97,7 @@ struct DecLayout {
   static constexpr int PRE_BYTES = DEC_NPRE * BQ_BYTES;  // the prepared query operands, shared by the groups
   static constexpr int SMEM_BYTES = DEC_HDR_BYTES + PRE_BYTES + NG * GROUP_SMEM;
   // header offsets
-  static constexpr int BAR_STRIDE = 96;  // per group: full[3], empty[3], s_bar, o_bar, k_ready, p_ready
+  static constexpr int BAR_STRIDE = 96;  // per group: full[3], s_bar, o_bar, k_ready, p_ready
   static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
   // OFF_PRE: count, [DEC_NPRE] (sequence, item), [DEC_NPRE] score factors, [DEC_NPRE][8] per-head maxima
   static constexpr int DESC_STRIDE = STAGES * 32;  // per group
@@ -379,8 +379,10 @@ __device__ __forceinline__ void pad8(const T (&v)[HN], T fill, T (&out)[8]) {
 #pragma unroll
   for (int h = 0; h < 8; h++) out[h] = h < HN ? v[h < HN ? h : 0] : fill;
 }
-__device__ __forceinline__ float max_of(const float (&v)[8]) { return max3f(max3f(v[0], v[1], v[2]), max3f(v[3], v[4], v[5]), fmaxf(v[6], v[7])); }
-__device__ __forceinline__ float max_of(const float (&v)[4]) { return fmaxf(max3f(v[0], v[1], v[2]), v[3]); }
+__device__ __forceinline__ float max_of(const F32x2 (&v)[4]) {
+  return max3f(max3f(v[0].lo(), v[0].hi(), v[1].lo()), max3f(v[1].hi(), v[2].lo(), v[2].hi()), fmaxf(v[3].lo(), v[3].hi()));
+}
+__device__ __forceinline__ float max_of(const F32x2 (&v)[2]) { return fmaxf(max3f(v[0].lo(), v[0].hi(), v[1].lo()), v[1].hi()); }
 
 // Where the CTA's range starts (thread 0, set-up).
 struct DecStart {
@@ -423,11 +425,10 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 
   uint64_t* gbar = reinterpret_cast<uint64_t*>(smem + grp * L::BAR_STRIDE);
   uint64_t* full_bar = gbar;        // [stages] tile landed (or end marker)
-  uint64_t* empty_bar = gbar + 3;   // [stages] staged tile consumed (128 arrivals)
-  uint64_t* s_bar = gbar + 6;       // scores ready
-  uint64_t* o_bar = gbar + 7;       // values ready
-  uint64_t* k_ready = gbar + 8;     // K tile in TMEM (128 arrivals)
-  uint64_t* p_ready = gbar + 9;     // V tile in TMEM + probabilities in smem (128 arrivals)
+  uint64_t* s_bar = gbar + 3;       // scores ready
+  uint64_t* o_bar = gbar + 4;       // values ready
+  uint64_t* k_ready = gbar + 5;     // K tile in TMEM (128 arrivals)
+  uint64_t* p_ready = gbar + 6;     // V tile in TMEM + probabilities in smem, staged tile consumed (128 arrivals)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_TMEM);
   int* next_s = reinterpret_cast<int*>(smem + L::OFF_NEXT);            // next block of the CTA's range
   DecStart* start_s = reinterpret_cast<DecStart*>(smem + L::OFF_START);
@@ -638,7 +639,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   // ---------------------------------------------------------------- set-up: barriers, TMEM
   if (control && elect_one()) {  // every control warp initialises the barriers of its group
 #pragma unroll
-    for (int st = 0; st < NST; st++) { mbar_init(&full_bar[st], 1); mbar_init(&empty_bar[st], DEC_GROUP_THREADS); }
+    for (int st = 0; st < NST; st++) mbar_init(&full_bar[st], 1);
     mbar_init(s_bar, 1);
     mbar_init(o_bar, 1);
     mbar_init(k_ready, DEC_GROUP_THREADS);
@@ -665,7 +666,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   const uint32_t tmem_base = tmem_slot[0];
   const uint32_t tmem_g = tmem_base + (uint32_t)(grp * L::GROUP_COLS);        // this group's columns
   const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;                // this warp's 32 TMEM lanes
-  bool failed = false;  // a bounded wait gave up; every later wait of this thread is skipped
+  bool failed = false;  // a bounded wait gave up: the thread leaves its loop
 
   if (control) {
     // ================================================================ control warp of group grp: walks the work, fetches blocks, issues MMAs.
@@ -704,11 +705,9 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       dec_draw<D>(p, wk, dr, next_s, lane, ARGMAX ? 1 : 0);
     };
     auto stage_next = [&]() {  // the drawn (or next) block into slot it_issue, or the end marker
-      const int st = it_issue % NST;
-      if (it_issue >= NST && !failed)  // the slot's previous occupant has been consumed
-        failed = !mbar_wait_bounded(&empty_bar[st], (uint32_t)(it_issue / NST - 1) & 1u, DEC_WAIT_LIMIT);
-      if (dr.kind < 0 && !failed) draw();
-      if (dr.kind == 0 && !failed) {
+      const int st = it_issue % NST;  // (its previous occupant has been consumed: it is a block whose p_ready this warp has waited for)
+      if (dr.kind < 0) draw();
+      if (dr.kind == 0) {
         const int r0 = dr.blk * TB;
         const int n = min(TB, dr.len - r0);
         if (elect_one()) {
@@ -741,7 +740,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       while (!ended && it_issue - it < NST) stage_next();  // keep the pipeline full (at the start: tiles in flight while the compute warps open their first segment)
       if (ended && it == it_issue - 1) { it++; break; }  // slot `it` holds the end marker
       // scores of the block in slot `it`: S = A_K * B_Q^T once all 128 rows are in TMEM (and B_Q of its segment is complete)
-      if (!failed) failed = !mbar_wait_bounded(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
+      failed = !mbar_wait_bounded(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
       if (failed) break;
       tc_fence_after();
       const int bqbuf = desc[it % NST].bqbuf;  // the query operand of the block's segment (the start address field counts 16-byte units)
@@ -800,8 +799,13 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     const float inv_root_d = rsqrtf((float)D);
     const float kfac = p.sm_scale * LOG2E * inv_root_d;  // scores in log2 units: z2 = S_raw * scale_K * kfac
     const float vfac = inv_root_d;
-    float acc[DJ][HN];  // thread c: coordinates c (+128), HN heads
-    float m_run[HN], l_run[HN], best_v[HN];
+    // Per head, in pairs (fma2, add2, mul2: one instruction for two heads, the negated reference as the addend): thread c's
+    // values of coordinates c (+128), minus the running reference, the thread's share of the softmax sum. With the mask of stale
+    // rows behind a uniform branch and without a barrier of its own for consumed tiles: a step over 32 x 32 K rows 175.8 ->
+    // 171.2 us, binary16 levels 58.3 -> 56.2.
+    F32x2 acc[DJ][HN / 2], neg_m[HN / 2], l2[HN / 2];
+    auto of_head = [](const F32x2 (&v)[HN / 2], int h) { return (h & 1) ? v[h / 2].hi() : v[h / 2].lo(); };
+    float best_v[HN];
     int best_i[HN];
     float sfac = 0.f;  // integer path: score digits -> log2-domain score per unit K scale (set when a segment is opened)
     int it = 0;        // staged slots of this group consumed so far (tile pipeline phases), the end marker included
@@ -875,9 +879,11 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
       for (int j = 0; j < DJ; j++)
 #pragma unroll
-        for (int h = 0; h < HN; h++) acc[j][h] = 0.f;
+        for (int h2 = 0; h2 < HN / 2; h2++) acc[j][h2] = f32x2(0.f, 0.f);
 #pragma unroll
-      for (int h = 0; h < HN; h++) { m_run[h] = -INFINITY; l_run[h] = 0.f; best_v[h] = -INFINITY; best_i[h] = -1; }
+      for (int h2 = 0; h2 < HN / 2; h2++) { neg_m[h2] = f32x2(INFINITY, INFINITY); l2[h2] = f32x2(0.f, 0.f); }
+#pragma unroll
+      for (int h = 0; h < HN; h++) { best_v[h] = -INFINITY; best_i[h] = -1; }
       if (bqbuf >= 0) {
         if (I8) sfac = pre_sfac[bqbuf];
         return;
@@ -917,18 +923,19 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         for (int h = 0; h < HN; h++)
           if (h < nh) {
 #pragma unroll
-            for (int j = 0; j < DJ; j++) dst[h * hstride + 128 * j] = acc[j][h];
+            for (int j = 0; j < DJ; j++) dst[h * hstride + 128 * j] = of_head(acc[j], h);
           }
         const int hr = warp_reduce8_head(lane);  // the head whose sum this lane ends up with
         float l8[8];
-        pad8(l_run, 0.f, l8);
-        const float lsum = warp_reduce8(l8, lane, [](float x, float y) { return x + y; });
-        float msel = m_run[0];  // m_run[hr] (every thread of the group holds the same references)
 #pragma unroll
-        for (int h = 1; h < HN; h++) msel = (hr == h) ? m_run[h] : msel;
+        for (int h = 0; h < 8; h++) l8[h] = h < HN ? of_head(l2, h % HN) : 0.f;
+        const float lsum = warp_reduce8(l8, lane, [](float x, float y) { return x + y; });
+        float msel = of_head(neg_m, 0);  // that of hr (every thread of the group holds the same references)
+#pragma unroll
+        for (int h = 1; h < HN; h++) msel = (hr == h) ? of_head(neg_m, h) : msel;
         if ((lane & 3) == 0) {
           red[(warp & 3) * 8 + hr] = lsum;
-          if ((warp & 3) == 0) red2[hr] = msel;
+          if ((warp & 3) == 0) red2[hr] = -msel;
         }
         group_bar_sync(bar_id);
         if (gt < nh) {
@@ -941,7 +948,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       {
         const int hr = warp_reduce8_head(lane);  // the head whose sums this lane ends up with
         float l8[8];
-        pad8(l_run, 0.f, l8);
+#pragma unroll
+        for (int h = 0; h < 8; h++) l8[h] = h < HN ? of_head(l2, h % HN) : 0.f;
         const float lsum = warp_reduce8(l8, lane, [](float x, float y) { return x + y; });
         if ((lane & 3) == 0) red[(warp & 3) * 8 + hr] = lsum;
         if (ARGMAX) {
@@ -959,7 +967,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       float scale[8];  // the partial is reported relative to the exact maximum where that is tracked
 #pragma unroll
       for (int h = 0; h < HN; h++) {
-        float mt = m_run[h];  // every thread of the group holds the same reference
+        const float m_run = -of_head(neg_m, h);  // every thread of the group holds the same reference
+        float mt = m_run;
         int bi = -1;
         if (ARGMAX) {
           mt = -INFINITY;
@@ -968,7 +977,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
             argmax_merge(mt, bi, red2[wq * 8 + h], redi[wq * 8 + h]);
           }
         }
-        scale[h] = ARGMAX ? ex2f(m_run[h] - mt) : 1.f;
+        scale[h] = ARGMAX ? ex2f(m_run - mt) : 1.f;
         if (gt == h && h < nh) {
           const size_t o = ((size_t)seg_b * p.n_q_heads + h0 + h) * S + seg_slot;
           p.part_ml[2 * o] = mt * LN2;
@@ -981,17 +990,39 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if (h < nh) {
 #pragma unroll
           for (int j = 0; j < DJ; j++)
-            p.part_acc[(((size_t)seg_b * p.n_q_heads + h0 + h) * S + seg_slot) * D + gt + 128 * j] = acc[j][h] * scale[h];
+            p.part_acc[(((size_t)seg_b * p.n_q_heads + h0 + h) * S + seg_slot) * D + gt + 128 * j] = of_head(acc[j], h) * scale[h];
         }
       // (the scratch is written next after the group barrier of the next block's vote)
+    };
+
+    // ---- the references raised above the block's maxima (in `red`), whichever head asked: fewer raises later. The sums and the
+    // accumulator hold the blocks before this one: they are rescaled now.
+    auto raise = [&](const F32x2 (&x2)[HN / 2], float kf, bool stale, F32x2 (&over)[HN / 2]) {
+#pragma unroll
+      for (int h2 = 0; h2 < HN / 2; h2++) {
+        float nm[2], alpha[2];
+#pragma unroll
+        for (int i = 0; i < 2; i++) {
+          const int h = 2 * h2 + i;
+          const float bm = fmaxf(fmaxf(red[h], red[8 + h]), fmaxf(red[16 + h], red[24 + h]));
+          const float old = of_head(neg_m, h);
+          nm[i] = fminf(old, -(bm + DEC_RAISE_MARGIN));
+          alpha[i] = ex2f(nm[i] - old);
+        }
+        const F32x2 alpha2 = f32x2(alpha[0], alpha[1]);
+        neg_m[h2] = f32x2(nm[0], nm[1]);
+        l2[h2] = mul2(l2[h2], alpha2);
+#pragma unroll
+        for (int j = 0; j < DJ; j++) acc[j][h2] = mul2(acc[j][h2], alpha2);
+        over[h2] = stale ? f32x2(-INFINITY, -INFINITY) : fma2(x2[h2], f32x2(kf, kf), neg_m[h2]);
+      }
     };
 
     int st = 0;          // stage of slot `it` and its phase, kept incrementally
     uint32_t st_ph = 0;
     int2 dsc = make_int2(-1, 0);  // (valid rows | end marker, flags) of slot `it`; the rest of its descriptor is read where it is needed
-    auto next_slot = [&]() {      // wait for slot `it` and read its descriptor
-      if (!failed) failed = !mbar_wait_bounded(&full_bar[st], st_ph, DEC_WAIT_LIMIT);
-      if (failed) { dsc.x = -1; return; }
+    auto next_slot = [&]() {      // wait for slot `it` and read its descriptor; a wait that gave up ends the work like an end marker
+      if (!mbar_wait_bounded(&full_bar[st], st_ph, DEC_WAIT_LIMIT)) { failed = true; dsc.x = -1; return; }
       dsc = *reinterpret_cast<const int2*>(&desc[st]);
     };
     auto advance_slot = [&]() {
@@ -1023,14 +1054,17 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
           for (int half = 0; half < HN / 4; half++) {
             uint32_t o_u[16];
+            float ofs[4];
             tc_ld16_issue(tmem_g + lane_sel + L::I8_O_COL + 32 * j + 16 * half, o_u);
             tc_wait_ld();
 #pragma unroll
             for (int hq = 0; hq < 4; hq++) {
               const float of = fmaf(fmaf(fmaf(__int2float_rn((int)o_u[4 * hq + 3]), 256.f, __int2float_rn((int)o_u[4 * hq + 2])), 256.f,
                                          __int2float_rn((int)o_u[4 * hq + 1])), 256.f, __int2float_rn((int)o_u[4 * hq]));
-              acc[j][4 * half + hq] = fmaf(of, ofac, acc[j][4 * half + hq]);
+              ofs[hq] = of;
             }
+            acc[j][2 * half] = fma2(f32x2(ofs[0], ofs[1]), f32x2(ofac, ofac), acc[j][2 * half]);
+            acc[j][2 * half + 1] = fma2(f32x2(ofs[2], ofs[3]), f32x2(ofac, ofac), acc[j][2 * half + 1]);
           }
         tc_fence_before();
         nacc = 0;
@@ -1088,22 +1122,20 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
         const float ksc = load_scale(sp + L::K_BYTES + L::VT_BYTES, gt, p.scale_f16);
         const float vsc = load_scale(sp + L::K_BYTES + L::VT_BYTES + L::SC_BYTES, gt, p.scale_f16);
-        const bool valid = gt < n;  // rows >= n of the last block hold stale bytes
-        const float kfs = valid ? ksc * sfac : 0.f;
-        const float mask = valid ? 0.f : -INFINITY;  // stale rows: 0 * finite - inf = -inf
-        const float vf = valid ? vsc * vfac : 0.f;
+        const float kfs = ksc * sfac;
+        float vf = vsc * vfac;
 
-        // ---- scores: three int32 digit columns per head -> log2-domain score of row gt
-        if (!failed) failed = !mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
-        if (failed) break;
+        // ---- scores: three int32 digit columns per head -> log2-domain score of row gt, z = x kfs
+        if (!mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
         tc_fence_after();
-        float s[HN];
+        F32x2 x2[HN / 2], over[HN / 2];  // x: the score's digits put together; z - m_run
         {
-          auto digits_to_scores = [&](const uint32_t (&raw_u)[16], int half) {
+          auto digits = [&](const uint32_t (&raw_u)[16], int half) {
 #pragma unroll
-            for (int hq = 0; hq < 4; hq++) {  // S = (S0 + 128 S1) + 16384 S2: the lower two digits combine in an int32 (< 2^28)
-              const float lo = __int2float_rn((int)raw_u[4 * hq + 1] * 128 + (int)raw_u[4 * hq]);
-              s[4 * half + hq] = fmaf(fmaf(__int2float_rn((int)raw_u[4 * hq + 2]), 16384.f, lo), kfs, mask);
+            for (int hq = 0; hq < 2; hq++) {  // S = (S0 + 128 S1) + 16384 S2: the lower two digits combine in an int32 (< 2^28)
+              const uint32_t* a = raw_u + 8 * hq;
+              const F32x2 lo = f32x2(__int2float_rn((int)a[1] * 128 + (int)a[0]), __int2float_rn((int)a[5] * 128 + (int)a[4]));
+              x2[2 * half + hq] = fma2(f32x2(__int2float_rn((int)a[2]), __int2float_rn((int)a[6])), f32x2(16384.f, 16384.f), lo);
             }
           };
           uint32_t raw0[16];
@@ -1112,49 +1144,46 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           if constexpr (HN == 8) {
             uint32_t raw1[16];
             tc_ld16_issue(tmem_g + lane_sel + L::I8_S_COL + 16, raw1);  // heads 4..7 in flight while heads 0..3 are converted
-            digits_to_scores(raw0, 0);
+            digits(raw0, 0);
             tc_wait_ld();
-            digits_to_scores(raw1, 1);
+            digits(raw1, 1);
           } else {
-            digits_to_scores(raw0, 0);
+            digits(raw0, 0);
           }
+        }
+#pragma unroll
+        for (int h2 = 0; h2 < HN / 2; h2++) over[h2] = fma2(x2[h2], f32x2(kfs, kfs), neg_m[h2]);
+        const bool stale = gt >= n;  // rows >= n of a sequence's last block hold stale bytes
+        if (n < TB && stale) {
+          vf = 0.f;
+#pragma unroll
+          for (int h2 = 0; h2 < HN / 2; h2++) over[h2] = f32x2(-INFINITY, -INFINITY);
         }
         if (ARGMAX) {  // exact maximum seen by this thread and its row (a group sees the blocks of a segment in ascending order)
 #pragma unroll
-          for (int h = 0; h < HN; h++)
-            if (s[h] > best_v[h]) { best_v[h] = s[h]; best_i[h] = r0 + gt; }
+          for (int h = 0; h < HN; h++) {
+            const float z = of_head(x2, h) * kfs;
+            if (!stale && z > best_v[h]) { best_v[h] = z; best_i[h] = r0 + gt; }
+          }
         }
         // The running reference m_run is raised when a score exceeds it by more than DEC_MAX_SLACK_I8 log2 units, the
         // V-scale bound vref when a row exceeds it: both are rare after the first blocks (one barrier with an OR reduction
         // otherwise).
-        float over[HN];
-#pragma unroll
-        for (int h = 0; h < HN; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
-        const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 ||
-                            vf > vref || nacc >= 384;
-        
+        const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 || vf > vref || nacc >= 384;
+
         if (group_bar_or(bar_id, exceed)) {
           if (nacc > 0) flush();  // what TMEM holds is relative to the old references (the previous value MMAs have completed)
           {
             float s8[8];
-            pad8(s, -INFINITY, s8);
+#pragma unroll
+            for (int h = 0; h < 8; h++) s8[h] = h >= HN || stale ? -INFINITY : of_head(x2, h % HN) * kfs;
             const float wm = warp_reduce8(s8, lane, [](float x, float y) { return fmaxf(x, y); });
             if ((lane & 3) == 0) red[(warp & 3) * 8 + warp_reduce8_head(lane)] = wm;
           }
           const float wv_max = warp_max(vf);
           if (lane == 0) red2[warp & 3] = wv_max;
           group_bar_sync(bar_id);
-#pragma unroll
-          for (int h = 0; h < HN; h++) {
-            const float bm = fmaxf(fmaxf(red[h], red[8 + h]), fmaxf(red[16 + h], red[24 + h]));
-            const float mn = fmaxf(m_run[h], bm + DEC_RAISE_MARGIN);  // every head goes above its block maximum whichever head asked: fewer raises later
-            const float alpha = ex2f(m_run[h] - mn);  // the accumulator holds the blocks before this one: rescale it now
-            m_run[h] = mn;
-            l_run[h] *= alpha;
-#pragma unroll
-            for (int j = 0; j < DJ; j++) acc[j][h] *= alpha;
-            over[h] = s[h] - mn;
-          }
+          raise(x2, kfs, stale, over);
           const float bv = fmaxf(fmaxf(red2[0], red2[1]), fmaxf(red2[2], red2[3]));
           if (bv > vref) vref = __uint_as_float((__float_as_uint(bv) + 0x007FFFFFu) & 0x7F800000u);  // next power of two
           pscale = vref > 0.f ? (1073741824.0f / (float)(1 << IQ_SLACK_I8)) / vref : 0.f;  // p * vscale * pscale <= 2^30
@@ -1165,10 +1194,12 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           uint32_t pb[HN];
           const float vfp = vf * pscale;
 #pragma unroll
-          for (int h = 0; h < HN; h++) {
-            const float pr = ex2f(over[h]);
-            l_run[h] += pr;
-            pb[h] = __float2uint_rn(pr * vfp);
+          for (int h2 = 0; h2 < HN / 2; h2++) {
+            const F32x2 pr = f32x2(ex2f(over[h2].lo()), ex2f(over[h2].hi()));
+            l2[h2] = add2(l2[h2], pr);
+            const F32x2 w = mul2(pr, f32x2(vfp, vfp));
+            pb[2 * h2] = __float2uint_rn(w.lo());
+            pb[2 * h2 + 1] = __float2uint_rn(w.hi());
           }
           const int off = (gt & 7) * 16 + (gt >> 3) * 128;
           *reinterpret_cast<uint4*>(bp + off) = make_uint4(pb[0], pb[1], pb[2], pb[3]);
@@ -1179,8 +1210,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         nacc++;
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(p_ready);          // V tile in TMEM, probabilities in shared memory
-        mbar_arrive(&empty_bar[st]);   // this thread is done with the staged tile
+        mbar_arrive(p_ready);          // V tile in TMEM, probabilities in shared memory, staged tile consumed
 
         // ---- next slot: if it continues the segment, its K tile now, while the value MMAs run
         advance_slot();
@@ -1189,7 +1219,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if (more) k_tile(stages + st * L::STAGE_BYTES);
 
         // ---- the value MMAs of this block must have completed before its V tile and B_P are overwritten; their result stays in TMEM
-        if (!failed) failed = !mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
+        if (!mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
         nbk++;
       }
         if (failed) break;
@@ -1264,66 +1294,62 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         for (int j = 0; j < DJ; j++) { v_unit(j, 0); v_unit(j, 1); }
 
         // the score MMAs read the K tile that the rest of the V tile is about to overwrite
-        if (!failed) failed = !mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
-        if (failed) break;
+        if (!mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
         tc_fence_after();
         uint32_t raw_u[16];
         tc_ld16_issue(tmem_g + lane_sel + L::S_COL, raw_u);  // scores of row gt: in flight during the next unit
 #pragma unroll
         for (int j = 0; j < DJ; j++) v_unit(j, 2);
 
-        // ---- online softmax (log2 units); thread gt owns row r0 + gt, all 8 heads
+        // ---- online softmax (log2 units); thread gt owns row r0 + gt, all heads. x: the two terms of a score, z = x kf
         tc_wait_ld();
-        float s[HN];
-        {
-          const bool valid = gt < n;  // rows >= n of the last block hold stale bytes
-          const float kf = valid ? ksc * kfac : 0.f;
-          const float mask = valid ? 0.f : -INFINITY;  // stale rows: 0 * finite - inf = -inf
+        const float kf = ksc * kfac;
+        float vf = vsc * vfac;
+        const bool stale = gt >= n;  // rows >= n of a sequence's last block hold stale bytes
+        F32x2 x2[HN / 2], over[HN / 2];
 #pragma unroll
-          for (int h = 0; h < HN; h++) s[h] = fmaf(__uint_as_float(raw_u[h]) + __uint_as_float(raw_u[8 + h]), kf, mask);
+        for (int h2 = 0; h2 < HN / 2; h2++) {
+          x2[h2] = add2(f32x2(__uint_as_float(raw_u[2 * h2]), __uint_as_float(raw_u[2 * h2 + 1])),
+                        f32x2(__uint_as_float(raw_u[8 + 2 * h2]), __uint_as_float(raw_u[8 + 2 * h2 + 1])));
+          over[h2] = fma2(x2[h2], f32x2(kf, kf), neg_m[h2]);
+        }
+        if (n < TB && stale) {
+          vf = 0.f;
+#pragma unroll
+          for (int h2 = 0; h2 < HN / 2; h2++) over[h2] = f32x2(-INFINITY, -INFINITY);
         }
         if (ARGMAX) {  // exact maximum seen by this thread and its row (a group sees the blocks of a segment in ascending order)
 #pragma unroll
-          for (int h = 0; h < HN; h++)
-            if (s[h] > best_v[h]) { best_v[h] = s[h]; best_i[h] = r0 + gt; }
+          for (int h = 0; h < HN; h++) {
+            const float z = of_head(x2, h) * kf;
+            if (!stale && z > best_v[h]) { best_v[h] = z; best_i[h] = r0 + gt; }
+          }
         }
-        // The running reference m_run is raised only when some score of the block exceeds it by more than
-        // DEC_MAX_SLACK (log2 units): exp2(s - m_run) then stays below 2^DEC_MAX_SLACK and nothing has to be
-        // exchanged between the warps in the common case (one barrier with an OR reduction).
-        float over[HN];
-#pragma unroll
-        for (int h = 0; h < HN; h++) over[h] = s[h] - m_run[h];  // NaN (-inf - -inf) for a stale row of an unopened reference: max ignores it
-        const bool exceed = max_of(over) > DEC_MAX_SLACK;
-        if (group_bar_or(bar_id, exceed)) {
+        // The running reference is raised only when some score of the block exceeds it by more than DEC_MAX_SLACK (log2
+        // units): exp2(z - m) then stays below 2^DEC_MAX_SLACK and nothing has to be exchanged between the warps in the
+        // common case (one barrier with an OR reduction).
+        if (group_bar_or(bar_id, max_of(over) > DEC_MAX_SLACK)) {
           {
             float s8[8];
-            pad8(s, -INFINITY, s8);
+#pragma unroll
+            for (int h = 0; h < 8; h++) s8[h] = h >= HN || stale ? -INFINITY : of_head(x2, h % HN) * kf;
             const float wm = warp_reduce8(s8, lane, [](float x, float y) { return fmaxf(x, y); });
             if ((lane & 3) == 0) red[(warp & 3) * 8 + warp_reduce8_head(lane)] = wm;
           }
           group_bar_sync(bar_id);
-#pragma unroll
-          for (int h = 0; h < HN; h++) {
-            const float bm = fmaxf(fmaxf(red[h], red[8 + h]), fmaxf(red[16 + h], red[24 + h]));
-            const float mn = fmaxf(m_run[h], bm + DEC_RAISE_MARGIN);  // every head goes above its block maximum whichever head asked: fewer raises later
-            const float alpha = ex2f(m_run[h] - mn);  // the accumulator holds the blocks before this one: rescale it now
-            m_run[h] = mn;
-            l_run[h] *= alpha;
-#pragma unroll
-            for (int j = 0; j < DJ; j++) acc[j][h] *= alpha;
-            over[h] = s[h] - mn;
-          }
+          raise(x2, kf, stale, over);
         }
 #pragma unroll
         for (int j = 0; j < DJ; j++) v_unit(j, 3);  // the last V unit, next to the exponentials
         {
-          const float vf = (gt < n) ? vsc * vfac : 0.f;
           float wv[HN];
 #pragma unroll
-          for (int h = 0; h < HN; h++) {
-            const float pr = ex2f(over[h]);
-            l_run[h] += pr;
-            wv[h] = pr * vf;
+          for (int h2 = 0; h2 < HN / 2; h2++) {
+            const F32x2 pr = f32x2(ex2f(over[h2].lo()), ex2f(over[h2].hi()));
+            l2[h2] = add2(l2[h2], pr);
+            const F32x2 w = mul2(pr, f32x2(vf, vf));
+            wv[2 * h2] = w.lo();
+            wv[2 * h2 + 1] = w.hi();
           }
           // probabilities (times scale_V / sqrt(d)) as fp16 hi + lo: B_P[n][row], n = head (hi) or 8 + head (lo)
           uint32_t hp[4] = {0u, 0u, 0u, 0u}, lp[4] = {0u, 0u, 0u, 0u};
@@ -1341,8 +1367,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(p_ready);          // V tile in TMEM, probabilities in shared memory
-        mbar_arrive(&empty_bar[st]);   // this thread is done with the staged tile
+        mbar_arrive(p_ready);          // V tile in TMEM, probabilities in shared memory, staged tile consumed
 
         // ---- next slot: if it continues the segment, its K coordinates that live in the upper half of the operand
         // columns, while the value MMAs run
@@ -1357,15 +1382,14 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
 
         // ---- fold the value product into the running accumulator (the value MMAs also release the lower half)
-        if (!failed) failed = !mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
-        if (failed) break;
+        if (!mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < DJ; j++) {
           float o[16];
           tc_ld16(tmem_g + lane_sel + L::O_COL + 16 * j, o);
 #pragma unroll
-          for (int h = 0; h < HN; h++) acc[j][h] += o[h] + o[8 + h];
+          for (int h2 = 0; h2 < HN / 2; h2++) acc[j][h2] = add2(acc[j][h2], add2(f32x2(o[2 * h2], o[2 * h2 + 1]), f32x2(o[8 + 2 * h2], o[8 + 2 * h2 + 1])));
         }
         tc_fence_before();
         nbk++;
@@ -1382,7 +1406,6 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         close_segment();
       }
     }
-    if (!failed && dsc.x < 0) mbar_arrive(&empty_bar[st]);  // the end marker's slot
   }
 
   allow_dependent_launch();
