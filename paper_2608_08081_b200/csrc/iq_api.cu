@@ -496,7 +496,7 @@ static int decode_params(const iq_shape* shape, const float* rot_dev, const iq_c
     }
   }
   p.use_i8 = grid8 ? 1 : 0;
-  p.neg_zero = iq::NEG_ZERO_F16X2;
+  p.lookup = iq::LOOKUP_CONST;
   p.delta = delta;
   p.delta_v = delta_v;
   p.k_new = p.v_new = nullptr;

@@ -77,30 +77,44 @@ template <int N>
 constexpr uint32_t DEC_IDESC_I8_SU = (2u << 4) | (1u << 7) | (0u << 10) | (1u << 16) | (((uint32_t)N >> 3) << 17) | ((128u >> 4) << 24);
 
 // ---------------------------------------------------------------------------------------------- dequantisation
+// The shift/logic pipe, which carries the byte permutes at half rate, bounds the lookups, so what can go elsewhere does. A 128 x 128
+// tile of 3-bit codes, its loads and stores included, takes a scheduler 140 cycles (however many warps it has): 190 with the shifts
+// and masks on that pipe or as high words of products (which occupy the multiplier for four cycles each), 162 with only the upper
+// halves elsewhere.
 // The upper half of a word of nibbles below 8 in the lower half, for the byte permutes, which take their selectors from there: an
 // fp16x2 addition of -0 that reads the upper half twice. Exact: no such half is an infinity or a NaN (bit 11 is clear), and
-// subnormals are kept. The shift/logic pipe, which carries the permutes and the masks at half rate, bounds the lookups, the
-// fp16 addition runs beside it: 163 cycles of a scheduler for a 128 x 128 tile of 3-bit codes (with its loads and stores), where
-// shifts take 190, and so do high words of products, which occupy the multiplier for four cycles each.
-__device__ __forceinline__ uint32_t upper_nibbles(uint32_t x, uint32_t neg_zero) {
+// subnormals are kept.
+__device__ __forceinline__ uint32_t upper_nibbles(uint32_t x, LookupConst c) {
   uint32_t r;
-  asm("{\n\t.reg .b16 l, h;\n\t.reg .b32 t;\n\tmov.b32 {l, h}, %1;\n\tmov.b32 t, {h, h};\n\tadd.f16x2 %0, t, %2;\n\t}" : "=r"(r) : "r"(x), "r"(neg_zero));
+  asm("{\n\t.reg .b16 l, h;\n\t.reg .b32 t;\n\tmov.b32 {l, h}, %1;\n\tmov.b32 t, {h, h};\n\tadd.f16x2 %0, t, %2;\n\t}" : "=r"(r) : "r"(x), "r"(c.neg_zero));
   return r;
 }
-// Selectors of the 8 entries whose code bits sit in bit 3 of the nibbles of the unit's three words.
-__device__ __forceinline__ uint32_t sliced_selectors(uint32_t w0, uint32_t w1, uint32_t w2) {
-  return ((w0 >> 3) & 0x11111111u) | ((w1 >> 2) & 0x22222222u) | ((w2 >> 1) & 0x44444444u);
+// w without the bits of `part` (part = w & mask), by a multiply-add.
+__device__ __forceinline__ uint32_t without(uint32_t w, uint32_t part, LookupConst c) {
+  uint32_t r;
+  asm("mad.lo.u32 %0, %1, %2, %3;" : "=r"(r) : "r"(part), "r"(c.minus_one), "r"(w));
+  return r;
+}
+// The selectors of one packing unit's 32 entries (3 bits), 8 to a word: the low three bits of the nibbles, and for the last 8, whose
+// code bits sit in bit 3 of the nibbles of the three words, these put together.
+__device__ __forceinline__ void unit_selectors(uint32_t w0, uint32_t w1, uint32_t w2, LookupConst c, uint32_t (&sel)[4]) {
+  const uint32_t g0 = w0 & 0x88888888u, g1 = w1 & 0x88888888u, g2 = w2 & 0x88888888u;
+  sel[0] = without(w0, g0, c);
+  sel[1] = without(w1, g1, c);
+  sel[2] = without(w2, g2, c);
+  sel[3] = (g0 >> 3) | (g1 >> 2) | (g2 >> 1);
 }
 // One packing unit (32 codes in 3 words) -> 16 registers of two fp16 levels each, entries in natural order:
 // out[r] = (level[code 2r], level[code 2r+1]). Byte lookups with prmt: 8 levels x (low byte, high byte).
 __device__ __forceinline__ void dequant_unit(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t lo0, uint32_t lo1, uint32_t hi0,
-                                             uint32_t hi1, uint32_t neg_zero, uint32_t (&out)[16]) {
-  const uint32_t sel[4] = {w0 & 0x77777777u, w1 & 0x77777777u, w2 & 0x77777777u, sliced_selectors(w0, w1, w2)};
+                                             uint32_t hi1, LookupConst c, uint32_t (&out)[16]) {
+  uint32_t sel[4];
+  unit_selectors(w0, w1, w2, c, sel);
 #pragma unroll
   for (int k = 0; k < 4; k++)
 #pragma unroll
     for (int hh = 0; hh < 2; hh++) {
-      const uint32_t x = hh ? upper_nibbles(sel[k], neg_zero) : sel[k];
+      const uint32_t x = hh ? upper_nibbles(sel[k], c) : sel[k];
       const uint32_t l = prmt(lo0, lo1, x), h = prmt(hi0, hi1, x);
       out[4 * k + 2 * hh] = prmt(l, h, 0x5140u);
       out[4 * k + 2 * hh + 1] = prmt(l, h, 0x7362u);
@@ -108,12 +122,13 @@ __device__ __forceinline__ void dequant_unit(uint32_t w0, uint32_t w1, uint32_t 
 }
 
 // Integer path: one packing unit -> 8 registers of four int8 levels each, entries in natural order (one prmt per 4 codes).
-__device__ __forceinline__ void dequant_unit8(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t l0, uint32_t l1, uint32_t neg_zero, uint32_t* out) {
-  const uint32_t sel[4] = {w0 & 0x77777777u, w1 & 0x77777777u, w2 & 0x77777777u, sliced_selectors(w0, w1, w2)};
+__device__ __forceinline__ void dequant_unit8(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t l0, uint32_t l1, LookupConst c, uint32_t* out) {
+  uint32_t sel[4];
+  unit_selectors(w0, w1, w2, c, sel);
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     out[2 * k] = prmt(l0, l1, sel[k]);
-    out[2 * k + 1] = prmt(l0, l1, upper_nibbles(sel[k], neg_zero));
+    out[2 * k + 1] = prmt(l0, l1, upper_nibbles(sel[k], c));
   }
 }
 // ---- the same for every bit width: 32 consecutive entries of a packed run (BITS words at w) -> natural order.
@@ -123,25 +138,25 @@ __device__ __forceinline__ void dequant_unit8(uint32_t w0, uint32_t w1, uint32_t
 __device__ __forceinline__ uint32_t byte_select(uint32_t lo, uint32_t hi, uint32_t mask) { return (hi & mask) | (lo & ~mask); }
 
 template <int BITS>
-__device__ __forceinline__ void dequant32_i8(const uint32_t* w, const uint32_t (&t)[4], uint32_t neg_zero, uint32_t* out) {
+__device__ __forceinline__ void dequant32_i8(const uint32_t* w, const uint32_t (&t)[4], LookupConst c, uint32_t* out) {
   if constexpr (BITS == 3) {
-    dequant_unit8(w[0], w[1], w[2], t[0], t[1], neg_zero, out);
+    dequant_unit8(w[0], w[1], w[2], t[0], t[1], c, out);
   } else if constexpr (BITS == 2) {
 #pragma unroll
     for (int j = 0; j < 2; j++) {
-      const uint32_t a = w[j] & 0x33333333u, b = (w[j] >> 2) & 0x33333333u;
+      const uint32_t g = w[j] & 0xCCCCCCCCu, a = without(w[j], g, c), b = g >> 2;
       out[4 * j] = prmt(t[0], t[0], a);
-      out[4 * j + 1] = prmt(t[0], t[0], upper_nibbles(a, neg_zero));
+      out[4 * j + 1] = prmt(t[0], t[0], upper_nibbles(a, c));
       out[4 * j + 2] = prmt(t[0], t[0], b);
-      out[4 * j + 3] = prmt(t[0], t[0], upper_nibbles(b, neg_zero));
+      out[4 * j + 3] = prmt(t[0], t[0], upper_nibbles(b, c));
     }
   } else {
 #pragma unroll
     for (int j = 0; j < 4; j++) {
-      const uint32_t s7 = w[j] & 0x77777777u, s3 = (w[j] >> 3) & 0x11111111u;
+      const uint32_t g = w[j] & 0x88888888u, s7 = without(w[j], g, c), s3 = g >> 3;
 #pragma unroll
       for (int hh = 0; hh < 2; hh++) {
-        const uint32_t x = hh ? upper_nibbles(s7, neg_zero) : s7, mx = hh ? upper_nibbles(s3, neg_zero) : s3;
+        const uint32_t x = hh ? upper_nibbles(s7, c) : s7, mx = hh ? upper_nibbles(s3, c) : s3;
         out[2 * j + hh] = byte_select(prmt(t[0], t[1], x), prmt(t[2], t[3], x), prmt(0x0000FF00u, 0u, mx));
       }
     }
@@ -150,30 +165,31 @@ __device__ __forceinline__ void dequant32_i8(const uint32_t* w, const uint32_t (
 
 // fp16 levels: out[r] = (level[code 2r], level[code 2r+1]), 16 registers for the 32 entries.
 template <int BITS>
-__device__ __forceinline__ void dequant32_f16(const uint32_t* w, const uint32_t (&lo)[4], const uint32_t (&hi)[4], uint32_t neg_zero, uint32_t (&out)[16]) {
+__device__ __forceinline__ void dequant32_f16(const uint32_t* w, const uint32_t (&lo)[4], const uint32_t (&hi)[4], LookupConst c, uint32_t (&out)[16]) {
   if constexpr (BITS == 3) {
-    dequant_unit(w[0], w[1], w[2], lo[0], lo[1], hi[0], hi[1], neg_zero, out);
+    dequant_unit(w[0], w[1], w[2], lo[0], lo[1], hi[0], hi[1], c, out);
   } else {
     uint32_t sel[4], top[4];  // four selectors of 8 entries each (b = 4: and the top bits of their codes)
     if constexpr (BITS == 2) {
-      sel[0] = w[0] & 0x33333333u; sel[1] = (w[0] >> 2) & 0x33333333u;
-      sel[2] = w[1] & 0x33333333u; sel[3] = (w[1] >> 2) & 0x33333333u;
+      const uint32_t g0 = w[0] & 0xCCCCCCCCu, g1 = w[1] & 0xCCCCCCCCu;
+      sel[0] = without(w[0], g0, c); sel[1] = g0 >> 2;
+      sel[2] = without(w[1], g1, c); sel[3] = g1 >> 2;
       top[0] = top[1] = top[2] = top[3] = 0u;
     } else {
 #pragma unroll
-      for (int k = 0; k < 4; k++) { sel[k] = w[k] & 0x77777777u; top[k] = (w[k] >> 3) & 0x11111111u; }
+      for (int k = 0; k < 4; k++) { const uint32_t g = w[k] & 0x88888888u; sel[k] = without(w[k], g, c); top[k] = g >> 3; }
     }
 #pragma unroll
     for (int k = 0; k < 4; k++)
 #pragma unroll
       for (int hh = 0; hh < 2; hh++) {
-        const uint32_t x = hh ? upper_nibbles(sel[k], neg_zero) : sel[k];
+        const uint32_t x = hh ? upper_nibbles(sel[k], c) : sel[k];
         uint32_t l, h;
         if constexpr (BITS == 2) {
           l = prmt(lo[0], lo[0], x);
           h = prmt(hi[0], hi[0], x);
         } else {
-          const uint32_t m = prmt(0x0000FF00u, 0u, hh ? upper_nibbles(top[k], neg_zero) : top[k]);
+          const uint32_t m = prmt(0x0000FF00u, 0u, hh ? upper_nibbles(top[k], c) : top[k]);
           l = byte_select(prmt(lo[0], lo[1], x), prmt(lo[2], lo[3], x), m);
           h = byte_select(prmt(hi[0], hi[1], x), prmt(hi[2], hi[3], x), m);
         }

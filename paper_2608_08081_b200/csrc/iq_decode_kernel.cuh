@@ -1089,8 +1089,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
         for (int u = 0; u < 4 * DJ; u += 2) {  // twice 32 coordinates per TMEM store
           uint32_t f[16];
-          dequant32_i8<BITS>(kw + BITS * u, lk8, p.neg_zero, f);
-          dequant32_i8<BITS>(kw + BITS * (u + 1), lk8, p.neg_zero, f + 8);
+          dequant32_i8<BITS>(kw + BITS * u, lk8, p.lookup, f);
+          dequant32_i8<BITS>(kw + BITS * (u + 1), lk8, p.lookup, f + 8);
           tc_st16(tmem_g + lane_sel + L::I8_K_COL + 8 * u, f);
         }
         tc_wait_st();
@@ -1124,8 +1124,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 #pragma unroll
           for (int u = 0; u < 4; u += 2) {  // twice 32 rows per TMEM store
             uint32_t f[16];
-            dequant32_i8<BITS>(wd + BITS * u, lv8, p.neg_zero, f);
-            dequant32_i8<BITS>(wd + BITS * (u + 1), lv8, p.neg_zero, f + 8);
+            dequant32_i8<BITS>(wd + BITS * u, lv8, p.lookup, f);
+            dequant32_i8<BITS>(wd + BITS * (u + 1), lv8, p.lookup, f + 8);
             tc_st16(tmem_g + lane_sel + L::I8_V_COL + 32 * j + 8 * u, f);
           }
         }
@@ -1261,7 +1261,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       };
       auto k_unit = [&](int u) {
         uint32_t f[16];
-        dequant32_f16<BITS>(kw + BITS * u, lk_lo, lk_hi, p.neg_zero, f);
+        dequant32_f16<BITS>(kw + BITS * u, lk_lo, lk_hi, p.lookup, f);
         tc_st16(tmem_g + lane_sel + L::A_COL + 16 * u, f);
       };
 #pragma unroll 1
@@ -1295,7 +1295,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         const float vsc = load_scale(sp + L::K_BYTES + L::VT_BYTES + L::SC_BYTES, gt, p.scale_f16);
         auto v_unit = [&](int j, int u) {  // rows 32u .. 32u+31 of coordinate gt + 128 j
           uint32_t f[16];
-          dequant32_f16<BITS>(wd[j] + BITS * u, lv_lo, lv_hi, p.neg_zero, f);
+          dequant32_f16<BITS>(wd[j] + BITS * u, lv_lo, lv_hi, p.lookup, f);
           const uint32_t col = (u < 2) ? (uint32_t)(L::V_COL + 32 * j + 16 * u) : (uint32_t)(L::A_COL + 64 * j + 16 * (u - 2));
           tc_st16(tmem_g + lane_sel + col, f);
         };

@@ -77,7 +77,10 @@ cudaError_t launch_wht_coordinates(const WhtParams& p, int head_dim, int batch, 
 
 // ---- fused decode
 constexpr int DEC_BLOCK_TOKENS = 128;  // cached rows per block of the decode kernel = rows of one transposed V block
-constexpr uint32_t NEG_ZERO_F16X2 = 0x80008000u;  // passed to the kernels as a parameter: an addition of a constant -0 would be dropped by the compiler
+// Constants of the lookups (iq_decode_common.cuh) that the kernels take as parameters: an addition of -0 or a product with -1 that the
+// compiler sees as such becomes the logic that it is there to avoid.
+struct LookupConst { uint32_t neg_zero, minus_one; };
+constexpr LookupConst LOOKUP_CONST = {0x80008000u, 0xFFFFFFFFu};
 constexpr int DEC_HEADS = 8;          // query heads of one KV head that a work item covers (they share the N columns of one MMA)
 
 struct DecodeParams {
@@ -103,7 +106,7 @@ struct DecodeParams {
   uint32_t lut8[4], lut8_v[4];
   float delta, delta_v;
   int use_i8;
-  uint32_t neg_zero;  // NEG_ZERO_F16X2
+  LookupConst lookup;
   // Decode with append (k_new != nullptr; otherwise none of the following is read): the step's new K and V rows
   // [batch][n_kv_heads][head_dim] are quantised and appended at row seq_lens[b] by one warp per (sequence, KV head),
   // which also writes the new row's own partial (new_acc [batch][n_q_heads][head_dim], new_ml [batch][n_q_heads][2]);

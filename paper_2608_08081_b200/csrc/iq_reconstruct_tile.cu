@@ -36,7 +36,7 @@ struct ReconstructTileParams {
   int batch;
   uint32_t lo[2][3][4], hi[2][3][4];  // K and V: low / high bytes of the binary16 operand values of each pass (4 per register)
   int passes[2];                      // 1: the values with both terms of W; 3: with the lower, the upper, the upper term
-  uint32_t neg_zero;                  // upper_nibbles
+  LookupConst lookup;
   float factor[2];                    // level = factor * the value of the one pass, or the values of the two that meet the upper term
 };
 
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(ReconLayout<D>::THREADS, 1) reconstruct_tile_k
 #pragma unroll
         for (int u = 0; u < UPH; u++) {  // 32 entries -> four 16-byte pieces of the operand
           uint32_t lv[16];
-          dequant32_f16<BITS>(words + hf * WPH + BITS * u, l_lo, l_hi, q.neg_zero, lv);
+          dequant32_f16<BITS>(words + hf * WPH + BITS * u, l_lo, l_hi, q.lookup, lv);
 #pragma unroll
           for (int k = 0; k < 4; k++) {
             const int c = part * (16 / NJ) + 4 * u + k;  // piece: 8 coordinates of the row (K), 8 rows of the coordinate (V)
@@ -390,7 +390,7 @@ bool launch_reconstruct_tiles(const ReconstructParams& p, int head_dim, int batc
   ReconstructTileParams q;
   q.r = p;
   q.batch = batch;
-  q.neg_zero = NEG_ZERO_F16X2;
+  q.lookup = LOOKUP_CONST;
   if (!operand_levels(p.levels_k, 1 << p.bits, q.lo[0], q.hi[0], q.passes[0], q.factor[0])) return false;
   if (!operand_levels(p.levels_v, 1 << p.bits, q.lo[1], q.hi[1], q.passes[1], q.factor[1])) return false;
   e = q.passes[0] + q.passes[1] > 2 ? launch_bits<true>(q, head_dim, stream) : launch_bits<false>(q, head_dim, stream);
