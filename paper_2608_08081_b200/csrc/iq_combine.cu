@@ -5,22 +5,24 @@
 
 namespace iq {
 
-constexpr int CMB_WARPS = 4;
+constexpr int CMB_WARPS = 8;
 
-// WPH = 1: one warp per (sequence, query head), CMB_WARPS heads per CTA. WPH > 1 (many slots): one CTA of WPH warps
-// per head; warp w merges slots w, w + WPH, ... and warp 0 merges the warps' results. Lane l owns rotated
-// coordinates l*E .. l*E+E-1, i.e. whole SO(4) blocks, so M_b^T is applied in registers and H_d by the warp butterfly.
+// CTAs of 8 warps, WPH of them to a (sequence, query head): warp w of a head merges a run of consecutive slots, warp 0 of the head the
+// warps' results. Lane l owns rotated coordinates l*E .. l*E+E-1, i.e. whole SO(4) blocks, so M_b^T is applied in registers and
+// H_d by the warp butterfly. Bound by latency: a launch is a few KB per warp. So the acc rows of a warp's first 8 slots are
+// requested together with their (m, l), whether they turn out to be in use or not.
 template <int D, int WPH>
-__global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_kernel(const CombineParams p) {
-  constexpr int E = D / 32;
+__global__ void __launch_bounds__(CMB_WARPS * 32) combine_kernel(const CombineParams p) {
+  constexpr int E = D / 32, HPC = CMB_WARPS / WPH;
   grid_dependency_wait();
   allow_dependent_launch();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int bh = WPH == 1 ? blockIdx.x * CMB_WARPS + warp : blockIdx.x;
-  if (bh >= p.batch * p.n_q_heads) return;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % WPH, hc = (threadIdx.x >> 5) / WPH;
+  const int bh = blockIdx.x * HPC + hc;
+  const bool present = bh < p.batch * p.n_q_heads;
+  if (WPH == 1 && !present) return;
   const int h = bh % p.n_q_heads;
   const int kvh = h / (p.n_q_heads / p.n_kv_heads);
-  const int S1 = p.splits, S = p.splits * p.shards;  // slots of one shard, of all shards
+  const int S1 = p.splits, S = present ? p.splits * p.shards : 0;  // slots of one shard, of all shards
   const size_t shard_heads = (size_t)p.batch * p.n_q_heads;
   // slot s of this head: shard s / S1, its slot s % S1 (one shard: s itself)
   auto slot_index = [&](int s) { return p.shards == 1 ? (size_t)bh * S1 + s : ((size_t)(s / S1) * shard_heads + bh) * S1 + (s % S1); };
@@ -29,11 +31,20 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
     if (idx >= 0 && p.row_offsets) idx += p.row_offsets[(size_t)(s / S1) * p.batch + bh / p.n_q_heads];
     return idx;
   };
-  const int s0 = WPH == 1 ? 0 : warp;
 
-  // the rotation block of this lane first: its loads do not depend on the partials and overlap with theirs
+  // the rotation block of this lane and the partial of the step's new row first: their loads overlap with those of the slots
   QuatPairs<E> qp;
-  if (WPH == 1 || warp == 0) qp.load(p.rot + (size_t)kvh * (D / 4) * 8, lane);
+  float mn = -INFINITY, ln = 0.f;
+  float4 vn[E / 4];
+  if (warp == 0 && present) {
+    qp.load(p.rot + (size_t)kvh * (D / 4) * 8, lane);
+    if (p.new_ml) {
+      mn = p.new_ml[2 * (size_t)bh];
+      ln = p.new_ml[2 * (size_t)bh + 1];
+#pragma unroll
+      for (int e4 = 0; e4 < E / 4; e4++) vn[e4] = *reinterpret_cast<const float4*>(p.new_acc + (size_t)bh * D + lane * E + 4 * e4);
+    }
+  }
 
   float m = -INFINITY;
   int best = -1;
@@ -41,13 +52,15 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
   float v[E];
 #pragma unroll
   for (int e = 0; e < E; e++) v[e] = 0.f;
-  // The warp's run of slots: all of them (WPH = 1), else an equal share of consecutive slots.
-  const int chunk = WPH == 1 ? S : (S + WPH - 1) / WPH;
-  const int c0 = WPH == 1 ? 0 : warp * chunk;
+  // The warp's run of slots: an equal share of consecutive ones.
+  const int chunk = (S + WPH - 1) / WPH;
+  const int c0 = warp * chunk;
   const int cn = max(0, min(chunk, S - c0));
   if (chunk <= 32) {
     // at most 32 slots per warp: lane j takes (m, l, argmax) of slot c0 + j, the reference and the weights come from warp
-    // reductions, and the acc rows are then loaded eight at a time (their addresses do not depend on one another)
+    // reductions, and the acc rows are loaded eight at a time (their addresses do not depend on one another)
+    constexpr int NF = 8;  // rows in flight
+    float4 f[NF][E / 4];
     float ms = -INFINITY, ls = 0.f;
     int idx = -1;
     size_t o = 0;
@@ -55,9 +68,19 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
       o = slot_index(c0 + lane);
       ms = p.part_ml[2 * o];
       ls = p.part_ml[2 * o + 1];
-      if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
-      else ms = -INFINITY;
     }
+    auto load_rows = [&](int sb) {
+#pragma unroll
+      for (int k = 0; k < NF; k++) {
+        const size_t ok = __shfl_sync(FULL, o, (sb + k) & 31);
+#pragma unroll
+        for (int e4 = 0; e4 < E / 4; e4++)
+          f[k][e4] = sb + k < cn ? *reinterpret_cast<const float4*>(p.part_acc + ok * D + lane * E + 4 * e4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    load_rows(0);
+    if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
+    else ms = -INFINITY;
     m = ms;
     best = idx;
 #pragma unroll
@@ -71,58 +94,53 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
     l = ls * w;
 #pragma unroll
     for (int d2 = 16; d2 > 0; d2 >>= 1) l += __shfl_xor_sync(FULL, l, d2);
-    constexpr int NF = 8;  // rows in flight
     for (int sb = 0; sb < cn; sb += NF) {
-      float4 f[NF][E / 4];
-      float ws[NF];
+      if (sb > 0) load_rows(sb);
 #pragma unroll
       for (int k = 0; k < NF; k++) {
-        ws[k] = __shfl_sync(FULL, w, (sb + k) & 31);
-        const size_t ok = __shfl_sync(FULL, o, (sb + k) & 31);
-        if (sb + k >= cn) ws[k] = 0.f;
-#pragma unroll
-        for (int e4 = 0; e4 < E / 4; e4++)
-          f[k][e4] = ws[k] != 0.f ? *reinterpret_cast<const float4*>(p.part_acc + ok * D + lane * E + 4 * e4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-#pragma unroll
-      for (int k = 0; k < NF; k++)
+        const float ws = __shfl_sync(FULL, w, (sb + k) & 31);
+        if (sb + k >= cn || ws == 0.f) continue;  // (the row of a slot that is not in use holds anything)
 #pragma unroll
         for (int e4 = 0; e4 < E / 4; e4++) {
-          v[4 * e4] += ws[k] * f[k][e4].x; v[4 * e4 + 1] += ws[k] * f[k][e4].y; v[4 * e4 + 2] += ws[k] * f[k][e4].z; v[4 * e4 + 3] += ws[k] * f[k][e4].w;
+          v[4 * e4] += ws * f[k][e4].x; v[4 * e4 + 1] += ws * f[k][e4].y; v[4 * e4 + 2] += ws * f[k][e4].z; v[4 * e4 + 3] += ws * f[k][e4].w;
         }
+      }
     }
   } else {
-  for (int s = s0; s < S; s += WPH) {
-    const size_t o = slot_index(s);
-    const float ms = p.part_ml[2 * o], ls = p.part_ml[2 * o + 1];
-    if (!(ls > 0.f)) continue;
-    const int idx = slot_argmax(s, o);
-    if (ms > m) { m = ms; best = idx; }
-    else if (ms == m && idx >= 0 && (best < 0 || idx < best)) best = idx;
-  }
-  for (int s = s0; s < S; s += WPH) {
-    const size_t o = slot_index(s);
-    const float ms = p.part_ml[2 * o], ls = p.part_ml[2 * o + 1];
-    if (!(ls > 0.f)) continue;
-    const float w = __expf(ms - m);
-    l += ls * w;
-    const float* a = p.part_acc + o * D + lane * E;
+    for (int s = c0; s < c0 + cn; s++) {
+      const size_t o = slot_index(s);
+      const float ms = p.part_ml[2 * o], ls = p.part_ml[2 * o + 1];
+      if (!(ls > 0.f)) continue;
+      const int idx = slot_argmax(s, o);
+      if (ms > m) { m = ms; best = idx; }
+      else if (ms == m && idx >= 0 && (best < 0 || idx < best)) best = idx;
+    }
+    for (int s = c0; s < c0 + cn; s++) {
+      const size_t o = slot_index(s);
+      const float ms = p.part_ml[2 * o], ls = p.part_ml[2 * o + 1];
+      if (!(ls > 0.f)) continue;
+      const float w = __expf(ms - m);
+      l += ls * w;
+      const float* a = p.part_acc + o * D + lane * E;
 #pragma unroll
-    for (int e4 = 0; e4 < E; e4 += 4) {
-      const float4 f = *reinterpret_cast<const float4*>(a + e4);
-      v[e4] += w * f.x; v[e4 + 1] += w * f.y; v[e4 + 2] += w * f.z; v[e4 + 3] += w * f.w;
+      for (int e4 = 0; e4 < E; e4 += 4) {
+        const float4 f = *reinterpret_cast<const float4*>(a + e4);
+        v[e4] += w * f.x; v[e4 + 1] += w * f.y; v[e4 + 2] += w * f.z; v[e4 + 3] += w * f.w;
+      }
     }
   }
-  }
   if constexpr (WPH > 1) {  // the warps' results (relative to their own maxima) merged by warp 0
-    __shared__ float sv[WPH][D];
-    __shared__ float sm[WPH], sl[WPH];
-    __shared__ int sb[WPH];
+    __shared__ float sv_s[HPC][WPH][D];
+    __shared__ float sm_s[HPC][WPH], sl_s[HPC][WPH];
+    __shared__ int sb_s[HPC][WPH];
+    float (&sv)[WPH][D] = sv_s[hc];
+    float (&sm)[WPH] = sm_s[hc], (&sl)[WPH] = sl_s[hc];
+    int (&sb)[WPH] = sb_s[hc];
 #pragma unroll
     for (int e = 0; e < E; e++) sv[warp][lane * E + e] = v[e];
     if (lane == 0) { sm[warp] = m; sl[warp] = l; sb[warp] = best; }
     __syncthreads();
-    if (warp != 0) return;
+    if (warp != 0 || !present) return;
     m = -INFINITY;
     best = -1;
     for (int w2 = 0; w2 < WPH; w2++) {
@@ -142,15 +160,13 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
     }
   }
   if (p.new_ml) {  // the step's new row: one more slot (its row index is the highest of the sequence: it wins no tie)
-    const float mn = p.new_ml[2 * (size_t)bh], ln = p.new_ml[2 * (size_t)bh + 1];
     if (ln > 0.f) {
       const bool had = l > 0.f;
       const float m2 = had ? fmaxf(m, mn) : mn;
       const float wa = had ? __expf(m - m2) : 0.f, wn = __expf(mn - m2);
-      const float4* a = reinterpret_cast<const float4*>(p.new_acc + (size_t)bh * D + lane * E);
 #pragma unroll
       for (int e4 = 0; e4 < E / 4; e4++) {
-        const float4 f = a[e4];
+        const float4 f = vn[e4];
         v[4 * e4] = fmaf(wn, f.x, wa * v[4 * e4]);
         v[4 * e4 + 1] = fmaf(wn, f.y, wa * v[4 * e4 + 1]);
         v[4 * e4 + 2] = fmaf(wn, f.z, wa * v[4 * e4 + 2]);
@@ -188,19 +204,24 @@ __global__ void __launch_bounds__(WPH == 1 ? CMB_WARPS * 32 : WPH * 32) combine_
   }
 }
 
-constexpr int CMB_WIDE = 8;  // warps per head when there are many slots
+template <int D>
+static cudaError_t launch_combine(const CombineParams& p, cudaStream_t stream) {
+  const long long n = (long long)p.batch * p.n_q_heads, slots = (long long)p.splits * p.shards;
+  auto go = [&](void (*kernel)(CombineParams), int wph) {
+    return launch_after_predecessor(kernel, dim3((unsigned)((n * wph + CMB_WARPS - 1) / CMB_WARPS)), dim3(CMB_WARPS * 32), 0, stream, p);
+  };
+  // Warps per head: eight slots to a warp, whose rows it has in flight at once. Against one warp for up to 16 slots and eight for
+  // more, and rows requested once the weights are known: 16 layers of one 32 K sequence (116 slots) 296 -> 283 us, a step over
+  // 8 x 4 K rows (20 slots) 26.1 -> 25.1, over 32 x 32 K (8 slots) 161 -> 159.
+  if (slots <= 8) return go(combine_kernel<D, 1>, 1);
+  if (slots <= 16) return go(combine_kernel<D, 2>, 2);
+  if (slots <= 32) return go(combine_kernel<D, 4>, 4);
+  return go(combine_kernel<D, 8>, 8);
+}
 
 cudaError_t launch_combine_splits(const CombineParams& p, int head_dim, cudaStream_t stream) {
-  const int n = p.batch * p.n_q_heads;
-  if (n <= 0) return cudaSuccess;
-  if (p.splits * p.shards > 16) {  // many slots per head (small batches cut into many pieces): the slots of a head spread over a CTA
-    dim3 grid(n), block(CMB_WIDE * 32);
-    if (head_dim == 128) return launch_after_predecessor(combine_kernel<128, CMB_WIDE>, grid, block, 0, stream, p);
-    return launch_after_predecessor(combine_kernel<256, CMB_WIDE>, grid, block, 0, stream, p);
-  }
-  dim3 grid((n + CMB_WARPS - 1) / CMB_WARPS), block(CMB_WARPS * 32);
-  if (head_dim == 128) return launch_after_predecessor(combine_kernel<128, 1>, grid, block, 0, stream, p);
-  return launch_after_predecessor(combine_kernel<256, 1>, grid, block, 0, stream, p);
+  if ((long long)p.batch * p.n_q_heads <= 0) return cudaSuccess;
+  return head_dim == 128 ? launch_combine<128>(p, stream) : launch_combine<256>(p, stream);
 }
 
 // ------------------------------------------------------------------------------------------------
