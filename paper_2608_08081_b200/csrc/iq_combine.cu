@@ -5,15 +5,17 @@
 
 namespace iq {
 
-constexpr int CMB_WARPS = 8;
+template <int WPH>
+constexpr int CMB_WARPS = WPH == 1 ? 4 : 8;  // warps per CTA
 
-// CTAs of 8 warps, WPH of them to a (sequence, query head): warp w of a head merges a run of consecutive slots, warp 0 of the head the
-// warps' results. Lane l owns rotated coordinates l*E .. l*E+E-1, i.e. whole SO(4) blocks, so M_b^T is applied in registers and
-// H_d by the warp butterfly. Bound by latency: a launch is a few KB per warp. So the acc rows of a warp's first 8 slots are
-// requested together with their (m, l), whether they turn out to be in use or not.
+// WPH warps to a (sequence, query head): warp w of a head merges a run of consecutive slots, warp 0 of the head the warps' results.
+// Lane l owns rotated coordinates l*E .. l*E+E-1, i.e. whole SO(4) blocks, so M_b^T is applied in registers and H_d by the warp
+// butterfly. Bound by latency while the heads are few, by the rows of the slots in use when they are many: eight of them are in
+// flight per warp, rows of other slots are not read. (CTAs per SM are stated so that the compiler takes the registers for eight
+// rows: left alone it takes 48 or 64 and loads fewer at a time, 16 layers of one 32 K sequence 299 us instead of 280.)
 template <int D, int WPH>
-__global__ void __launch_bounds__(CMB_WARPS * 32) combine_kernel(const CombineParams p) {
-  constexpr int E = D / 32, HPC = CMB_WARPS / WPH;
+__global__ void __launch_bounds__(CMB_WARPS<WPH> * 32, D == 128 && WPH > 1 ? 3 : 2) combine_kernel(const CombineParams p) {
+  constexpr int E = D / 32, HPC = CMB_WARPS<WPH> / WPH;
   grid_dependency_wait();
   allow_dependent_launch();
   const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % WPH, hc = (threadIdx.x >> 5) / WPH;
@@ -58,9 +60,8 @@ __global__ void __launch_bounds__(CMB_WARPS * 32) combine_kernel(const CombinePa
   const int cn = max(0, min(chunk, S - c0));
   if (chunk <= 32) {
     // at most 32 slots per warp: lane j takes (m, l, argmax) of slot c0 + j, the reference and the weights come from warp
-    // reductions, and the acc rows are loaded eight at a time (their addresses do not depend on one another)
-    constexpr int NF = 8;  // rows in flight
-    float4 f[NF][E / 4];
+    // reductions, and the acc rows of the slots in use are loaded eight at a time (their addresses do not depend on one another),
+    // the first eight while the weights are made
     float ms = -INFINITY, ls = 0.f;
     int idx = -1;
     size_t o = 0;
@@ -68,19 +69,28 @@ __global__ void __launch_bounds__(CMB_WARPS * 32) combine_kernel(const CombinePa
       o = slot_index(c0 + lane);
       ms = p.part_ml[2 * o];
       ls = p.part_ml[2 * o + 1];
+      if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
+      else ms = -INFINITY;
     }
-    auto load_rows = [&](int sb) {
+    constexpr int NF = 8;  // rows in flight
+    float4 f[NF][E / 4];
+    int from[NF];  // the lane that holds the row's slot
+    uint32_t todo = __ballot_sync(FULL, ls > 0.f);
+    int n_rows = 0;
+    auto request = [&]() {
+      n_rows = min(NF, __popc(todo));
+      const int j0 = __ffs(todo) - 1;
 #pragma unroll
       for (int k = 0; k < NF; k++) {
-        const size_t ok = __shfl_sync(FULL, o, (sb + k) & 31);
+        // fewer than eight left: the first one's row again (loads under a condition are issued one by one, 288 us instead of 280)
+        from[k] = todo ? __ffs(todo) - 1 : j0;
+        const size_t ok = __shfl_sync(FULL, o, from[k]);
 #pragma unroll
-        for (int e4 = 0; e4 < E / 4; e4++)
-          f[k][e4] = sb + k < cn ? *reinterpret_cast<const float4*>(p.part_acc + ok * D + lane * E + 4 * e4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int e4 = 0; e4 < E / 4; e4++) f[k][e4] = *reinterpret_cast<const float4*>(p.part_acc + ok * D + lane * E + 4 * e4);
+        todo &= todo - 1u;
       }
     };
-    load_rows(0);
-    if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
-    else ms = -INFINITY;
+    if (todo) request();
     m = ms;
     best = idx;
 #pragma unroll
@@ -94,17 +104,18 @@ __global__ void __launch_bounds__(CMB_WARPS * 32) combine_kernel(const CombinePa
     l = ls * w;
 #pragma unroll
     for (int d2 = 16; d2 > 0; d2 >>= 1) l += __shfl_xor_sync(FULL, l, d2);
-    for (int sb = 0; sb < cn; sb += NF) {
-      if (sb > 0) load_rows(sb);
+    while (n_rows) {
 #pragma unroll
       for (int k = 0; k < NF; k++) {
-        const float ws = __shfl_sync(FULL, w, (sb + k) & 31);
-        if (sb + k >= cn || ws == 0.f) continue;  // (the row of a slot that is not in use holds anything)
+        const float wk = __shfl_sync(FULL, w, from[k]);
+        if (k >= n_rows || wk == 0.f) continue;
 #pragma unroll
         for (int e4 = 0; e4 < E / 4; e4++) {
-          v[4 * e4] += ws * f[k][e4].x; v[4 * e4 + 1] += ws * f[k][e4].y; v[4 * e4 + 2] += ws * f[k][e4].z; v[4 * e4 + 3] += ws * f[k][e4].w;
+          v[4 * e4] += wk * f[k][e4].x; v[4 * e4 + 1] += wk * f[k][e4].y; v[4 * e4 + 2] += wk * f[k][e4].z; v[4 * e4 + 3] += wk * f[k][e4].w;
         }
       }
+      n_rows = 0;
+      if (todo) request();
     }
   } else {
     for (int s = c0; s < c0 + cn; s++) {
@@ -208,14 +219,16 @@ template <int D>
 static cudaError_t launch_combine(const CombineParams& p, cudaStream_t stream) {
   const long long n = (long long)p.batch * p.n_q_heads, slots = (long long)p.splits * p.shards;
   auto go = [&](void (*kernel)(CombineParams), int wph) {
-    return launch_after_predecessor(kernel, dim3((unsigned)((n * wph + CMB_WARPS - 1) / CMB_WARPS)), dim3(CMB_WARPS * 32), 0, stream, p);
+    const int warps = wph == 1 ? CMB_WARPS<1> : CMB_WARPS<8>;
+    return launch_after_predecessor(kernel, dim3((unsigned)((n * wph + warps - 1) / warps)), dim3(warps * 32), 0, stream, p);
   };
-  // Warps per head: eight slots to a warp, whose rows it has in flight at once. Against one warp for up to 16 slots and eight for
-  // more, and rows requested once the weights are known: 16 layers of one 32 K sequence (116 slots) 296 -> 283 us, a step over
-  // 8 x 4 K rows (20 slots) 26.1 -> 25.1, over 32 x 32 K (8 slots) 161 -> 159.
+  // Warps per head. Two to eight need a pass through shared memory: that pays for more than 16 slots (d = 256: more than 8, for few
+  // heads), and eight instead of four only for few heads, whose rows are then loaded in one go. Merges alone, d = 128, all slots in
+  // use, in us: 32 heads with 16 slots 2.8 (two warps: 3.1), 2048 heads with 16 slots 5.8 (10.1), with 20 slots 12.3 (eight
+  // warps: 18.8). 2048 heads with 256 slots, a tenth in use: 19.2; with the rows of unused slots read too it was 48.8.
   if (slots <= 8) return go(combine_kernel<D, 1>, 1);
-  if (slots <= 16) return go(combine_kernel<D, 2>, 2);
-  if (slots <= 32) return go(combine_kernel<D, 4>, 4);
+  if (slots <= 16) return D == 256 && n <= 512 ? go(combine_kernel<D, 2>, 2) : go(combine_kernel<D, 1>, 1);
+  if (slots <= 32 && n > 128) return go(combine_kernel<D, 4>, 4);
   return go(combine_kernel<D, 8>, 8);
 }
 

@@ -222,3 +222,13 @@ def test_other_bit_widths_take_the_three_launch_route(iq, torch, bits):
     w2 = workloads.Workload("bits", B, H_q, H_kv, d, w.t_cap, w.k, w.v, w.q, w.quats, now)
     res = dict(out=out.cpu().numpy().astype(np.float64), lse=lse.cpu().numpy().astype(np.float64), argmax=am.cpu().numpy())
     check_decode(w2, lv, w.q, res, g, now)
+
+
+@pytest.mark.parametrize("d", [128, 256])
+@pytest.mark.parametrize("B,S", [(4, 20), (17, 17), (17, 20), (17, 32)])
+def test_new_row_among_17_to_32_slots(iq, torch, codebooks, d, B, S):
+    """The merge of 32 and of 136 heads (eight and four warps to a head) takes the new row as one more slot."""
+    lens = np.random.default_rng(B + S).integers(0, 900, B).astype(np.int32)
+    lens[0] = 0
+    w = workloads.tiny(900 + S, B, 8, 1, d, int(lens.max()) + 2)
+    _step(iq, torch, codebooks, w, lens, S)
