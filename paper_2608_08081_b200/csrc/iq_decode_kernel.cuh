@@ -97,7 +97,7 @@ struct DecLayout {
   static constexpr int PRE_BYTES = DEC_NPRE * BQ_BYTES;  // the prepared query operands, shared by the groups
   static constexpr int SMEM_BYTES = DEC_HDR_BYTES + PRE_BYTES + NG * GROUP_SMEM;
   // header offsets
-  static constexpr int BAR_STRIDE = 96;  // per group: full[3], s_bar, o_bar, k_ready, p_ready
+  static constexpr int BAR_STRIDE = 96;  // per group: full[3], s_bar, o_bar, k_ready, p_ready, drain
   static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
   // OFF_PRE: count, [DEC_NPRE] (sequence, item), [DEC_NPRE] score factors, [DEC_NPRE][8] per-head maxima
   static constexpr int DESC_STRIDE = STAGES * 32;  // per group
@@ -439,6 +439,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   uint64_t* o_bar = gbar + 4;       // values ready
   uint64_t* k_ready = gbar + 5;     // K tile in TMEM (128 arrivals)
   uint64_t* p_ready = gbar + 6;     // V tile in TMEM + probabilities in smem, staged tile consumed (128 arrivals)
+  uint64_t* drain_bar = gbar + 7;   // a launch that gave up: the MMAs in flight have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::OFF_TMEM);
   int* next_s = reinterpret_cast<int*>(smem + L::OFF_NEXT);            // next block of the CTA's range
   DecStart* start_s = reinterpret_cast<DecStart*>(smem + L::OFF_START);
@@ -653,6 +654,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     mbar_init(o_bar, 1);
     mbar_init(k_ready, DEC_GROUP_THREADS);
     mbar_init(p_ready, DEC_GROUP_THREADS);
+    mbar_init(drain_bar, 1);
     fence_mbar_init();
     fence_proxy_async();
   }
@@ -798,8 +800,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     }
     if (failed) {
       // Give-up path. Tiles staged and not consumed may still be landing: wait (bounded) for each of them, so that no
-      // bulk copy targets this CTA's shared memory after it has left. Tensor-core work in flight is covered by the
-      // fence before the TMEM release at the end of the kernel.
+      // bulk copy targets this CTA's shared memory after it has left. (MMAs in flight: at the end of the kernel.)
       for (int s = it; s < it_issue; s++) mbar_wait_bounded(&full_bar[s % NST], (uint32_t)(s / NST) & 1u, DEC_WAIT_LIMIT);
     }
   }
@@ -1418,7 +1419,14 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   }
 
   allow_dependent_launch();
-  if (__syncthreads_or(failed) && tid == 0 && p.status) atomicOr(&p.status[0], IQ_STATUS_WAIT_TIMEOUT);
+  if (__syncthreads_or(failed)) {
+    if (tid == 0 && p.status) atomicOr(&p.status[0], IQ_STATUS_WAIT_TIMEOUT);
+    if (control) {  // MMAs may still be running, whichever warp gave up: they are waited for, again with a limit, before the tensor memory goes
+      if (elect_one()) tc_commit(drain_bar);
+      __syncwarp();
+      mbar_wait_bounded(drain_bar, 0u, DEC_WAIT_LIMIT);
+    }
+  }
   tc_fence_before();
   __syncthreads();
   if (warp == NG * 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512));
