@@ -255,6 +255,10 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }
+// The same for a converged warp, with one verdict for its lanes: if any of them gave up, the warp did.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t limit) {
+  return __all_sync(0xFFFFFFFFu, mbar_wait_bounded(bar, parity, limit));
+}
 // 1-D bulk asynchronous copy global -> shared, completion counted in bytes on an mbarrier. Both addresses
 // 16-byte aligned, size a multiple of 16 bytes.
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src, uint32_t bytes, uint64_t* bar) {

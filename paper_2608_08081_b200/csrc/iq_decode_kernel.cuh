@@ -98,12 +98,13 @@ struct DecLayout {
   static constexpr int SMEM_BYTES = DEC_HDR_BYTES + PRE_BYTES + NG * GROUP_SMEM;
   // header offsets
   static constexpr int BAR_STRIDE = 96;  // per group: full[3], s_bar, o_bar, k_ready, p_ready, drain
-  static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
+  static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_GAVE_UP = 416, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
   // OFF_PRE: count, [DEC_NPRE] (sequence, item), [DEC_NPRE] score factors, [DEC_NPRE][8] per-head maxima
   static constexpr int DESC_STRIDE = STAGES * 32;  // per group
   static constexpr int RED_STRIDE = 384;            // per group: 3 x [4 warps][8 heads] words
 };
 static_assert(DEC_BLOCK_TOKENS == 128, "the TMEM operand layout assumes 128-row blocks");
+static_assert(DecLayout<128>::OFF_GAVE_UP + 4 * 4 <= DecLayout<128>::OFF_START, "header overflow");
 static_assert(DecLayout<128>::OFF_DESC + 4 * DecLayout<128>::DESC_STRIDE <= DecLayout<128>::OFF_QFAC, "header overflow");
 static_assert(DecLayout<128>::OFF_RED + 4 * DecLayout<128>::RED_STRIDE <= DecLayout<128>::OFF_PRE, "header overflow");
 static_assert(DecLayout<128>::OFF_PRE + 8 + 8 * DEC_NPRE + 4 * DEC_NPRE + 32 * DEC_NPRE <= DEC_HDR_BYTES, "header overflow");
@@ -655,6 +656,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     mbar_init(k_ready, DEC_GROUP_THREADS);
     mbar_init(p_ready, DEC_GROUP_THREADS);
     mbar_init(drain_bar, 1);
+    *reinterpret_cast<volatile int*>(smem + L::OFF_GAVE_UP + 4 * grp) = 0;
     fence_mbar_init();
     fence_proxy_async();
   }
@@ -677,7 +679,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   const uint32_t tmem_base = __shfl_sync(FULL, tmem_slot[0], 0);
   const uint32_t tmem_g = tmem_base + (uint32_t)(grp * L::GROUP_COLS);        // this group's columns
   const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;                // this warp's 32 TMEM lanes
-  bool failed = false;  // a bounded wait gave up: the thread leaves its loop
+  bool failed = false;  // a bounded wait gave up: the control warp, or all four warps of the group, leave their loop
 
   if (control) {
     // ================================================================ control warp of group grp: walks the work, fetches blocks, issues MMAs.
@@ -750,7 +752,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       // scores of the block in slot `it`: S = A_K * B_Q^T once all 128 rows are in TMEM (and B_Q of its segment is complete)
       const int bqbuf = __shfl_sync(FULL, desc[it % NST].bqbuf, 0);  // the query operand of the block's segment (the start address field counts 16-byte units)
       const uint64_t bq_desc0 = bqbuf < 0 ? bq_desc_own : bq_desc_pre + (uint64_t)(bqbuf * (L::BQ_BYTES / 16));
-      failed = !mbar_wait_bounded(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
+      failed = !mbar_wait_warp(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
       if (failed) break;
       tc_fence_after();
       if (elect_one()) {
@@ -771,7 +773,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       if (!ended && it_issue - it < NST) stage_next();
       if (!ended && dr.kind < 0) draw();
       // values: O = A_V * B_P^T once the V tile is in TMEM and the probabilities are in shared memory
-      failed = !mbar_wait_bounded(p_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
+      failed = !mbar_wait_warp(p_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
       if (failed) break;
       tc_fence_after();
       const bool keep_values = I8 && *reinterpret_cast<volatile int*>(smem + L::OFF_ACCF + 4 * grp) != 0;
@@ -947,7 +949,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           red[(warp & 3) * 8 + hr] = lsum;
           if ((warp & 3) == 0) red2[hr] = -msel;
         }
-        group_bar_sync(bar_id);
+        if (group_bar_or(bar_id, false)) { failed = true; return; }  // (see give_up)
         if (gt < nh) {
           const size_t o = ((size_t)seg_b * p.n_q_heads + h0 + gt) * S + seg_slot;
           p.part_ml[2 * o] = red2[gt] * LN2;
@@ -973,7 +975,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           if ((lane & 3) == 0) { red2[(warp & 3) * 8 + hr] = bv; redi[(warp & 3) * 8 + hr] = bi; }
         }
       }
-      group_bar_sync(bar_id);
+      if (group_bar_or(bar_id, false)) { failed = true; return; }
       float scale[8];  // the partial is reported relative to the exact maximum where that is tracked
 #pragma unroll
       for (int h = 0; h < HN; h++) {
@@ -1031,15 +1033,28 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     int st = 0;          // stage of slot `it` and its phase, kept incrementally
     uint32_t st_ph = 0;
     int2 dsc = make_int2(-1, 0);  // (valid rows | end marker, flags) of slot `it`; the rest of its descriptor is read where it is needed
-    auto next_slot = [&]() {      // wait for slot `it` and read its descriptor; a wait that gave up ends the work like an end marker
-      if (!mbar_wait_bounded(&full_bar[st], st_ph, DEC_WAIT_LIMIT)) { failed = true; dsc.x = -1; return; }
+    auto next_slot = [&]() {      // wait for slot `it` and read its descriptor
+      if (!mbar_wait_warp(&full_bar[st], st_ph, DEC_WAIT_LIMIT)) return false;
       dsc = *reinterpret_cast<const int2*>(&desc[st]);
+      return true;
+    };
+    // A wait of this warp gave up. Others of the group may get theirs, so the group leaves as one: whichever way a warp goes
+    // from here, the next barrier that it comes to is a vote (that of a block or that of a segment's end; nothing is waited for
+    // between a vote that passed and the barriers behind it). This warp votes there with the rest, and the note tells a block's
+    // vote from one about its scores. What the warp no longer signals runs out for the others, who then come here too.
+    volatile int* const gave_up = reinterpret_cast<volatile int*>(smem + L::OFF_GAVE_UP + 4 * grp);
+    auto give_up = [&]() {
+      if (lane == 0) *gave_up = 1;
+      __syncwarp();
+      group_bar_or(bar_id, true);
+      failed = true;
     };
     auto advance_slot = [&]() {
       it++;
       if (++st == NST) { st = 0; st_ph ^= 1u; }
     };
-    next_slot();
+    failed = group_bar_or(bar_id, !next_slot());  // (an end marker in the first slot: no vote would follow)
+    if (failed) dsc.x = -1;
 
     if constexpr (I8) {
       // Integer path. The group's TMEM columns: K tile (d/4), V tile (32 per 128 coordinates), scores (32 = 8 heads x 4
@@ -1136,7 +1151,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         float vf = vsc * vfac;
 
         // ---- scores: three int32 digit columns per head -> log2-domain score of row gt, z = x kfs
-        if (!mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
+        if (!mbar_wait_warp(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
         tc_fence_after();
         F32x2 x2[HN / 2], over[HN / 2];  // x: the score's digits put together; z - m_run
         {
@@ -1182,6 +1197,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 || vf > vref || nacc >= 384;
 
         if (group_bar_or(bar_id, exceed)) {
+          if (*gave_up) { failed = true; break; }
           if (nacc > 0) flush();  // what TMEM holds is relative to the old references (the previous value MMAs have completed)
           {
             float s8[8];
@@ -1224,17 +1240,18 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
 
         // ---- next slot: if it continues the segment, its K tile now, while the value MMAs run
         advance_slot();
-        next_slot();
+        if (!next_slot()) { give_up(); break; }
         more = dsc.x >= 0 && !(dsc.y & 1);
         if (more) k_tile(stages + st * L::STAGE_BYTES);
 
         // ---- the value MMAs of this block must have completed before its V tile and B_P are overwritten; their result stays in TMEM
-        if (!mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
+        if (!mbar_wait_warp(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
         nbk++;
       }
         if (failed) break;
         if (nacc > 0) flush();
         close_segment();
+        if (failed) break;
       }
     } else {
       // fp16 path. The group's 128 TMEM columns: [0, 64 DJ) operand tile, then scores, values, and V_COL.. a second home for
@@ -1304,7 +1321,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         for (int j = 0; j < DJ; j++) { v_unit(j, 0); v_unit(j, 1); }
 
         // the score MMAs read the K tile that the rest of the V tile is about to overwrite
-        if (!mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
+        if (!mbar_wait_warp(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
         tc_fence_after();
         uint32_t raw_u[16];
         tc_ld16_issue(tmem_g + lane_sel + L::S_COL, raw_u);  // scores of row gt: in flight during the next unit
@@ -1339,6 +1356,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         // units): exp2(z - m) then stays below 2^DEC_MAX_SLACK and nothing has to be exchanged between the warps in the
         // common case (one barrier with an OR reduction).
         if (group_bar_or(bar_id, max_of(over) > DEC_MAX_SLACK)) {
+          if (*gave_up) { failed = true; break; }
           {
             float s8[8];
 #pragma unroll
@@ -1382,7 +1400,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         // ---- next slot: if it continues the segment, its K coordinates that live in the upper half of the operand
         // columns, while the value MMAs run
         advance_slot();
-        next_slot();
+        if (!next_slot()) { give_up(); break; }
         more = dsc.x >= 0 && !(dsc.y & 1);
         if (more) {
           k_load(stages + st * L::STAGE_BYTES);
@@ -1392,7 +1410,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
 
         // ---- fold the value product into the running accumulator (the value MMAs also release the lower half)
-        if (!mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { failed = true; break; }
+        if (!mbar_wait_warp(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < DJ; j++) {
@@ -1414,6 +1432,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       }
         if (failed) break;
         close_segment();
+        if (failed) break;
       }
     }
   }

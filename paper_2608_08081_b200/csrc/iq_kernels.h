@@ -8,8 +8,8 @@ namespace iq {
 
 // Polls one mbarrier wait of a kernel may take before it gives up (IQ_STATUS_WAIT_TIMEOUT; the reconstruction: rows of NaN):
 // with the 20 us suspend hint of a poll that is at most 65536 * 20 us = 1.3 s (and a few milliseconds at least). Waits that
-// work last microseconds. A thread that has given up skips every later wait, so a CTA returns within about that time
-// after its first failed wait.
+// work last microseconds. A warp that has given up waits no more, and what it no longer signals runs out once for the warps that
+// need it, so a CTA returns within about twice that time after its first failed wait.
 constexpr uint32_t DEC_WAIT_LIMIT = 1u << 16;
 
 // Addressing of the cache arrays: contiguous per sequence (table == nullptr) or a pool of pages with a block table
