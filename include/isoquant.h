@@ -236,8 +236,8 @@ int iq_selftest_append_wait(const iq_shape* shape, const float* rot_dev, const i
  *                  in the rotated space, natural coordinate order. 16-byte aligned.
  *   part_ml        device fp32 [batch][n_q_heads][S][2] = (m, l): the slot's reference m and l = sum_j exp(z_j - m),
  *                  z_j = sm_scale * q~ . k~_j. With part_argmax, m = max_j z_j exactly; without it m is the kernel's
- *                  running reference, max_j z_j - 4 ln 2 <= m <= max_j z_j (acc and l are relative to the same m
- *                  either way). An unused slot holds (-inf, 0), and its acc is not written (the merge skips a slot
+ *                  running reference, max_j z_j - 4 ln 2 <= m <= max_j z_j + 3 ln 2 up to the rounding of z_j (acc and l
+ *                  are relative to the same m either way). An unused slot holds (-inf, 0), and its acc is not written (the merge skips a slot
  *                  with l = 0 without reading acc); (m, l) of every slot of every head is written on every call.
  *   part_argmax    device int32 [batch][n_q_heads][S] or NULL: row index attaining m (lowest on ties), -1 if empty.
  *   status_dev     optional (see top).
@@ -246,8 +246,9 @@ int iq_selftest_append_wait(const iq_shape* shape, const float* rot_dev, const i
  * KV head group), the probabilities times V scale as four base-256 digits of a 30-bit fixed-point number; softmax
  * statistics and the running output in fp32. Other codebooks: levels must be exact binary16 values; q~ and the
  * probabilities enter fp16 operands as two-term sums (hi + lo), every accumulation is fp32. Blocks are handed to the
- * warps of an SM dynamically, so the order of the fp32 additions -- and with it the last bits of the
- * result -- can differ between two calls on the same inputs; m and the argmax do not.
+ * warps of an SM dynamically, so in the balanced mode the rows of a slot, its m and its row of the maximum, and the order of the
+ * fp32 additions -- and with it the last bits of the merged result -- can differ between two calls on the same inputs; the merged
+ * argmax does not. With S < 2 G the slots' rows and partials are the same in every call.
  */
 int iq_decode_attention(const iq_shape* shape, const float* rot_dev, const iq_codebook* codebook,
                         const void* q, const iq_cache* cache, const int32_t* seq_lens_dev,
