@@ -30,11 +30,6 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&o)[16]) {
 #pragma unroll
   for (int i = 0; i < 16; i++) o[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]),
-               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
 // The same load without the wait: the registers are valid after tc_wait_ld().
 __device__ __forceinline__ void tc_ld16_issue(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -226,9 +221,6 @@ __device__ __forceinline__ F32x2 mul2(F32x2 a, F32x2 b) {
   return r;
 }
 
-// int32 -> float for |x| < 2^22, on the integer and FMA pipes (the conversion instruction runs at a quarter of their rate).
-__device__ __forceinline__ float i2f_small(uint32_t x) { return __uint_as_float(x + 0x4B400000u) - 12582912.0f; }
-
 // One lane of a converged warp. Issuing the MMAs / bulk copies from an elected lane of a converged warp keeps
 // their operands in uniform registers; a lone divergent thread issues the same sequence about 3x slower.
 __device__ __forceinline__ bool elect_one() {
@@ -246,8 +238,6 @@ __device__ __forceinline__ bool group_bar_or(int id, bool pred) {
                : "=r"(r) : "r"(id), "r"((uint32_t)pred) : "memory");
   return r != 0;
 }
-// Barrier 0 over the whole CTA, for the places where the control and the compute warps arrive from different code.
-__device__ __forceinline__ void cta_bar_sync() { asm volatile("barrier.sync 0;" ::: "memory"); }
 // The same over `count` threads.
 __device__ __forceinline__ bool cta_bar_or_n(int id, int count, bool pred) {
   uint32_t r;

@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     int it_issue = 0;   // slots staged so far
     int nbk = 0;        // blocks processed (phases of k_ready, s_bar, p_ready, o_bar)
     bool ended = false; // the work ran out and the end marker has been staged
-    // The walk over the CTA's work lives in a struct and advances in an out-of-line function (dec_draw).
+    // The walk over the CTA's work lives in a struct and advances in dec_draw.
     DecWalk wk;
     wk.range_mode = range_mode ? 1 : 0;
     wk.grp = grp;
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     wk.unit = min(wk.n_units, grp * n_cta + cta);
     wk.ub = wk.uy = wk.uk = wk.ublk = wk.uhi = wk.unew = wk.ulen = 0;
     // The next block is drawn (shared counter; with a paged cache also its block-table entry, a load from global
-    // memory) while the compute warps are busy with the softmax of the current one, and staged after the value MMAs.
+    // memory) while the compute warps are busy with the softmax of the current one, and staged after the score MMAs of the one after.
     DecDrawn dr;
     dr.kind = -1;
     auto draw = [&]() {
