@@ -69,8 +69,6 @@ __global__ void __launch_bounds__(CMB_WARPS<WPH> * 32, D == 128 && WPH > 1 ? 3 :
       o = slot_index(c0 + lane);
       ms = p.part_ml[2 * o];
       ls = p.part_ml[2 * o + 1];
-      if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
-      else ms = -INFINITY;
     }
     constexpr int NF = 8;  // rows in flight
     float4 f[NF][E / 4];
@@ -90,7 +88,9 @@ __global__ void __launch_bounds__(CMB_WARPS<WPH> * 32, D == 128 && WPH > 1 ? 3 :
         todo &= todo - 1u;
       }
     };
-    if (todo) request();
+    if (todo) request();  // before anything else that waits: 16 layers of one 32 K sequence 280 us instead of 283 with the argmax first
+    if (ls > 0.f) idx = slot_argmax(c0 + lane, o);
+    else ms = -INFINITY;
     m = ms;
     best = idx;
 #pragma unroll
