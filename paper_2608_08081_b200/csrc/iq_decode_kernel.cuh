@@ -98,13 +98,12 @@ struct DecLayout {
   static constexpr int SMEM_BYTES = DEC_HDR_BYTES + PRE_BYTES + NG * GROUP_SMEM;
   // header offsets
   static constexpr int BAR_STRIDE = 96;  // per group: full[3], s_bar, o_bar, k_ready, p_ready, drain
-  static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_GAVE_UP = 416, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
+  static constexpr int OFF_TMEM = 384, OFF_NEXT = 388, OFF_ACCF = 400, OFF_START = 448, OFF_DESC = 512, OFF_QFAC = 896, OFF_SEGID = 960, OFF_RED = 1024, OFF_PRE = 2560;
   // OFF_PRE: count, [DEC_NPRE] (sequence, item), [DEC_NPRE] score factors, [DEC_NPRE][8] per-head maxima
   static constexpr int DESC_STRIDE = STAGES * 32;  // per group
   static constexpr int RED_STRIDE = 384;            // per group: 3 x [4 warps][8 heads] words
 };
 static_assert(DEC_BLOCK_TOKENS == 128, "the TMEM operand layout assumes 128-row blocks");
-static_assert(DecLayout<128>::OFF_GAVE_UP + 4 * 4 <= DecLayout<128>::OFF_START, "header overflow");
 static_assert(DecLayout<128>::OFF_DESC + 4 * DecLayout<128>::DESC_STRIDE <= DecLayout<128>::OFF_QFAC, "header overflow");
 static_assert(DecLayout<128>::OFF_RED + 4 * DecLayout<128>::RED_STRIDE <= DecLayout<128>::OFF_PRE, "header overflow");
 static_assert(DecLayout<128>::OFF_PRE + 8 + 8 * DEC_NPRE + 4 * DEC_NPRE + 32 * DEC_NPRE <= DEC_HDR_BYTES, "header overflow");
@@ -655,8 +654,6 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
     mbar_init(o_bar, 1);
     mbar_init(k_ready, DEC_GROUP_THREADS);
     mbar_init(p_ready, DEC_GROUP_THREADS);
-    mbar_init(drain_bar, 1);
-    *reinterpret_cast<volatile int*>(smem + L::OFF_GAVE_UP + 4 * grp) = 0;
     fence_mbar_init();
     fence_proxy_async();
   }
@@ -679,7 +676,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   const uint32_t tmem_base = __shfl_sync(FULL, tmem_slot[0], 0);
   const uint32_t tmem_g = tmem_base + (uint32_t)(grp * L::GROUP_COLS);        // this group's columns
   const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;                // this warp's 32 TMEM lanes
-  bool failed = false;  // a bounded wait gave up: the control warp, or all four warps of the group, leave their loop
+  bool failed = false;  // a bounded wait gave up: the control warp, or all four warps of the group, leave their loop at their next vote
 
   if (control) {
     // ================================================================ control warp of group grp: walks the work, fetches blocks, issues MMAs.
@@ -752,8 +749,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       // scores of the block in slot `it`: S = A_K * B_Q^T once all 128 rows are in TMEM (and B_Q of its segment is complete)
       const int bqbuf = __shfl_sync(FULL, desc[it % NST].bqbuf, 0);  // the query operand of the block's segment (the start address field counts 16-byte units)
       const uint64_t bq_desc0 = bqbuf < 0 ? bq_desc_own : bq_desc_pre + (uint64_t)(bqbuf * (L::BQ_BYTES / 16));
-      failed = !mbar_wait_warp(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
-      if (failed) break;
+      // (a wait that gave up: MMAs over whatever is there are issued all the same, and the lanes vote behind them, where nobody waits)
+      failed = !mbar_wait_bounded(k_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
       tc_fence_after();
       if (elect_one()) {
         if constexpr (I8) {
@@ -767,14 +764,14 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
         tc_commit(s_bar);
       }
-      __syncwarp();
+      failed = __any_sync(FULL, failed);
+      if (failed) break;
       // The slot of the block before, which the compute threads released when they signalled its p_ready, is staged here, where
       // they have the softmax to do: a hundred instructions between value and score MMAs would hold the next scores up.
       if (!ended && it_issue - it < NST) stage_next();
       if (!ended && dr.kind < 0) draw();
       // values: O = A_V * B_P^T once the V tile is in TMEM and the probabilities are in shared memory
-      failed = !mbar_wait_warp(p_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
-      if (failed) break;
+      failed = !mbar_wait_bounded(p_ready, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
       tc_fence_after();
       const bool keep_values = I8 && *reinterpret_cast<volatile int*>(smem + L::OFF_ACCF + 4 * grp) != 0;
       if (elect_one()) {
@@ -796,7 +793,8 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
         tc_commit(o_bar);
       }
-      __syncwarp();
+      failed = __any_sync(FULL, failed);
+      if (failed) break;
       it++;
       nbk++;
     }
@@ -949,7 +947,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           red[(warp & 3) * 8 + hr] = lsum;
           if ((warp & 3) == 0) red2[hr] = -msel;
         }
-        if (group_bar_or(bar_id, false)) { failed = true; return; }  // (see give_up)
+        if (group_bar_or(bar_id, failed)) { failed = true; group_bar_or(bar_id, true); return; }  // (see give_up)
         if (gt < nh) {
           const size_t o = ((size_t)seg_b * p.n_q_heads + h0 + gt) * S + seg_slot;
           p.part_ml[2 * o] = red2[gt] * LN2;
@@ -975,7 +973,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           if ((lane & 3) == 0) { red2[(warp & 3) * 8 + hr] = bv; redi[(warp & 3) * 8 + hr] = bi; }
         }
       }
-      if (group_bar_or(bar_id, false)) { failed = true; return; }
+      if (group_bar_or(bar_id, failed)) { failed = true; group_bar_or(bar_id, true); return; }
       float scale[8];  // the partial is reported relative to the exact maximum where that is tracked
 #pragma unroll
       for (int h = 0; h < HN; h++) {
@@ -1038,16 +1036,16 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
       dsc = *reinterpret_cast<const int2*>(&desc[st]);
       return true;
     };
-    // A wait of this warp gave up. Others of the group may get theirs, so the group leaves as one: whichever way a warp goes
-    // from here, the next barrier that it comes to is a vote (that of a block or that of a segment's end; nothing is waited for
-    // between a vote that passed and the barriers behind it). This warp votes there with the rest, and the note tells a block's
-    // vote from one about its scores. What the warp no longer signals runs out for the others, who then come here too.
-    volatile int* const gave_up = reinterpret_cast<volatile int*>(smem + L::OFF_GAVE_UP + 4 * grp);
+    // A wait may give up in some threads and not in others of the group: it leaves as one. The next barrier behind a wait is a vote on
+    // every way from there, that of a block or that of a segment's end, and a vote that passed is followed by a second one, on
+    // leaving, before anything is waited for. A thread that has no scores or values goes on to it over whatever is there. A tile's
+    // wait decides where the warp goes, so it has one verdict per warp, and the warp votes twice at once; what it no longer
+    // signals runs out for the others, who then come to these votes too. (With a verdict per
+    // warp at every wait and a note in shared memory for one vote: 32 x 32 K rows 166 us instead of 164.)
     auto give_up = [&]() {
-      if (lane == 0) *gave_up = 1;
-      __syncwarp();
-      group_bar_or(bar_id, true);
       failed = true;
+      group_bar_or(bar_id, true);
+      group_bar_or(bar_id, true);
     };
     auto advance_slot = [&]() {
       it++;
@@ -1151,7 +1149,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         float vf = vsc * vfac;
 
         // ---- scores: three int32 digit columns per head -> log2-domain score of row gt, z = x kfs
-        if (!mbar_wait_warp(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
+        failed |= !mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
         tc_fence_after();
         F32x2 x2[HN / 2], over[HN / 2];  // x: the score's digits put together; z - m_run
         {
@@ -1194,10 +1192,9 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         // The running reference m_run is raised when a score exceeds it by more than DEC_MAX_SLACK_I8 log2 units, the
         // V-scale bound vref when a row exceeds it: both are rare after the first blocks (one barrier with an OR reduction
         // otherwise).
-        const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 || vf > vref || nacc >= 384;
+        const bool exceed = max_of(over) > DEC_MAX_SLACK_I8 || vf > vref || nacc >= 384 || failed;
 
         if (group_bar_or(bar_id, exceed)) {
-          if (*gave_up) { failed = true; break; }
           if (nacc > 0) flush();  // what TMEM holds is relative to the old references (the previous value MMAs have completed)
           {
             float s8[8];
@@ -1208,7 +1205,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           }
           const float wv_max = warp_max(vf);
           if (lane == 0) red2[warp & 3] = wv_max;
-          group_bar_sync(bar_id);
+          if (group_bar_or(bar_id, failed)) { failed = true; break; }
           raise(x2, kfs, stale, over);
           const float bv = fmaxf(fmaxf(red2[0], red2[1]), fmaxf(red2[2], red2[3]));
           if (bv > vref) vref = __uint_as_float((__float_as_uint(bv) + 0x007FFFFFu) & 0x7F800000u);  // next power of two
@@ -1245,10 +1242,10 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         if (more) k_tile(stages + st * L::STAGE_BYTES);
 
         // ---- the value MMAs of this block must have completed before its V tile and B_P are overwritten; their result stays in TMEM
-        if (!mbar_wait_warp(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
+        failed |= !mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
         nbk++;
       }
-        if (failed) break;
+        if (more) break;  // left in the middle, by all four warps; a thread that has no values goes on to the segment's vote
         if (nacc > 0) flush();
         close_segment();
         if (failed) break;
@@ -1321,7 +1318,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         for (int j = 0; j < DJ; j++) { v_unit(j, 0); v_unit(j, 1); }
 
         // the score MMAs read the K tile that the rest of the V tile is about to overwrite
-        if (!mbar_wait_warp(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
+        failed |= !mbar_wait_bounded(s_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
         tc_fence_after();
         uint32_t raw_u[16];
         tc_ld16_issue(tmem_g + lane_sel + L::S_COL, raw_u);  // scores of row gt: in flight during the next unit
@@ -1355,8 +1352,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         // The running reference is raised only when some score of the block exceeds it by more than DEC_MAX_SLACK (log2
         // units): exp2(z - m) then stays below 2^DEC_MAX_SLACK and nothing has to be exchanged between the warps in the
         // common case (one barrier with an OR reduction).
-        if (group_bar_or(bar_id, max_of(over) > DEC_MAX_SLACK)) {
-          if (*gave_up) { failed = true; break; }
+        if (group_bar_or(bar_id, max_of(over) > DEC_MAX_SLACK || failed)) {
           {
             float s8[8];
 #pragma unroll
@@ -1364,7 +1360,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
             const float wm = warp_reduce8(s8, lane, [](float x, float y) { return fmaxf(x, y); });
             if ((lane & 3) == 0) red[(warp & 3) * 8 + warp_reduce8_head(lane)] = wm;
           }
-          group_bar_sync(bar_id);
+          if (group_bar_or(bar_id, failed)) { failed = true; break; }
           raise(x2, kf, stale, over);
         }
 #pragma unroll
@@ -1410,7 +1406,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
         }
 
         // ---- fold the value product into the running accumulator (the value MMAs also release the lower half)
-        if (!mbar_wait_warp(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT)) { give_up(); break; }
+        failed |= !mbar_wait_bounded(o_bar, (uint32_t)nbk & 1u, DEC_WAIT_LIMIT);
         tc_fence_after();
 #pragma unroll
         for (int j = 0; j < DJ; j++) {
@@ -1430,7 +1426,7 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
           mbar_arrive(k_ready);
         }
       }
-        if (failed) break;
+        if (more) break;
         close_segment();
         if (failed) break;
       }
@@ -1441,7 +1437,11 @@ __global__ void __launch_bounds__(DecLayout<D, BITS>::THREADS, 1) decode_kernel(
   if (__syncthreads_or(failed)) {
     if (tid == 0 && p.status) atomicOr(&p.status[0], IQ_STATUS_WAIT_TIMEOUT);
     if (control) {  // MMAs may still be running, whichever warp gave up: they are waited for, again with a limit, before the tensor memory goes
-      if (elect_one()) tc_commit(drain_bar);
+      if (elect_one()) {
+        mbar_init(drain_bar, 1);
+        fence_mbar_init();
+        tc_commit(drain_bar);
+      }
       __syncwarp();
       mbar_wait_bounded(drain_bar, 0u, DEC_WAIT_LIMIT);
     }

@@ -34,11 +34,13 @@ TOKEN = re.compile(r"mbar_wait_\w+\(&?(?P<wait>s_bar|o_bar)\b|(?P<slot>next_slot
 def _tokens(text):
     out = []
     for m in TOKEN.finditer(text):
-        statement = text[m.start():m.start() + 120].split("}")[0]
-        if m["wait"] or m["slot"]:
-            out.append(("wait", m["wait"] or "full", "give_up()" in statement))
-        elif m["vote"]:
-            out.append(("vote", "*gave_up" in statement))
+        statement = text[m.start():].split(";")[0]
+        if m["wait"] or m["slot"]:  # a wait that gave up: the warp votes at once, goes on to the next vote, or leaves
+            goes_on = "failed |=" in text[:m.start()].rsplit("\n", 1)[1]
+            out.append(("wait", m["wait"] or "full", "vote" if "give_up()" in statement else "go on" if goes_on else "leave"))
+        elif m["vote"]:  # whether a warp that gave up before votes for leaving
+            named = re.search(r"\bexceed\)", statement) and re.search(r"bool exceed = [^;]*\bfailed;", text)
+            out.append(("vote", bool(re.search(r"\bfailed\)", statement) or named)))
         elif m["sync"]:
             out.append(("sync",))
         else:
@@ -47,21 +49,25 @@ def _tokens(text):
 
 
 def _program(path):
-    """What a compute warp does: at the first slot, when it opens a segment, in a block, when it closes the segment."""
+    """What a compute warp does: at the first slot, when it opens a segment, in a block, when it closes the segment, when it gives up."""
     text = re.sub(r"//[^\n]*", "", open(SOURCE).read())
     text = text[text.index("if (!control) {"):text.index("allow_dependent_launch();\n  if (__syncthreads_or")]
     opening = _tokens(_body(text, r"auto open_segment = [^{]*\{")[0])
     close = _body(text, r"auto close_segment = [^{]*\{")[0]
     plain, end = _body(close, r"if constexpr \(!ARGMAX\) \{")
     closes = [_tokens(plain), _tokens(close[end:])]
+    give_up = _tokens(_body(text, r"auto give_up = [^{]*\{")[0]) if "auto give_up" in text else []
     first = re.search(r"\n[^\n]*next_slot\(\);?[^\n]*\n\s*(if \(failed\)[^\n]*\n\s*)?if constexpr \(I8\) \{", text)
     assert first
     int8, end = _body(text, r"if constexpr \(I8\) \{\s*constexpr int NLR")
-    f16 = _body(text[end:], r"^ else \{")[0]
-    block = _tokens(_body(int8 if path == "int8" else f16, r"while \(more\) \{")[0])
-    assert [t[1] for t in block if t[0] == "wait"] == ["s_bar", "full", "o_bar"] and sum(t[0] == "vote" for t in block) == 1
-    assert opening == [("sync",)] and all(len(c) == 1 for c in closes)
-    return dict(first_vote="group_bar_or" in first[0], opening=opening if path == "int8" else [], block=block, closes=closes)
+    segments = int8 if path == "int8" else _body(text[end:], r"^ else \{")[0]
+    block, end = _body(segments, r"while \(more\) \{")
+    behind = re.match(r"\s*if \((\w+)\) break;", segments[end:])[1]  # who leaves behind the blocks: warps that gave up, or that left a block
+    block = _tokens(block)
+    assert [t[1] for t in block if t[0] == "wait"] == ["s_bar", "full", "o_bar"] and [t[0] for t in block][1] == "vote"
+    assert opening == [("sync",)] and all(1 <= len(c) <= 2 for c in closes) and behind in ("failed", "more")
+    return dict(first_vote="group_bar_or" in first[0], opening=opening if path == "int8" else [], block=block, closes=closes, give_up=len(give_up),
+                behind=behind)
 
 
 class _Left(Exception):
@@ -70,16 +76,22 @@ class _Left(Exception):
 
 def _warp(prog, close, segments, raises, own_operand):
     """One warp as a generator of requests; returns True if it gave up."""
-    def wait(bar, n, meets):
+    gave_up = False
+
+    def wait(bar, n, then):
+        nonlocal gave_up
         if not (yield ("wait", bar, n)):
-            if meets:
-                yield ("vote", True, True)
-            raise _Left
+            gave_up = True
+            if then == "vote":
+                for _ in range(prog["give_up"]):
+                    yield ("vote", True)
+            if then != "go on":
+                raise _Left
 
     try:
         ok = yield ("wait", "full", 0)
         if prog["first_vote"]:
-            if (yield ("vote", not ok, False))[0]:
+            if (yield ("vote", not ok)):
                 return True
         elif not ok:
             return True
@@ -90,14 +102,15 @@ def _warp(prog, close, segments, raises, own_operand):
                     yield ("sync",)
             yield ("arrive", "k_ready", n)
             for i in range(blocks):
-                raised = False
+                raised = None
                 for t in prog["block"]:
                     if t[0] == "wait":
                         yield from wait(t[1], n + (t[1] == "full"), t[2])
-                    elif t[0] == "vote":
-                        raised, noted = yield ("vote", raises[n], False)
-                        if raised and t[1] and noted:
-                            return True
+                    elif t[0] == "vote" and raised is None:
+                        raised = yield ("vote", raises[n] or (t[1] and gave_up))
+                    elif t[0] == "vote":  # behind a vote that passed: on leaving
+                        if raised and (yield ("vote", t[1] and gave_up)):
+                            raise _Left
                     elif t[0] == "sync":
                         if raised:
                             yield ("sync",)
@@ -106,11 +119,14 @@ def _warp(prog, close, segments, raises, own_operand):
                     elif i + 1 < blocks:  # the next block of the segment
                         yield ("arrive", "k_ready", n + 1)
                 n += 1
-            for t in close:
-                if t[0] == "sync":
-                    yield ("sync",)
-                elif (yield ("vote", False, False))[0]:
-                    return True
+            if prog["behind"] == "failed" and gave_up:
+                raise _Left
+            if close[0][0] == "sync":
+                yield ("sync",)
+            elif (yield ("vote", close[0][1] and gave_up)):
+                for _ in close[1:]:
+                    yield ("vote", True)
+                raise _Left
         return False
     except _Left:
         return True
@@ -121,10 +137,13 @@ def _run(prog, close, segments, raises, own_operand, gives_up, rng):
     warps = [_warp(prog, close, segments, raises, own_operand) for _ in range(4)]
     asks = [next(w) for w in warps]
     waits, result = [0] * 4, [None] * 4
-    arrived, at_barrier, noted = {}, [], False
+    arrived, at_barrier = {}, []
+    control_left = []  # the last MMAs that the control warp issued, over whatever was there, when its own wait gave up
 
     def done(bar, n):
         full = lambda kind, i: len(arrived.get((kind, i), ())) == 4  # noqa: E731
+        if control_left:
+            return (bar, n) in control_left or bar == "full" and n < STAGES or n < control_left[0][1]
         if bar == "full":  # a slot is staged again once the scores of the block after its last one have been issued
             return n < STAGES or full("k_ready", n - STAGES + 1)
         return full("k_ready" if bar == "s_bar" else "p_ready", n)
@@ -143,7 +162,10 @@ def _run(prog, close, segments, raises, own_operand, gives_up, rng):
             (stuck if a[0] == "wait" and not done(a[1], a[2]) and (w, waits[w]) not in gives_up else ready).append(w)
         if not ready and not stuck:
             return None  # everybody that is left stands at a barrier
-        w = rng.choice(ready or stuck)  # nothing else moves: a wait runs out
+        if not ready and not control_left and rng.random() < 0.5:  # nothing moves: a wait runs out, the control warp's ...
+            control_left.append(max((asks[v][1:] for v in stuck if asks[v][1] != "full"), key=lambda x: x[1], default=("full", 0)))
+            continue
+        w = rng.choice(ready or stuck)  # ... or one of these warps'
         a = asks[w]
         if a[0] == "wait":
             ok = bool(ready) and (w, waits[w]) not in gives_up
@@ -153,11 +175,10 @@ def _run(prog, close, segments, raises, own_operand, gives_up, rng):
             arrived.setdefault(a[1:], set()).add(w)
             answer(w, None)
         else:
-            noted |= a[0] == "vote" and a[2]
             assert all(asks[v][0] == a[0] for v in at_barrier), "a vote and a plain barrier meet"
             at_barrier.append(w)
             if len(at_barrier) == 4:
-                value = (any(asks[v][1] for v in at_barrier), noted) if a[0] == "vote" else None
+                value = any(asks[v][1] for v in at_barrier) if a[0] == "vote" else None
                 everybody, at_barrier = at_barrier, []
                 for v in everybody:
                     answer(v, value)
